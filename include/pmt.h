@@ -476,14 +476,15 @@ pm_status pm_profile_read(pm_ctx *ctx, double *ms, long long *calls, int reset);
 /* Work counters of the 2D triangulation (Sec. 3.2 particle functions),
  * collected while pm_profile(ctx, 2) is in effect: that mode runs a counting
  * build of the triangulation kernel (same results, slower; not for timing).
- * counts[0..4] = candidates examined, candidates within the distance bound,
- * in-circle vertex tests, clips of the Voronoi cell, sum of the cell sizes
- * after each clip, summed over all particles and calls since the last reset,
- * each particle counted once, in the pass that completes its cell.
- * counts[5] = cells the main pass gave up to the retry passes (capacity 9),
- * counts[6] = cells the first retry pass gave up to the last (capacity 12),
- * counts[7] = in-circle vertex tests the float filter could not decide and
- * left to the exact 128-bit predicate.
+ * counts[0..4] = candidates examined, candidates within the search radius (or
+ * the distance bound of the exact passes), tests of a candidate against a star
+ * edge or cell vertex, vertices inserted into a star (clips), sum of the star
+ * sizes after each, summed over all particles and calls since the last reset,
+ * each particle counted once, in the pass that completes its star.
+ * counts[5] = stars the main pass gave up to the later passes,
+ * counts[6] = stars of the later passes with more than 12 neighbours,
+ * counts[7] = tests that float arithmetic could not decide and left to the
+ * exact 128-bit predicate.
  * Waits for the context's stream. Host array of `ncounts` entries (entries
  * past 7 are written as 0). PM_EINVAL on a NULL ctx or array. */
 pm_status pm_work_read(pm_ctx *ctx, long long *counts, int ncounts, int reset);

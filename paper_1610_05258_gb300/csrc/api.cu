@@ -208,7 +208,7 @@ pm_status pm_ctx_create_mesh(pm_ctx **out, int dim, int n, double L, long long m
     w.nblk_psum = 4 * 152;  // enough loads in flight to stream the particle arrays
     bool ok = alloc(c, &w.fx, np) && alloc(c, &w.key, np) && alloc(c, &w.slot, np) && alloc(c, &w.count, nc) &&
               alloc(c, &w.cell_start, nc + 1) && alloc(c, &w.scan_tmp, nc / 4096 + 2) && alloc(c, &w.tmp, np) &&
-              alloc(c, &w.perm, np) && alloc(c, &w.pos, np) && alloc(c, &w.vals, np * F) &&
+              alloc(c, &w.perm, np) && alloc(c, &w.pos, np + PM_POS_PAD) && alloc(c, &w.vals, np * F) &&
               alloc(c, &w.maxabs, PM_MAXF) && alloc(c, &w.deg, np) && alloc(c, &w.vol, np) &&
               alloc(c, &w.part, (dim == 2 ? 4 : 2) * (F + 1) * nc) && alloc(c, &w.bfix, F * nc) &&
               alloc(c, &w.psum, 2 * PM_MAXF * (ll)w.nblk_psum) &&
@@ -216,7 +216,7 @@ pm_status pm_ctx_create_mesh(pm_ctx **out, int dim, int n, double L, long long m
               alloc(c, &w.p, F * nc) && alloc(c, &w.q, F * nc) && alloc(c, &w.b, F * nc) &&
               alloc(c, &w.red, 6LL * PM_MAXF * 4096) && alloc(c, &w.scal, 16LL * PM_MAXF) &&
               alloc(c, &w.bar, 2) && alloc(c, &w.status, 1) && alloc(c, &w.empty, 1) && alloc(c, &w.ntri, 1) &&
-              alloc(c, &w.wsum, 8) && alloc(c, &w.nretry, 1) && alloc(c, &w.meshmax, PM_MAXF) &&
+              alloc(c, &w.wsum, 8) && alloc(c, &w.nretry, 2) && alloc(c, &w.meshmax, PM_MAXF) &&
               alloc(c, &w.pc, F * np) && alloc(c, &w.px, pcg_width((int)F) * np) &&
               alloc(c, &w.pq, pcg_width((int)F) * np) && alloc(c, &w.prp, 2LL * pcg_width((int)F) * np) &&
               alloc(c, &w.pp2, pcg_width((int)F) * np);

@@ -558,11 +558,11 @@ pm_status pm_batch_create(pm_batch **out, int ninst, const int *n, const double 
               cudaEventCreate(&b->t0) == cudaSuccess && cudaEventCreate(&b->t1) == cudaSuccess;
     ok = ok && balloc(&w.fx, NP) && balloc(&w.key, NP) && balloc(&w.slot, NP) && balloc(&w.count, NC) &&
          balloc(&w.cell_start, NC + 1) && balloc(&w.scan_tmp, NC / 4096 + 2) && balloc(&w.tmp, NP) &&
-         balloc(&w.perm, NP) && balloc(&w.pos, NP) && balloc(&w.vals, NP * F) &&
+         balloc(&w.perm, NP) && balloc(&w.pos, NP + PM_POS_PAD) && balloc(&w.vals, NP * F) &&
          balloc(&w.maxabs, (ll)PM_MAXF * ninst) && balloc(&w.deg, NP) && balloc(&w.vol, NP) &&
          balloc(&w.nbr, (ll)PM_MAXDEG * NP) && balloc(&w.bfix, F * NC) && balloc(&w.b, F * NC) &&
          balloc(&w.r, F * NC) && balloc(&w.p, F * NC) && balloc(&w.q, F * NC) &&
-         balloc(&w.scal, 16LL * PM_MAXF * ninst) && balloc(&w.status, 1) && balloc(&w.nretry, 1) &&
+         balloc(&w.scal, 16LL * PM_MAXF * ninst) && balloc(&w.status, 1) && balloc(&w.nretry, 2) &&
          balloc(&b->in_px, NP) && balloc(&b->in_py, NP) && balloc(&b->in_vals, NP * F) &&
          balloc(&b->d_inst, ninst) && balloc(&b->d_poff, ninst + 1) && balloc(&b->d_coff, ninst + 1) &&
          balloc(&b->d_rtile, ninst + 1) && balloc(&b->d_dtile, ninst + 1) && balloc(&b->d_order, ninst) &&

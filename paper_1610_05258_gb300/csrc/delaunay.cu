@@ -3,21 +3,36 @@
 // the periodically ordered particles (1D); and particle volumes
 // v_mu = int psi_mu (Sec. 2.1, Eq. part_v).
 //
-// 2D: one thread per particle p computes its Voronoi cell by clipping with
-// the bisectors of nearby particles, scanned ring by ring of mesh cells from
-// the cell-sorted array. The cell is a cyclic list of neighbours q_k; its
-// vertex k is the circumcentre of (p, q_k, q_k+1). A candidate s removes
-// vertex k iff s lies strictly inside the circle through (p, q_k, q_k+1):
-// the in-circle predicate, equivalently 2 c_k . s > |s|^2 for the
-// circumcentre c_k. It is decided in float from c_k and a rigorous bound on
-// its error, and exactly on the 32-bit torus coordinates (128-bit integers)
-// when the float value falls inside the error margin; exact ties are broken
-// by symbolic perturbation of the lifted coordinate |r|^2 + eps^rank, rank =
-// caller index. After ring r the cell is final once every vertex v
-// satisfies 2|v| < (distance from p to the unscanned cells). The neighbour
-// cycle is p's Delaunay star. Because every decision is exact and the
-// perturbation is a property of the point set, the stars of all particles
-// agree: every triangle (p, a, b) appears in the stars of p, a and b.
+// 2D: the Delaunay star of a particle p comes from three kinds of passes.
+//  * k_delaunay, one thread per particle: the star is the convex hull of the
+//    particles around p after inversion about p, found with float arithmetic
+//    whose every decision is certain (see below).
+//  * k_delaunay_wide, 8 lanes per particle, for what the first pass gives up:
+//    the same hull with a wider search, undecided tests made exactly.
+//  * k_delaunay_retry, one thread per particle, for the rest (regular lattices,
+//    stars of more than 24 neighbours, coincident particles, sets too sparse to
+//    certify): p's Voronoi cell is clipped by the bisectors of nearby
+//    particles, scanned ring by ring of mesh cells. The cell is a cyclic list of
+//    neighbours q_k; its vertex k is the circumcentre of (p, q_k, q_k+1). A
+//    candidate s removes vertex k iff s lies strictly inside the circle
+//    through (p, q_k, q_k+1): the in-circle predicate, equivalently
+//    2 c_k . s > |s|^2 for the circumcentre c_k. It is decided in float from
+//    c_k and a rigorous bound on its error, and exactly on the 32-bit torus
+//    coordinates (128-bit integers) when the float value falls inside the error
+//    margin. After ring r the cell is final once every vertex v satisfies
+//    2|v| < (distance from p to the unscanned cells).
+// Exact ties are broken by symbolic perturbation of the lifted coordinate
+// |r|^2 + eps^rank, rank = caller index. Because every decision is exact and
+// the perturbation is a property of the point set, the stars of all particles
+// agree, whatever pass made them: every triangle (p, a, b) appears in the stars
+// of p, a and b.
+//
+// Measured (16.8M clustered particles on 2048^2, all passes): 6.1 ms, against
+// 17.2 ms with the clipping alone as the main pass. Clipping ran 853 warp
+// instructions per particle with 8 of 32 lanes active, every lane at its own
+// candidate and its own polygon; the hull runs about 240 (+ 65 in the wide
+// pass, for 4 % of the particles) with 26 lanes active. Smallest calls gain
+// too, 262,144 particles from 518 to 170 us: no lane walks a long chain.
 #include "internal.cuh"
 
 PM_DEBUG_DECL(delaunay)
@@ -67,8 +82,6 @@ __device__ __forceinline__ int prio(int enc, const int *__restrict__ perm) {
     return id >= PM_VIRT ? 0x7ffffff0 + (id - PM_VIRT) : __ldg(perm + id);
 }
 
-#define DBLK 64     // threads per block of the main triangulation pass
-#define DCAP 9      // polygon capacity of the main pass (22 warps per SM)
 #define R1BLK 32    // threads per block of the first retry pass
 #define R1CAP 12    // polygon capacity of the first retry pass (17 warps per SM)
 #define RBLK 32     // threads per block of the last retry pass
@@ -423,46 +436,677 @@ __device__ __forceinline__ void add_counts(const WorkCount &wc, ull *__restrict_
     }
 }
 
-// Main pass: one thread per particle, polygon capacity DCAP. A particle whose
-// cell outgrows it is appended to the retry list (no output written).
-// Counters: wsum[0..4] the work of completed cells, wsum[5] the cells given
-// up by the main pass, wsum[6] those given up by the first retry pass.
+// ---------------------------------------------------------------------------
+// Main pass: the star as a convex hull.
+//
+// Inversion about p (u_s = (s - p) / |s - p|^2) takes the circles through p to
+// lines, and the neighbours of p's Voronoi cell to the vertices of the convex
+// hull of the inverted points: a circle through p, a, b is empty exactly when
+// every other u_s lies on the origin's side of the line through u_a and u_b.
+// So one thread per particle collects the candidates within a radius r_c and
+// finds the hull of their inversions by repeated queries "the point farthest
+// beyond the directed edge (a, b)": a point beyond the edge is inserted
+// between a and b, and an edge with nothing beyond it is a star triangle. All
+// lanes of a warp run the same straight-line query over the same number of
+// list slots; only the number of queries differs (2 m - 1 for m neighbours).
+//
+// Every decision is certain or taken exactly. With E = 5e-7 bounding the
+// relative error of each component of u (conversion, |s|^2, reciprocal and
+// product roundings) and U = max |u| (the nearest particle), the float value of
+// n . (u_s - u_a), n the float normal of (a, b), is off by less than
+//   mg = 2.7e-6 U (|u_a| + |u_b|)
+// (2 E |n| U for the points, 2 E U (|u_a| + |u_b|) for the normal, 10 units of
+// roundoff times |n| U for the evaluation, |n| <= |u_a| + |u_b|). Queries run on
+// w = (n . (u_s - u_a)) / mg + 1.25, itself good to 0.1: a maximum above 2.5 is
+// certainly beyond the edge; points with w <= 0 are certainly not. When a and b
+// are the only points with w > 0 (the sum of w clamped to [0, 1] is 2) nothing is
+// beyond; otherwise the few others are decided by the exact predicate. The
+// points that were not collected are at least r_c away, so their inversions lie
+// in the disc of radius 1 / r_c, which a final edge must clear too (this is the
+// test that the cell is certified: 2 |circumcentre| < r_c). A hull that meets
+// the disc, a full list, more than HDEG neighbours, or an edge whose side of p
+// is not certain sends the particle to the wide pass; coincident particles go
+// to the exact passes.
+// ---------------------------------------------------------------------------
+// HN and HL are a balance: fewer candidates make the queries shorter and the
+// wide list longer (HN 24, 26, 28, 30 with HL 40: 6.57, 6.35, 6.43, 6.87 ms on
+// the set above before the 5 x 5 density, 28 best with it; HL 32: 8.2 ms, HL 48:
+// 8.3 ms). The lists take 80 registers, so 8 blocks of 64 threads are resident.
+#define HBLK 64        // threads per block
+#define HMINB 8        // resident blocks per SM
+#define HL 40          // list slots per particle
+#define HN 28.0f       // expected number of candidates within r_c
+#define HRMAX 6        // largest r_c, in cells
+#define HDEG 10        // largest star of this pass (6-bit indices packed into 64 bits)
+
+typedef unsigned long long f32x2;  // two floats of a packed FP32 operation
+__device__ __forceinline__ f32x2 pk2(float a, float b) {
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ void up2(f32x2 v, float &a, float &b) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+    f32x2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ float fma_sat(float a, float b, float c) {
+    float r;
+    asm("fma.rn.sat.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+    return r;
+}
+__device__ __forceinline__ float rcp_approx(float x) {
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+__device__ __forceinline__ float sqrt_approx(float x) {
+    float r;
+    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+
+// The bits of w with the low 6 replaced by the slot (0..63); positive values
+// order as integers.
+__device__ __forceinline__ int tag6(float w, unsigned keep, unsigned slot) {
+    unsigned r;  // (w & keep) | slot
+    asm("lop3.b32 %0, %1, %2, %3, 0xEA;" : "=r"(r) : "r"(__float_as_uint(w)), "r"(keep), "r"(slot));
+    return (int)r;
+}
+
+// Search disc of a particle: radius in cells (at most lim) that holds about
+// `want` particles at the density of the 3 x 3 cells around (cx, cy), or, where
+// those hold fewer than 20, of the 5 x 5 (cut at the box edge in x).
+__device__ __forceinline__ float search_radius(const Geo &g, const int *__restrict__ cell_start, int cx, int cy,
+                                               float want, int lim) {
+    const int n = g.n;
+    int cnt = 0, cells = 0;
+    for (int h = 1; h <= 2; ++h) {
+        const int xa = max(cx - h, 0), xb = min(cx + h, n - 1);
+        cnt = 0;
+        cells = (2 * h + 1) * (xb - xa + 1);
+        for (int dy = -h; dy <= h; ++dy) {
+            int y = cy + dy;
+            y = y < 0 ? y + n : (y >= n ? y - n : y);
+            cnt += __ldg(cell_start + (ll)y * n + xb + 1) - __ldg(cell_start + (ll)y * n + xa);
+        }
+        if (cnt >= 20 || n < 8) break;
+    }
+    const float r2 = want * (1.0f / 3.14159265f) * (float)cells * rcp_approx((float)max(cnt, 1));
+    return fminf(sqrt_approx(r2), (float)min(lim, n / 4 - 1));
+}
+
+// Sorted slots of the cells of row cy + dy that the disc of radius rs around p
+// (offset (fx, fy) in its cell, cell units) meets: [s0, s1) and, where the row
+// crosses the box edge, [t0, t1). rs carries the slack against the roundings.
+__device__ __forceinline__ void row_range(const int *__restrict__ cell_start, int n, int cx, int cy, int dy, float fx,
+                                          float fy, float rs, int &s0, int &s1, int &t0, int &t1) {
+    const float gy = dy > 0 ? (float)dy - fy : (dy < 0 ? fy - (float)(dy + 1) : 0.0f);
+    const float hw = sqrt_approx(fmaxf(rs * rs - gy * gy, 0.0f)) * 1.0001f;
+    const int ux0 = cx + (int)floorf(fx - hw), ux1 = cx + (int)floorf(fx + hw);
+    int y = cy + dy;
+    y = y < 0 ? y + n : (y >= n ? y - n : y);
+    const int *cs = cell_start + (ll)y * n;
+    s0 = __ldg(cs + max(ux0, 0));
+    s1 = __ldg(cs + min(ux1, n - 1) + 1);
+    t0 = t1 = 0;
+    if (ux0 < 0) {
+        t0 = __ldg(cs + ux0 + n);
+        t1 = __ldg(cs + n);
+    } else if (ux1 >= n) {
+        t0 = __ldg(cs);
+        t1 = __ldg(cs + ux1 - n + 1);
+    }
+}
+
+// Star entry of sorted neighbour s at Xs: index and image code of its minimal
+// image; (rx, ry) its offset from p.
+__device__ __forceinline__ int star_entry(int s, uint2 Xs, uint2 Xp, int &rx, int &ry) {
+    rx = (int)(Xs.x - Xp.x);
+    ry = (int)(Xs.y - Xp.y);
+    const int ox = rx >= 0 ? (Xs.x < Xp.x ? 1 : 0) : (Xs.x > Xp.x ? -1 : 0);
+    const int oy = ry >= 0 ? (Xs.y < Xp.y ? 1 : 0) : (Xs.y > Xp.y ? -1 : 0);
+    return s | (((ox + 1) * 3 + (oy + 1)) << 28);
+}
+
+// Star written; needs a wider search; needs exact tests; undecided tests.
+enum { HULL_DONE = 1, HULL_WIDER = 2, HULL_EXACT = 3, HULL_UNSURE = 4 };
+
+// Inversion about Xp, in units of 1 / cell (cw: torus units per cell); the
+// origin for p itself.
+struct Inversion {
+    uint2 Xp;
+    float cw;
+    __device__ __forceinline__ float operator()(uint2 X, float &ux, float &uy) const {
+        const float sx = (float)(int)(X.x - Xp.x), sy = (float)(int)(X.y - Xp.y), d2 = sx * sx + sy * sy;
+        const float iv = d2 > 0.0f ? rcp_approx(d2) * cw : 0.0f;
+        ux = sx * iv;
+        uy = sy * iv;
+        return d2;
+    }
+};
+
+// All lanes of the warp call this together (live: the lane has a particle).
+// ids: the block's list columns, HL + 4 rows (the last rows take the candidates
+// of a full list); stk: the stack of hull vertices (u, slot).
 template <bool COUNT>
-__global__ void __launch_bounds__(DBLK, 11) k_delaunay(Geo g, ll np, const uint2 *__restrict__ pos,
-                                                   const int *__restrict__ cell_start, const int *__restrict__ perm,
-                                                   int *__restrict__ nbr, unsigned char *__restrict__ deg,
-                                                   float *__restrict__ vol, float vol_scale, int *__restrict__ status,
-                                                   int *__restrict__ retry, int *__restrict__ nretry,
-                                                   ull *__restrict__ wsum) {
-    __shared__ int4 sq[DCAP][DBLK];
-    __shared__ float4 sv[DCAP][DBLK];
-    const ll pl = (ll)blockIdx.x * DBLK + threadIdx.x;
-    WorkCount wc;
-    if (pl < np) {
-        const int p = (int)pl;
-        PolyS<DBLK> P{sq, sv, (int)threadIdx.x};
-        const int err = star_of<DCAP, DBLK, COUNT>(P, p, g, np, pos, cell_start, perm, nbr, deg, vol, vol_scale, wc);
-        if (err == ST_OVERFLOW) {
-            if (COUNT) {
-                wc = WorkCount{};
-                wc.over = 1;
+__device__ __forceinline__ int star_hull(int (*ids)[HBLK], float4 (*stk)[HBLK], bool live, int p, const Geo &g, ll np,
+                                         const uint2 *__restrict__ pos, const int *__restrict__ cell_start,
+                                         const int *__restrict__ perm, int *__restrict__ nbr,
+                                         unsigned char *__restrict__ deg, float *__restrict__ vol, float vol_scale,
+                                         WorkCount &wc) {
+    const int t = (int)threadIdx.x, n = g.n;
+    const uint2 Xp = live ? pos[p] : make_uint2(0u, 0u);
+    const Inversion inv{Xp, 4294967296.0f / (float)n};
+    int *const col = &ids[0][0];
+    int q = t;
+    float ri2 = 0.0f;
+    if (live) {
+        const int cx = cell_of(Xp.x, n), cy = cell_of(Xp.y, n);
+        const float fx = frac_f(Xp.x, n), fy = frac_f(Xp.y, n);
+        const float r = search_radius(g, cell_start, cx, cy, HN, HRMAX), rs = r * 1.0001f + 1e-6f;
+        const float r2 = (r * inv.cw) * (r * inv.cw);
+        ri2 = rcp_approx(r * r) * 1.0002f;
+        const int y1 = (int)floorf(fy + rs);
+        for (int dy = (int)floorf(fy - rs); dy <= y1; ++dy) {
+            int s0, s1, t0, t1;
+            row_range(cell_start, n, cx, cy, dy, fx, fy, rs, s0, s1, t0, t1);
+            for (;;) {
+                PM_CHK(s0 >= 0 && s1 <= np, 209, break)
+                if (COUNT) wc.cand += s1 - s0;
+                // four candidates at a time, the next four on their way, without
+                // branches: every slot is stored, the column advances past the
+                // ones in the disc. Loads past s1 stay within the array's
+                // padding and are masked.
+                uint2 Xn[4];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) Xn[k] = __ldg(pos + s0 + k);
+                for (int s = s0; s < s1; s += 4) {
+                    uint2 Xs[4];
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) Xs[k] = Xn[k];
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) Xn[k] = __ldg(pos + s + 4 + k);
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        const float sx = (float)(int)(Xs[k].x - Xp.x), sy = (float)(int)(Xs[k].y - Xp.y);
+                        col[q] = s + k;
+                        q += (s + k < s1 && sx * sx + sy * sy < r2) ? HBLK : 0;
+                    }
+                    q = min(q, HL * HBLK + t);
+                }
+                if (t0 >= t1) break;
+                s0 = t0;
+                s1 = t1;
+                t0 = t1;
             }
-            const int k = atomicAdd(nretry, 1);
-            PM_CHK(k >= 0 && k < np, 205, k = -1)
-            if (k >= 0) retry[k] = p;
-        } else if (err) {
-            atomicOr(status, err & ~ST_OVERFLOW);
-            deg[p] = 0;
-            vol[p] = 0.0f;
         }
     }
+    const int cnt = (q - t) / HBLK;  // p itself included; HL: the list is full
+    if (COUNT) wc.tested += cnt;
+    int state = !live || cnt < 4 || cnt >= HL ? HULL_WIDER : 0;  // 0: running
+    const int used = __reduce_max_sync(0xffffffffu, state == 0 ? cnt : 0);
+    if (used == 0) return state;
+    // The inverted candidates, in registers; slots past the lane's own list
+    // hold the origin, which is never beyond an edge. The extremes in x and y
+    // start the hull: the largest bit pattern as a signed integer is the
+    // largest positive value, as an unsigned one the most negative.
+    f32x2 xx[HL / 2], yy[HL / 2];
+    unsigned keep = 0xffffffc0u;
+    asm("" : "+r"(keep));  // one register: (w & keep) | slot is a single LOP3
+    int xmax = 0, ymax = 0, zeros = 0;
+    unsigned xmin = 0u, ymin = 0u;
+#pragma unroll
+    for (int c = 0; c < HL / 8; ++c) {
+        if (c * 8 < used) {
+            uint2 Xs[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) Xs[k] = c * 8 + k < cnt ? __ldg(pos + ids[c * 8 + k][t]) : Xp;
+#pragma unroll
+            for (int k = 0; k < 8; k += 2) {
+                const int j = c * 8 + k;
+                float ux[2], uy[2];
+                zeros += inv(Xs[k], ux[0], uy[0]) > 0.0f ? 0 : 1;
+                zeros += inv(Xs[k + 1], ux[1], uy[1]) > 0.0f ? 0 : 1;
+                const int x0 = tag6(ux[0], keep, j), x1 = tag6(ux[1], keep, j + 1);
+                const int y0 = tag6(uy[0], keep, j), y1 = tag6(uy[1], keep, j + 1);
+                xmax = __vimax3_s32(xmax, x0, x1);
+                ymax = __vimax3_s32(ymax, y0, y1);
+                xmin = __vimax3_u32(xmin, (unsigned)x0, (unsigned)x1);
+                ymin = __vimax3_u32(ymin, (unsigned)y0, (unsigned)y1);
+                xx[c * 4 + k / 2] = pk2(ux[0], ux[1]);
+                yy[c * 4 + k / 2] = pk2(uy[0], uy[1]);
+            }
+        }
+    }
+    const int fill = (used + 7) & ~7;
+    if (state == 0 && zeros != fill - cnt + 1) state = HULL_EXACT;  // coincident particles
+    // no point on one side of p in x or y: p is not inside the hull
+    if (state == 0 && (xmax < 64 || ymax < 64 || (int)xmin > -64 || (int)ymin > -64)) state = HULL_WIDER;
+    // U >= |u| of every candidate (the tags take at most 2^-17 off a component)
+    const float ex = fmaxf(__int_as_float(xmax), -__uint_as_float(xmin)), ey = fmaxf(__int_as_float(ymax), -__uint_as_float(ymin));
+    const float U27 = 2.7e-6f * 1.00003f * sqrt_approx(ex * ex + ey * ey);
+    int a = 0, b = 0, m = 0, depth = 0;  // edge (a, b); the stack's top, b, is row depth; row 0 closes the cycle
+    ull out = 0;
+    float ax = 0.0f, ay = 0.0f, bx = 0.0f, by = 0.0f;
+    if (state == 0) {
+        // ccw from the largest x: the vertices still ahead, the last one first
+        a = xmax & 63;
+        inv(__ldg(pos + ids[a][t]), ax, ay);
+        stk[0][t] = make_float4(ax, ay, __int_as_float(a), 0.0f);
+        b = a;
+        bx = ax;
+        by = ay;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const int v = (int)((k == 0 ? ymin : (k == 1 ? xmin : (unsigned)ymax)) & 63u);
+            if (v != b && v != a) {
+                b = v;
+                inv(__ldg(pos + ids[b][t]), bx, by);
+                stk[++depth][t] = make_float4(bx, by, __int_as_float(b), 0.0f);
+            }
+        }
+        if (depth == 0) state = HULL_WIDER;
+    }
+    while (__any_sync(0xffffffffu, state == 0)) {
+        // what lies beyond the edge (a, b)?
+        const float nx = by - ay, ny = ax - bx, mg = U27 * ((fabsf(ax) + fabsf(ay)) + (fabsf(bx) + fabsf(by)));
+        const float im = rcp_approx(mg), sx = nx * im, sy = ny * im, c0 = 1.25f - fmaf(sx, ax, sy * ay);
+        const f32x2 sx2 = pk2(sx, sx), sy2 = pk2(sy, sy), c2 = pk2(c0, c0);
+        int M = 0;       // largest w as an ordered integer, tagged with its slot
+        unsigned S = 0;  // number of w < 0
+#pragma unroll
+        for (int c = 0; c < HL / 8; ++c) {
+            if (c * 8 < used) {
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const int j = c * 4 + k;
+                    const f32x2 w = fma2(sy2, yy[j], fma2(sx2, xx[j], c2));
+                    float w0, w1;
+                    up2(w, w0, w1);
+                    S += __float_as_uint(w0) >> 31;
+                    S += __float_as_uint(w1) >> 31;
+                    M = __vimax3_s32(M, tag6(w0, keep, 2 * j), tag6(w1, keep, 2 * j + 1));
+                }
+            }
+        }
+        if (state == 0) {
+            const float T = fmaf(nx, ax, ny * ay);
+            if (COUNT) wc.vtests += cnt;
+            if (M >= 0x40200000 + 64) {  // w > 2.5: insert the vertex
+                ++depth;
+                b = M & 63;
+                if (COUNT) {
+                    wc.clips++;
+                    wc.msum += m + depth + 1;
+                }
+                if (depth >= HDEG || b >= cnt) {
+                    state = HULL_WIDER;
+                } else {
+                    inv(__ldg(pos + ids[b][t]), bx, by);
+                    stk[depth][t] = make_float4(bx, by, __int_as_float(b), 0.0f);
+                }
+            } else if (!(T > mg && (T - mg) * (T - mg) > (nx * nx + ny * ny) * ri2) || m >= HDEG) {
+                state = HULL_WIDER;
+            } else if (S != (unsigned)(fill - 2)) {
+                state = HULL_UNSURE;
+            } else {  // a final edge
+                out = (out << 6) | (ull)a;
+                ++m;
+                a = b;
+                ax = bx;
+                ay = by;
+                if (--depth < 0) {
+                    state = HULL_DONE;
+                } else {
+                    const float4 q4 = stk[depth][t];
+                    bx = q4.x;
+                    by = q4.y;
+                    b = __float_as_int(q4.z);
+                }
+            }
+        }
+    }
+    // A few undecided lanes go to the wide pass, which decides exactly; where
+    // they are many (a regular lattice) the exact passes are the faster way.
+    if (__popc(__ballot_sync(0xffffffffu, state == HULL_UNSURE)) > 4 && state == HULL_UNSURE) state = HULL_EXACT;
+    if (state != HULL_DONE || m < 3) return state == HULL_EXACT ? HULL_EXACT : HULL_WIDER;
+    // the star, counter-clockwise from the nearest particle
+    ll area2 = 0;
+    int fx0 = 0, fy0 = 0, px = 0, py = 0;
+    for (int k = 0; k < m; ++k) {
+        const int s = ids[(int)((out >> (6 * (m - 1 - k))) & 63)][t];
+        PM_CHK(s >= 0 && s < np, 210, return HULL_EXACT)
+        int rx, ry;
+        nbr[(ll)k * np + p] = star_entry(s, __ldg(pos + s), Xp, rx, ry);
+        if (k == 0) {
+            fx0 = rx;
+            fy0 = ry;
+        } else {
+            area2 += (ll)px * ry - (ll)py * rx;
+        }
+        px = rx;
+        py = ry;
+    }
+    area2 += (ll)px * fy0 - (ll)py * fx0;
+    deg[p] = (unsigned char)m;
+    vol[p] = (float)area2 * vol_scale;
+    return HULL_DONE;
+}
+
+// Append this lane's particle to a list (one atomic per warp).
+__device__ __forceinline__ void push_list(bool add, int p, ll np, int *__restrict__ list, int *__restrict__ count) {
+    const unsigned ball = __ballot_sync(0xffffffffu, add);
+    if (!ball) return;
+    const int lane = threadIdx.x & 31;
+    int base = 0;
+    if (lane == 0) base = atomicAdd(count, __popc(ball));
+    base = __shfl_sync(0xffffffffu, base, 0);
+    if (add) {
+        const int k = base + __popc(ball & ((1u << lane) - 1u));
+        PM_CHK(k >= 0 && k < np, 205, return)
+        list[k] = p;
+    }
+}
+
+// The lists of the particles that the hull passes give up: wide[] with
+// counts[0] entries (after the main pass) and exact[] with counts[1] entries.
+struct Lists {
+    int *wide, *exact, *counts;
+};
+
+// Counters: wsum[0..4] the work of completed cells, wsum[5] the cells given
+// up by the main pass, wsum[6] those given up by the first exact pass.
+template <bool COUNT>
+__global__ void __launch_bounds__(HBLK, HMINB) k_delaunay(Geo g, ll np, const uint2 *__restrict__ pos,
+                                                   const int *__restrict__ cell_start, const int *__restrict__ perm,
+                                                   int *__restrict__ nbr, unsigned char *__restrict__ deg,
+                                                   float *__restrict__ vol, float vol_scale, Lists L, ull *__restrict__ wsum) {
+    __shared__ int ids[HL + 4][HBLK];
+    __shared__ float4 stk[HDEG][HBLK];
+    const ll pl = (ll)blockIdx.x * HBLK + threadIdx.x;
+    const bool live = pl < np;
+    WorkCount wc;
+    const int e = star_hull<COUNT>(ids, stk, live, (int)pl, g, np, pos, cell_start, perm, nbr, deg, vol, vol_scale, wc);
+    if (COUNT && live && e != HULL_DONE) {
+        wc = WorkCount{};
+        wc.over = 1;
+    }
+    push_list(live && e == HULL_WIDER, (int)pl, np, L.wide, L.counts);
+    push_list(live && e == HULL_EXACT, (int)pl, np, L.exact, L.counts + 1);
     add_counts<COUNT>(wc, wsum, 5);
 }
 
-// Retry passes over the listed particles (grid-stride). The first (capacity
-// R1CAP, LAST false) marks a particle whose cell outgrows it by storing ~p in
-// its list entry; the last (capacity RCAP, LAST true) takes only the marked
-// entries.
+// ---------------------------------------------------------------------------
+// Wide pass: the hull of a particle of the wide list by a group of 8 lanes,
+// over up to 96 candidates (12 registers per lane). A query is 12 candidates
+// per lane and a 3-step reduction, so a star takes microseconds, where one lane
+// with a long list would hold up a warp. The same tests and margins as in the
+// main pass, with undecided candidates decided exactly on the spot. The first
+// search takes a disc that should hold 48 candidates; where the hull of what it
+// finds is complete but not certified, its largest circle gives the radius of
+// the next. Up to PM_MAXDEG neighbours.
+// ---------------------------------------------------------------------------
+#define WBLK 128
+#define WG (WBLK / 8)  // groups per block
+#define WL 96          // list slots per group
+#define WN 48.0f       // expected candidates of the first search
+#define WTRIES 4       // searches per particle
+
+struct WideS {
+    float x[WL], y[WL];
+    int id[WL];
+    float ex[PM_MAXDEG], ey[PM_MAXDEG], et[PM_MAXDEG];  // edges of the last complete hull
+    unsigned char st[PM_MAXDEG + 2], out[PM_MAXDEG + 2];
+};
+
+// All lanes of the warp call this together, the 8 lanes of a group with the
+// same particle. HULL_DONE, or HULL_EXACT where the exact passes are needed.
+template <bool COUNT>
+__device__ __forceinline__ int star_wide(WideS &G, bool live, int p, const Geo &g, ll np, const uint2 *__restrict__ pos,
+                                         const int *__restrict__ cell_start, const int *__restrict__ perm,
+                                         int *__restrict__ nbr, unsigned char *__restrict__ deg,
+                                         float *__restrict__ vol, float vol_scale, WorkCount &wc) {
+    const unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x & 31, sub = lane & 7, sh = lane & 24;
+    const int n = g.n;
+    const uint2 Xp = live ? pos[p] : make_uint2(0u, 0u);
+    const Inversion inv{Xp, 4294967296.0f / (float)n};
+    const int cx = cell_of(Xp.x, n), cy = cell_of(Xp.y, n);
+    const float fx = frac_f(Xp.x, n), fy = frac_f(Xp.y, n);
+    const float rlim = (float)min(PM_RCAP, n / 4 - 1);
+    float r = live ? search_radius(g, cell_start, cx, cy, WN, PM_RCAP) : 0.0f;
+    int result = live ? 0 : HULL_EXACT, cnt = 0, m = 0, edges = 0;  // result 0: not finished
+    for (int tries = 0; tries < WTRIES && __any_sync(FULL, result == 0); ++tries) {
+        const bool act = result == 0;
+        const float rs = r * 1.0001f + 1e-6f, r2 = (r * inv.cw) * (r * inv.cw), ri2 = rcp_approx(r * r) * 1.0002f;
+        bool dup = false;
+        if (act) cnt = 0;
+        const int y0 = (int)floorf(fy - rs), y1 = act ? (int)floorf(fy + rs) : y0 - 1;
+        for (int dy = y0; __any_sync(FULL, dy <= y1); ++dy) {
+            int s0 = 0, s1 = 0, t0 = 0, t1 = 0;
+            if (dy <= y1) row_range(cell_start, n, cx, cy, dy, fx, fy, rs, s0, s1, t0, t1);
+            for (;;) {
+                PM_CHK(s0 >= 0 && s1 <= np, 211, s1 = s0)
+                if (COUNT && sub == 0) wc.cand += s1 - s0;
+                for (int s = s0 + sub; __any_sync(FULL, s - sub < s1); s += 8) {
+                    bool hit = false;
+                    if (s < s1) {
+                        const uint2 Xs = __ldg(pos + s);
+                        const int rx = (int)(Xs.x - Xp.x), ry = (int)(Xs.y - Xp.y);
+                        const float sx = (float)rx, sy = (float)ry;
+                        hit = sx * sx + sy * sy < r2 && s != p;
+                        dup |= hit && (rx | ry) == 0;
+                        if (hit && edges) {  // strictly inside the last hull: cannot matter
+                            float ux, uy;
+                            inv(Xs, ux, uy);
+                            hit = false;
+                            for (int k = 0; k < edges; ++k) hit |= fmaf(G.ex[k], ux, G.ey[k] * uy) > G.et[k];
+                        }
+                    }
+                    const unsigned ball = (__ballot_sync(FULL, hit) >> sh) & 0xffu;
+                    const int k = cnt + __popc(ball & ((1u << sub) - 1u));
+                    if (hit && k < WL) G.id[k] = s;
+                    cnt += __popc(ball);
+                }
+                if (!__any_sync(FULL, t0 < t1)) break;
+                s0 = t0;
+                s1 = t1;
+                t0 = t1;
+            }
+        }
+        __syncwarp();
+        if (((__ballot_sync(FULL, dup) >> sh) & 0xffu) != 0 && act) result = HULL_EXACT;
+        if (COUNT && sub == 0 && act) wc.tested += cnt;
+        // 0: querying, 1: hull complete, 2: no use
+        int state = act && result == 0 && cnt >= 3 && cnt <= WL ? 0 : 2;
+        float X[WL / 8], Y[WL / 8];
+        unsigned near = 0xffffffffu;
+#pragma unroll
+        for (int k = 0; k < WL / 8; ++k) {
+            const int j = k * 8 + sub;
+            X[k] = Y[k] = __int_as_float(0x7fc00000);  // no slot: never beyond an edge
+            if (state == 0 && j < cnt) {
+                const float d2 = inv(__ldg(pos + G.id[j]), X[k], Y[k]);
+                G.x[j] = X[k];
+                G.y[j] = Y[k];
+                near = min(near, (__float_as_uint(d2) & ~127u) | (unsigned)j);
+            }
+        }
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) near = min(near, __shfl_xor_sync(FULL, near, o));
+        __syncwarp();
+        int a = (int)(near & 127u), depth = 1;
+        // U >= |u| of the nearest (the tag takes at most 2^-16 off |s|^2)
+        const float U = sqrt_approx(rcp_approx(__uint_as_float(near & ~127u)) * 1.00005f) * inv.cw;
+        float ax = 0.0f, ay = 0.0f, bx = 0.0f, by = 0.0f, need2 = 0.0f;
+        int b = 0;
+        if (state == 0) {
+            m = 0;
+            ax = G.x[a];
+            ay = G.y[a];
+            if (sub == 0) G.st[0] = (unsigned char)a;
+        }
+        bool first = true;
+        while (__any_sync(FULL, state == 0)) {
+            float nx = by - ay, ny = ax - bx, mg = 2.7e-6f * U * ((fabsf(ax) + fabsf(ay)) + (fabsf(bx) + fabsf(by)));
+            if (first) {
+                nx = -ax;
+                ny = -ay;
+                mg = U * U;
+            }
+            const float im = rcp_approx(mg), sx = nx * im, sy = ny * im, c0 = 1.25f - fmaf(sx, ax, sy * ay);
+            // largest w (as an ordered integer, tagged with its slot), number of w > 0
+            unsigned M = 0u;
+            int S = 0;
+#pragma unroll
+            for (int k = 0; k < WL / 8; ++k) {
+                const float w = fmaf(sy, Y[k], fmaf(sx, X[k], c0));
+                if (w > 0.0f) {
+                    M = max(M, (__float_as_uint(w) & ~127u) | (unsigned)(k * 8 + sub));
+                    ++S;
+                }
+            }
+#pragma unroll
+            for (int o = 4; o > 0; o >>= 1) {
+                M = max(M, __shfl_xor_sync(FULL, M, o));
+                S += __shfl_xor_sync(FULL, S, o);
+            }
+            if (COUNT && state == 0 && sub == 0) wc.vtests += cnt;
+            int v = first || M >= 0x40200000u + 128u ? (int)(M & 127u) : -1;  // w > 2.5: the vertex to insert
+            if (__any_sync(FULL, state == 0 && v < 0 && S != 2)) {
+                // undecided candidates, exactly
+                int e = 255;
+                if (state == 0 && v < 0 && S != 2 && fmaf(nx, ax, ny * ay) > mg) {
+                    const uint2 A = __ldg(pos + G.id[a]), B = __ldg(pos + G.id[b]);
+                    for (int j = sub; j < cnt && e == 255; j += 8) {
+                        if (j == a || j == b || !(fmaf(sy, G.y[j], fmaf(sx, G.x[j], c0)) > 0.0f)) continue;
+                        const uint2 Q = __ldg(pos + G.id[j]);
+                        if (incircle_exact((int)(A.x - Xp.x), (int)(A.y - Xp.y), (int)(B.x - Xp.x), (int)(B.y - Xp.y),
+                                           (int)(Q.x - Xp.x), (int)(Q.y - Xp.y), perm[p], perm[G.id[a]],
+                                           perm[G.id[b]], perm[G.id[j]]))
+                            e = j;
+                    }
+                    if (COUNT) wc.exact++;
+                }
+#pragma unroll
+                for (int o = 4; o > 0; o >>= 1) e = min(e, __shfl_xor_sync(FULL, e, o));
+                if (v < 0 && e < 255) v = e;
+            }
+            if (state == 0) {
+                const float T = fmaf(nx, ax, ny * ay);
+                if (v >= 0) {
+                    if (depth >= PM_MAXDEG || v >= cnt) {
+                        state = 2;
+                    } else {
+                        b = v;
+                        if (sub == 0) G.st[depth] = (unsigned char)b;
+                        ++depth;
+                        bx = G.x[b];
+                        by = G.y[b];
+                        if (COUNT && sub == 0) {
+                            wc.clips++;
+                            wc.msum += m + depth;
+                        }
+                    }
+                } else if ((!(T > mg) && S != 2) || m >= PM_MAXDEG) {
+                    state = 2;
+                } else {
+                    // a final edge of this hull; need2: the squared radius that certifies it
+                    need2 = fmaxf(need2, T > mg ? (nx * nx + ny * ny) * rcp_approx((T - mg) * (T - mg)) : 1e30f);
+                    if (sub == 0) G.out[m] = (unsigned char)a;
+                    ++m;
+                    a = b;
+                    ax = bx;
+                    ay = by;
+                    if (--depth == 0) {
+                        state = 1;
+                    } else {
+                        b = G.st[depth - 1];
+                        bx = G.x[b];
+                        by = G.y[b];
+                    }
+                }
+            }
+            first = false;
+            __syncwarp();
+        }
+        if (act && result == 0) {
+            if (state == 1 && need2 * ri2 * 1.0001f < 1.0f)
+                result = m >= 3 ? HULL_DONE : HULL_EXACT;
+            else if (cnt > WL)
+                r *= sqrt_approx(0.7f * (float)WL * rcp_approx((float)cnt));
+            else if (r >= rlim)
+                result = HULL_EXACT;
+            else
+                r = fminf(state == 1 && need2 < 1e30f ? sqrt_approx(need2) * 1.001f : 1.6f * r, rlim);
+            if (result == 0 && state == 1) {  // the next search drops what lies inside this hull
+                edges = m;
+                for (int k = sub; k < m; k += 8) {
+                    const int i0 = G.out[k], i1 = G.out[k + 1 == m ? 0 : k + 1];
+                    const float x0 = G.x[i0], y0 = G.y[i0], x1 = G.x[i1], y1 = G.y[i1];
+                    G.ex[k] = y1 - y0;
+                    G.ey[k] = x0 - x1;
+                    G.et[k] = fmaf(G.ex[k], x0, G.ey[k] * y0) -
+                              1e-5f * U * ((fabsf(x0) + fabsf(y0)) + (fabsf(x1) + fabsf(y1)));
+                }
+            }
+        }
+        __syncwarp();
+    }
+    const bool done = result == HULL_DONE;
+    ll area2 = 0;
+    for (int k = sub; done && k < m; k += 8) {
+        const int s = G.id[G.out[k]], s2 = G.id[G.out[k + 1 == m ? 0 : k + 1]];
+        int rx, ry, qx, qy;
+        nbr[(ll)k * np + p] = star_entry(s, __ldg(pos + s), Xp, rx, ry);
+        star_entry(s2, __ldg(pos + s2), Xp, qx, qy);
+        area2 += (ll)rx * qy - (ll)ry * qx;
+    }
+    __syncwarp();
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) area2 += __shfl_xor_sync(FULL, area2, o);
+    if (done && sub == 0) {
+        deg[p] = (unsigned char)m;
+        vol[p] = (float)area2 * vol_scale;
+        if (COUNT && m > R1CAP) wc.over++;
+    }
+    return done ? HULL_DONE : HULL_EXACT;
+}
+
+template <bool COUNT>
+__global__ void __launch_bounds__(WBLK) k_delaunay_wide(Geo g, ll np, const uint2 *__restrict__ pos,
+                                                        const int *__restrict__ cell_start,
+                                                        const int *__restrict__ perm, int *__restrict__ nbr,
+                                                        unsigned char *__restrict__ deg, float *__restrict__ vol,
+                                                        float vol_scale, Lists L, ull *__restrict__ wsum) {
+    __shared__ WideS G[WG];
+    const int cnt = L.counts[0], gid = threadIdx.x >> 3;
+    WorkCount wc;
+    for (ll j0 = (ll)blockIdx.x * WG; j0 < cnt; j0 += (ll)gridDim.x * WG) {
+        const ll j = j0 + gid;
+        const bool live = j < cnt;
+        const int p = live ? L.wide[j] : 0;
+        const WorkCount before = wc;
+        const int e = star_wide<COUNT>(G[gid], live, p, g, np, pos, cell_start, perm, nbr, deg, vol, vol_scale, wc);
+        const bool over = live && e != HULL_DONE && (threadIdx.x & 7) == 0;
+        if (COUNT && over) wc = before;
+        push_list(over, p, np, L.exact, L.counts + 1);
+    }
+    add_counts<COUNT>(wc, wsum, 6);
+}
+
+// Exact passes over the exact list (grid-stride). The first (capacity R1CAP,
+// LAST false) marks a particle whose cell outgrows it by storing ~p in its list
+// entry; the last (capacity RCAP, LAST true) takes only the marked entries.
 template <int CAP, int NB, bool LAST, bool COUNT>
 __global__ void __launch_bounds__(NB) k_delaunay_retry(Geo g, ll np, const uint2 *__restrict__ pos,
                                                        const int *__restrict__ cell_start,
@@ -497,37 +1141,47 @@ __global__ void __launch_bounds__(NB) k_delaunay_retry(Geo g, ll np, const uint2
             vol[p] = 0.0f;
         }
     }
-    add_counts<COUNT>(wc, wsum, 6);  // the first retry pass's give-ups (none in the last)
+    add_counts<COUNT>(wc, wsum, 6);  // the first exact pass's give-ups (none in the last)
 }
 
 // Batched passes: the particle's instance comes from the packed offsets; its
 // mesh, cell ranges and volume scale from the instance table. Stars hold
 // packed sorted indices (< 2^28 in total).
-__global__ void __launch_bounds__(DBLK, 11) k_delaunay_b(BTab t, const uint2 *__restrict__ pos,
+__global__ void __launch_bounds__(HBLK, HMINB) k_delaunay_b(BTab t, const uint2 *__restrict__ pos,
                                                      const int *__restrict__ cell_start, const int *__restrict__ perm,
-                                                     int *__restrict__ nbr, unsigned char *__restrict__ deg,
-                                                     float *__restrict__ vol, int *__restrict__ status,
-                                                     int *__restrict__ retry, int *__restrict__ nretry) {
-    __shared__ int4 sq[DCAP][DBLK];
-    __shared__ float4 sv[DCAP][DBLK];
-    const ll pl = (ll)blockIdx.x * DBLK + threadIdx.x;
+                                                     int *__restrict__ nbr,
+                                                     unsigned char *__restrict__ deg, float *__restrict__ vol,
+                                                     Lists L) {
+    __shared__ int ids[HL + 4][HBLK];
+    __shared__ float4 stk[HDEG][HBLK];
+    const ll pl = (ll)blockIdx.x * HBLK + threadIdx.x;
+    const bool live = pl < t.NP;
+    const int k = find_slot(t.poff, t.ninst, live ? pl : t.NP - 1);
+    const Geo g = batch_geo(t, k);
     WorkCount wc;
-    if (pl < t.NP) {
-        const int p = (int)pl;
-        const int k = find_slot(t.poff, t.ninst, pl);
+    const int e = star_hull<false>(ids, stk, live, (int)pl, g, t.NP, pos, cell_start + __ldg(t.coff + k), perm, nbr, deg, vol,
+                                   t.inst[k].vol_scale, wc);
+    push_list(live && e == HULL_WIDER, (int)pl, t.NP, L.wide, L.counts);
+    push_list(live && e == HULL_EXACT, (int)pl, t.NP, L.exact, L.counts + 1);
+}
+
+__global__ void __launch_bounds__(WBLK) k_delaunay_wide_b(BTab t, const uint2 *__restrict__ pos,
+                                                          const int *__restrict__ cell_start,
+                                                        const int *__restrict__ perm, int *__restrict__ nbr,
+                                                          unsigned char *__restrict__ deg, float *__restrict__ vol,
+                                                          Lists L) {
+    __shared__ WideS G[WG];
+    const int cnt = L.counts[0], gid = threadIdx.x >> 3;
+    WorkCount wc;
+    for (ll j0 = (ll)blockIdx.x * WG; j0 < cnt; j0 += (ll)gridDim.x * WG) {
+        const ll j = j0 + gid;
+        const bool live = j < cnt;
+        const int p = live ? L.wide[j] : 0;
+        const int k = find_slot(t.poff, t.ninst, (ll)p);
         const Geo g = batch_geo(t, k);
-        PolyS<DBLK> P{sq, sv, (int)threadIdx.x};
-        const int err = star_of<DCAP, DBLK, false>(P, p, g, t.NP, pos, cell_start + __ldg(t.coff + k), perm, nbr, deg,
-                                                   vol, t.inst[k].vol_scale, wc);
-        if (err == ST_OVERFLOW) {
-            const int j = atomicAdd(nretry, 1);
-            PM_CHK(j >= 0 && j < t.NP, 207, j = -1)
-            if (j >= 0) retry[j] = p;
-        } else if (err) {
-            atomicOr(status, err & ~ST_OVERFLOW);
-            deg[p] = 0;
-            vol[p] = 0.0f;
-        }
+        const int e = star_wide<false>(G[gid], live, p, g, t.NP, pos, cell_start + __ldg(t.coff + k), perm, nbr, deg,
+                                       vol, t.inst[k].vol_scale, wc);
+        push_list(live && e != HULL_DONE && (threadIdx.x & 7) == 0, p, t.NP, L.exact, L.counts + 1);
     }
 }
 
@@ -599,44 +1253,52 @@ __global__ void k_export(ll np, const uint2 *__restrict__ pos, const int *__rest
 
 }  // namespace
 
+namespace {
+// The passes' lists: the sort's scratch is free once the particles are sorted.
+Lists pass_lists(const Work &w) { return Lists{w.tmp, w.key, w.nretry}; }
+
+// Grids of the list passes (grid-stride): the wide pass with 8 resident blocks
+// per SM, the first exact pass with 17, the last (rare entries) with 8.
+constexpr int kWideGrid = 8 * 152, kExactGrid = 17 * 152, kLastGrid = 8 * 152;
+
+template <bool COUNT>
+void triangulate_passes(const Geo &g, Work &w, ll np, float scale, ull *wsum, cudaStream_t st) {
+    const Lists L = pass_lists(w);
+    k_delaunay<COUNT><<<div_up(np, HBLK), HBLK, 0, st>>>(g, np, w.pos, w.cell_start, w.perm, w.nbr, w.deg, w.vol, scale,
+                                                         L, wsum);
+    k_delaunay_wide<COUNT><<<min(kWideGrid, div_up(np, WG)), WBLK, 0, st>>>(g, np, w.pos, w.cell_start, w.perm, w.nbr,
+                                                                            w.deg, w.vol, scale, L, wsum);
+    k_delaunay_retry<R1CAP, R1BLK, false, COUNT><<<min(kExactGrid, div_up(np, R1BLK)), R1BLK, 0, st>>>(
+        g, np, w.pos, w.cell_start, w.perm, w.nbr, w.deg, w.vol, scale, w.status, L.exact, L.counts + 1, wsum);
+    k_delaunay_retry<RCAP, RBLK, true, COUNT><<<min(kLastGrid, div_up(np, RBLK)), RBLK, 0, st>>>(
+        g, np, w.pos, w.cell_start, w.perm, w.nbr, w.deg, w.vol, scale, w.status, L.exact, L.counts + 1, wsum);
+}
+}  // namespace
+
 void launch_triangulate(const Geo &g, Work &w, ll np, cudaStream_t st, bool count_work) {
     if (np <= 0) return;
     double u = g.L / 4294967296.0;
     float scale = (float)(u * u / 6.0);
-    cudaMemsetAsync(w.nretry, 0, sizeof(int), st);
-    // w.tmp (caller indices before the canonical cell order) is free after the sort
-    // grid-stride passes over the retry list: the first with 17 resident
-    // blocks per SM, the last (rare entries) with 8
-    const int r1grid = 17 * 152, rgrid = 8 * 152;
-    if (count_work) {
-        k_delaunay<true><<<div_up(np, DBLK), DBLK, 0, st>>>(g, np, w.pos, w.cell_start, w.perm, w.nbr, w.deg, w.vol,
-                                                             scale, w.status, w.tmp, w.nretry, w.wsum);
-        k_delaunay_retry<R1CAP, R1BLK, false, true><<<r1grid, R1BLK, 0, st>>>(
-            g, np, w.pos, w.cell_start, w.perm, w.nbr, w.deg, w.vol, scale, w.status, w.tmp, w.nretry, w.wsum);
-        k_delaunay_retry<RCAP, RBLK, true, true><<<rgrid, RBLK, 0, st>>>(
-            g, np, w.pos, w.cell_start, w.perm, w.nbr, w.deg, w.vol, scale, w.status, w.tmp, w.nretry, w.wsum);
-    } else {
-        k_delaunay<false><<<div_up(np, DBLK), DBLK, 0, st>>>(g, np, w.pos, w.cell_start, w.perm, w.nbr, w.deg,
-                                                              w.vol, scale, w.status, w.tmp, w.nretry, nullptr);
-        k_delaunay_retry<R1CAP, R1BLK, false, false><<<r1grid, R1BLK, 0, st>>>(
-            g, np, w.pos, w.cell_start, w.perm, w.nbr, w.deg, w.vol, scale, w.status, w.tmp, w.nretry, nullptr);
-        k_delaunay_retry<RCAP, RBLK, true, false><<<rgrid, RBLK, 0, st>>>(
-            g, np, w.pos, w.cell_start, w.perm, w.nbr, w.deg, w.vol, scale, w.status, w.tmp, w.nretry, nullptr);
-    }
-    count_launches(3);
+    cudaMemsetAsync(w.nretry, 0, 2 * sizeof(int), st);
+    if (count_work)
+        triangulate_passes<true>(g, w, np, scale, w.wsum, st);
+    else
+        triangulate_passes<false>(g, w, np, scale, nullptr, st);
+    count_launches(4);
 }
 
 void launch_triangulate_batched(const BTab &t, Work &w, cudaStream_t st) {
     if (t.NP <= 0) return;
-    cudaMemsetAsync(w.nretry, 0, sizeof(int), st);
-    const int r1grid = 17 * 152, rgrid = 8 * 152;
-    k_delaunay_b<<<div_up(t.NP, DBLK), DBLK, 0, st>>>(t, w.pos, w.cell_start, w.perm, w.nbr, w.deg, w.vol, w.status,
-                                                       w.tmp, w.nretry);
-    k_delaunay_retry_b<R1CAP, R1BLK, false><<<r1grid, R1BLK, 0, st>>>(t, w.pos, w.cell_start, w.perm, w.nbr, w.deg,
-                                                                       w.vol, w.status, w.tmp, w.nretry);
-    k_delaunay_retry_b<RCAP, RBLK, true><<<rgrid, RBLK, 0, st>>>(t, w.pos, w.cell_start, w.perm, w.nbr, w.deg, w.vol,
-                                                                  w.status, w.tmp, w.nretry);
-    count_launches(3);
+    cudaMemsetAsync(w.nretry, 0, 2 * sizeof(int), st);
+    const Lists L = pass_lists(w);
+    k_delaunay_b<<<div_up(t.NP, HBLK), HBLK, 0, st>>>(t, w.pos, w.cell_start, w.perm, w.nbr, w.deg, w.vol, L);
+    k_delaunay_wide_b<<<min(kWideGrid, div_up(t.NP, WG)), WBLK, 0, st>>>(t, w.pos, w.cell_start, w.perm, w.nbr, w.deg,
+                                                                         w.vol, L);
+    k_delaunay_retry_b<R1CAP, R1BLK, false><<<min(kExactGrid, div_up(t.NP, R1BLK)), R1BLK, 0, st>>>(
+        t, w.pos, w.cell_start, w.perm, w.nbr, w.deg, w.vol, w.status, L.exact, L.counts + 1);
+    k_delaunay_retry_b<RCAP, RBLK, true><<<min(kLastGrid, div_up(t.NP, RBLK)), RBLK, 0, st>>>(
+        t, w.pos, w.cell_start, w.perm, w.nbr, w.deg, w.vol, w.status, L.exact, L.counts + 1);
+    count_launches(4);
 }
 
 void launch_volumes_1d(const Geo &g, Work &w, ll np, cudaStream_t st) {

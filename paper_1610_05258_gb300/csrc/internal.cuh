@@ -8,6 +8,7 @@
 #define PM_MAXDEG 24   // Delaunay degree stored per particle
 #define PM_MAXW 32     // capacity of the working Voronoi polygon
 #define PM_MAXF 8      // fields per call
+#define PM_POS_PAD 8    // slots past the last sorted position that a load may touch (its value is not used)
 #define PM_RCAP 12     // rings of cells searched by the triangulation
 #define PM_NET_RSCALE 64.0f  // scale of the residual input and of the output of the warm-start network
 #define PM_NET_GATE 1e-4     // delta-start relative residual above which a field gets the network's correction
@@ -145,7 +146,7 @@ struct Work {
     int *scan_tmp;      // block sums of the scan
     int *tmp;           // caller indices placed by cell, before canonical order
     int *perm;          // sorted slot -> caller index
-    uint2 *pos;         // torus coordinates, sorted
+    uint2 *pos;         // [np + PM_POS_PAD] torus coordinates, sorted
     float *vals;        // [F][np] particle fields, sorted
     unsigned *maxabs;   // [F] max |A| bit patterns
     // particle functions
@@ -173,7 +174,7 @@ struct Work {
     float *corr;           // [F][ncell] network output
     double *hres;          // [PM_MAXF] pinned host: delta-start residual per field (network gating)
     ull *wsum;             // [8] triangulation work counters (counting mode)
-    int *nretry;           // particles handed to the triangulation's retry pass
+    int *nretry;           // [2] particles handed to the triangulation's wide and exact passes
     // mesh -> particle projections (particle-sized, sorted order)
     unsigned *meshmax;     // [PM_MAXF] max |Ab| bit patterns
     float *pc;             // [F][np] right-hand side c
