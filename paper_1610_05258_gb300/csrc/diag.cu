@@ -75,10 +75,9 @@ __global__ void __launch_bounds__(kThreads) k_energy_tris(ll np, const uint2 *__
         const uint2 Xp = pos[p];
         auto rel = [&](int e, int &id, ll &rx, ll &ry) {
             id = e & 0x0fffffff;
-            const int c = (unsigned)e >> 28, ox = c / 3 - 1, oy = c % 3 - 1;
             const uint2 Xq = pos[id];
-            rx = (ll)Xq.x + (ll)ox * 4294967296LL - (ll)Xp.x;
-            ry = (ll)Xq.y + (ll)oy * 4294967296LL - (ll)Xp.y;
+            rx = (int)(Xq.x - Xp.x);  // the neighbour's image: |.| <= 2^30
+            ry = (int)(Xq.y - Xp.y);
         };
         int ida;
         ll ax, ay;

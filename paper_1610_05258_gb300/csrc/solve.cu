@@ -1191,9 +1191,9 @@ __global__ void k_star_coef(ll np, const uint2 *__restrict__ pos, const int *__r
     const uint2 Xp = pos[s];
     const float k12 = unit * unit * (1.0f / 24.0f);  // |T|/12 = area2 unit^2 / 24
     auto rel = [&](int e, ll &rx, ll &ry) {
-        const int id = e & 0x0fffffff, cd = (unsigned)e >> 28;
-        rx = (ll)pos[id].x + (ll)(cd / 3 - 1) * 4294967296LL - (ll)Xp.x;
-        ry = (ll)pos[id].y + (ll)(cd % 3 - 1) * 4294967296LL - (ll)Xp.y;
+        const uint2 Xq = pos[e & 0x0fffffff];
+        rx = (int)(Xq.x - Xp.x);  // the neighbour's image: |.| <= 2^30
+        ry = (int)(Xq.y - Xp.y);
     };
     ll ax, ay, bx, by;
     rel(nbr[(ll)(m - 1) * np + s], ax, ay);
