@@ -210,9 +210,9 @@ pm_status pm_ctx_create_mesh(pm_ctx **out, int dim, int n, double L, long long m
               alloc(c, &w.cell_start, nc + 1) && alloc(c, &w.scan_tmp, nc / 4096 + 2) && alloc(c, &w.tmp, np) &&
               alloc(c, &w.perm, np) && alloc(c, &w.pos, np + PM_POS_PAD) && alloc(c, &w.vals, np * F) &&
               alloc(c, &w.maxabs, PM_MAXF) && alloc(c, &w.deg, np) && alloc(c, &w.vol, np) &&
-              alloc(c, &w.part, (dim == 2 ? 4 : 2) * (F + 1) * nc) && alloc(c, &w.bfix, F * nc) &&
+              alloc(c, &w.part, 4 * (F + 1) * nc) && alloc(c, &w.bfix, F * nc) &&
               alloc(c, &w.psum, 2 * PM_MAXF * (ll)w.nblk_psum) &&
-              alloc(c, &w.epart, 2 * PM_MAXF * (ll)energy_blocks()) && alloc(c, &w.r, F * nc) &&
+              alloc(c, &w.epart, 2 * PM_MAXF * (ll)energy_blocks()) && alloc(c, &w.r, F * nc) && alloc(c, &w.r2, F * nc) &&
               alloc(c, &w.p, F * nc) && alloc(c, &w.q, F * nc) && alloc(c, &w.b, F * nc) &&
               alloc(c, &w.red, 6LL * PM_MAXF * 4096) && alloc(c, &w.scal, 16LL * PM_MAXF) &&
               alloc(c, &w.bar, 2) && alloc(c, &w.status, 1) && alloc(c, &w.empty, 1) && alloc(c, &w.ntri, 1) &&
@@ -223,7 +223,7 @@ pm_status pm_ctx_create_mesh(pm_ctx **out, int dim, int n, double L, long long m
     w.cfix = (ll *)w.prp;
     w.red_blocks = 4096;
     if (ok && dim == 2)
-        ok = alloc(c, &w.nbr, (ll)PM_MAXDEG * np) && alloc(c, &w.pcoef, (ll)PM_MAXDEG * np) && alloc(c, &w.r2, F * nc);
+        ok = alloc(c, &w.nbr, (ll)PM_MAXDEG * np) && alloc(c, &w.pcoef, (ll)PM_MAXDEG * np);
     if (ok && F > 1) ok = alloc(c, &w.mesh_il, (ll)g2p_width((int)F) * nc);
     if (ok && dim == 2 && n % 128 == 0 && !g.p1)  // the network start: bilinear meshes
         ok = alloc(c, &w.feat, 2 * F * nc) && alloc(c, &w.corr, F * nc);

@@ -154,7 +154,7 @@ struct Work {
     unsigned char *deg; // [np]
     float *vol;         // [np] v_mu, sorted order
     // scatter / rhs
-    float *part;        // [4 (F+1)][ncell] per-cell corner partials (FLIP)
+    float *part;        // [4 (F+1)][ncell] per-cell corner partials (FLIP); vectors of the mesh solves
     ll *bfix;           // [F][ncell] fixed-point right-hand side
     double *psum;       // [2 F][nblk] per-block particle sums (sum v A, sum v |A|)
     int nblk_psum;
@@ -182,7 +182,7 @@ struct Work {
                            // fields interleaved; the solve of F fields uses stride pcg_width(F))
     float *prp;            // [2][np][W] D^-1 r and the even iterations' search direction
     float *pp2;            // [np][W] the odd iterations' search direction
-    float *r2;             // [F][ncell] second residual buffer of the blocked Chebyshev passes (2D)
+    float *r2;             // [F][ncell] second residual buffer of the mesh solves
     ll *cfix;              // = (ll *)prp: fixed-point c before conversion
     float *pcoef;          // [PM_MAXDEG][np] particle mass matrix rows (2D)
     float *mesh_il;        // [ncell][g2p_width(F_max)] mesh fields interleaved per node (G2P)

@@ -8,16 +8,21 @@
 // sums are compensated (error-free transformations), so M x is accurate to
 // about one rounding whatever the cancellation.
 //
-// The solve is conjugate gradients in ONE persistent cooperative kernel:
-// every block owns a strided share of the nodes of all F fields, vectors stay
-// in L2, and the three reductions per iteration go through per-block FP64
-// partials that every block then sums in the same fixed order (deterministic
-// and identical on all blocks, so all blocks take the same branch). Per-node
-// products are accumulated per thread in compensated FP32 before entering
-// FP64. Before iterating, the mean mode of x is set exactly from sum_j b_j
-// (1 is an eigenvector of the circulant M with eigenvalue h^dim, and CG keeps
-// the mean of the start vector), which makes the result conservative (Eq.
-// cons) to rounding at any iteration count.
+// The mesh solves are ONE persistent cooperative kernel each (k_cg, k_cheb):
+// every block owns a strided share of the nodes of all F fields, and the
+// reductions go through per-block FP64 partials that every block then sums in
+// the same fixed order (deterministic and identical on all blocks, so all
+// blocks take the same branch). Per-node products are accumulated per thread
+// and per warp in compensated FP32 before entering FP64. Before iterating, the
+// mean mode of x is set exactly from sum_j b_j (1 is an eigenvector of the
+// circulant M with eigenvalue h^dim, and the iterations keep the mean of the
+// start vector), which makes the result conservative (Eq. cons) to rounding at
+// any iteration count.
+//
+// What bounds them is the grid barrier with its reduction on small meshes
+// (FP64 runs at 1/64 of FP32 here, so one thread per field computes the step
+// lengths, and FP64 starts at the warp totals) and the passes over the vectors
+// on large ones.
 #include <cooperative_groups.h>
 
 #include <mutex>
@@ -34,11 +39,13 @@ struct CG {
     const float *bsrc;      // float right-hand side (or null)
     const ll *bfix;         // fixed-point right-hand side (or null)
     const unsigned *maxabs; // fixed-point scale source
-    float *x, *r, *p, *q, *b;
-    float *r2;              // second residual buffer of the blocked Chebyshev passes (2D)
+    float *x;               // [F][ncell] start and result (caller's)
+    float *b, *xw, *p;      // float right-hand side, iterate, search direction
+    float *r[2], *s[2], *w[2];  // CG: residual, M p, M r, alternating between passes
+                                // Chebyshev: r and d (in s)
     double *red;            // [6 * PM_MAXF][grid]
     double *scal;           // [F][16]
-    unsigned *bar;          // [2] barrier count, generation
+    unsigned *bar;          // [2] barrier count
     int *status;
     double rtol;
     int max_iter;
@@ -50,330 +57,623 @@ struct CG {
 enum { S_ITERS = 0, S_INIT = 1, S_RESID = 2, S_SUMMESH = 3, S_SUMPART = 4, S_SUMABS = 5 };
 
 // Grid-wide barrier with a bounded wait (about a second); on timeout the
-// status word gets ST_TIMEOUT and false is returned.
-__device__ bool grid_sync(unsigned *bar, int *status) {
+// status word gets ST_TIMEOUT and false is returned. The count only grows:
+// barrier k of a launch opens at k times the number of blocks. `passed` counts
+// the barriers of this launch.
+__device__ bool grid_sync(unsigned *bar, int *status, unsigned &passed) {
+    ++passed;
+    if (gridDim.x == 1) {
+        __syncthreads();
+        return true;
+    }
     __shared__ int ok;
     __syncthreads();
     if (threadIdx.x == 0) {
         ok = 1;
-        volatile unsigned *gen = bar + 1;
-        unsigned g0 = *gen;
-        __threadfence();
-        if (atomicAdd(bar, 1u) == gridDim.x - 1) {
-            bar[0] = 0;
-            __threadfence();
-            atomicAdd(bar + 1, 1u);
-        } else {
-            long long spins = 0;
-            while (*gen == g0) {
-                __nanosleep(64);
-                if (++spins > (1LL << 24)) {
-                    atomicOr(status, ST_TIMEOUT);
-                    ok = 0;
-                    break;
-                }
+        const unsigned target = passed * gridDim.x;
+        unsigned seen;
+        asm volatile("atom.add.release.gpu.global.u32 %0, [%1], 1;" : "=r"(seen) : "l"(bar) : "memory");
+        int spins = 0;
+        for (;;) {
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(bar) : "memory");
+            if ((int)(seen - target) >= 0) break;
+            if (++spins > 64) __nanosleep(64);
+            if (spins > (1 << 22)) {
+                atomicOr(status, ST_TIMEOUT);
+                ok = 0;
+                break;
             }
         }
-        __threadfence();
     }
     __syncthreads();
     return ok != 0;
 }
 
-// Block reduction of one double per field into red[slot*F + f][block].
-__device__ void block_partial(double v[PM_MAXF], int F, double *red, int slot) {
-    __shared__ double sh[PM_MAXF][32];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    for (int f = 0; f < F; ++f) {
-        double s = v[f];
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if (lane == 0) sh[f][wid] = s;
-    }
-    __syncthreads();
-    if (threadIdx.x < F) {
-        double s = 0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += sh[threadIdx.x][w];
-        PM_CHK((ll)(slot * F + threadIdx.x + 1) * gridDim.x <= 6LL * PM_MAXF * 1024, 401, s = 0)
-        red[(ll)(slot * F + threadIdx.x) * gridDim.x + blockIdx.x] = s;
-    }
-    __syncthreads();
+// Accumulators summed with another one, and over the warp (lane 0), in the same
+// compensated form.
+__device__ __forceinline__ void join(Dot2 &a, const Dot2 &b) {
+#if defined(PM_FP64_SUMS)
+    a.hi += b.hi;
+#else
+    a.add(b.hi);
+#endif
+    a.lo += b.lo;
 }
-
-// Sum of the partials of (slot, f) over all blocks, same order on every block.
-__device__ void grid_total(const double *red, int F, int slot, double out[PM_MAXF]) {
-    __shared__ double tot[PM_MAXF];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    if (wid < F) {
-        const double *src = red + (ll)(slot * F + wid) * gridDim.x;
-        double s = 0;
-        for (unsigned i = lane; i < gridDim.x; i += 32) s += src[i];
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if (lane == 0) tot[wid] = s;
+__device__ __forceinline__ Dot2 warp_total(Dot2 a) {
+    for (int o = 16; o > 0; o >>= 1) {
+        Dot2 b;
+        b.hi = __shfl_down_sync(0xffffffffu, a.hi, o);
+        b.lo = __shfl_down_sync(0xffffffffu, a.lo, o);
+        join(a, b);
     }
-    __syncthreads();
-    for (int f = 0; f < F; ++f) out[f] = tot[f];
-    __syncthreads();
+    return a;
 }
+__device__ __forceinline__ double total(const Dot2 &a) { return (double)a.hi + (double)a.lo; }
 
-// Totals of the per-block particle sums (sum v A, sum v |A|) of every field:
-// warp f sums field f's partials (lanes stride, fixed shuffle tree), so the
-// result is the same on every run. Called by all threads of one block.
-__device__ void particle_sums(const double *psum, int nblk, int F, double s1[PM_MAXF], double s2[PM_MAXF]) {
-    __shared__ double tot[2 * PM_MAXF];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    for (int k = wid; k < 2 * F; k += (int)(blockDim.x >> 5)) {
-        const double *src = psum + (ll)k * nblk;
-        double s = 0;
-        for (int i = lane; i < nblk; i += 32) s += src[i];
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if (lane == 0) tot[k] = s;
-    }
+// A sum over the grid goes through red[(slot + kind) * F + f][block]: every
+// thread puts its accumulator (the warp's total goes to shared memory), the block
+// flushes, and after a grid barrier every block sums the partials in the same
+// order. FP64 sums (flush_sums, grid_sum) from the warp totals on where the
+// total itself is used or reported; the inner products of an iteration, which
+// only set FP32 step lengths and the stop, stay compensated FP32 pairs
+// (flush_pairs, grid_pairs): an FP64 instruction holds its pipe for 16 cycles a
+// warp, and with the FP64 sums and divisions an iteration of one block took
+// 7500 cycles, of 64 blocks 14000; now 5200 and 10000, 2250 of them the barrier.
+struct BlockSums {
+    Dot2 v[3][PM_MAXF][8];
+};
+__device__ __forceinline__ void put_sum(BlockSums &B, int kind, int f, const Dot2 &a) {
+    const Dot2 t = warp_total(a);
+    if ((threadIdx.x & 31) == 0) B.v[kind][f][threadIdx.x >> 5] = t;
+}
+__device__ __forceinline__ void flush_sums(const BlockSums &B, int kinds, int F, double *red, int slot) {
     __syncthreads();
-    for (int f = 0; f < F; ++f) {
-        s1[f] = tot[2 * f];
-        s2[f] = tot[2 * f + 1];
+    const int t = threadIdx.x;
+    if (t < kinds * F) {
+        const Dot2 *v = B.v[t / F][t % F];
+        red[(ll)(slot * F + t) * gridDim.x + blockIdx.x] = ((total(v[0]) + total(v[1])) + (total(v[2]) + total(v[3]))) +
+                                                           ((total(v[4]) + total(v[5])) + (total(v[6]) + total(v[7])));
     }
 }
+// Total of (slot, f) over all blocks, by one warp.
+__device__ __forceinline__ double grid_sum(const double *red, int F, int slot, int f) {
+    const int lane = threadIdx.x & 31;
+    const double *src = red + (ll)(slot * F + f) * gridDim.x;
+    double s = 0;
+#pragma unroll 4
+    for (unsigned i = lane; i < gridDim.x; i += 32) s += __ldcg(src + i);
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    return s;
+}
+#if defined(PM_FP64_SUMS)
+__device__ __forceinline__ double pack(const Dot2 &a) { return total(a); }
+__device__ __forceinline__ Dot2 unpack(double v) {
+    Dot2 a;
+    a.hi = v;
+    return a;
+}
+#else
+__device__ __forceinline__ double pack(const Dot2 &a) {
+    return __hiloint2double(__float_as_int(a.hi), __float_as_int(a.lo));  // bits only
+}
+__device__ __forceinline__ Dot2 unpack(double v) {
+    Dot2 a;
+    a.hi = __int_as_float(__double2hiint(v));
+    a.lo = __int_as_float(__double2loint(v));
+    return a;
+}
+#endif
+__device__ __forceinline__ void flush_pairs(const BlockSums &B, int kinds, int F, double *red, int slot) {
+    __syncthreads();
+    const int t = threadIdx.x;
+    if (t < kinds * F) {
+        const Dot2 *v = B.v[t / F][t % F];
+        Dot2 a = v[0], b = v[4];
+#pragma unroll
+        for (int w = 1; w < 4; ++w) {
+            join(a, v[w]);
+            join(b, v[w + 4]);
+        }
+        join(a, b);
+        red[(ll)(slot * F + t) * gridDim.x + blockIdx.x] = pack(a);
+    }
+}
+// Totals of field f in K consecutive slots, by one warp; lane 0 has them.
+template <int K>
+__device__ __forceinline__ void grid_pairs(const double *red, int F, int slot, int f, double (&out)[K]) {
+    const int lane = threadIdx.x & 31;
+    Dot2 a[K];
+#pragma unroll 2
+    for (unsigned i = lane; i < gridDim.x; i += 32)
+#pragma unroll
+        for (int k = 0; k < K; ++k) join(a[k], unpack(__ldcg(red + (ll)((slot + k) * F + f) * gridDim.x + i)));
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            Dot2 b;
+            b.hi = __shfl_down_sync(0xffffffffu, a[k].hi, o);
+            b.lo = __shfl_down_sync(0xffffffffu, a[k].lo, o);
+            join(a[k], b);
+        }
+#pragma unroll
+    for (int k = 0; k < K; ++k) out[k] = total(a[k]);
+}
 
-template <int DIM, int P1>
-__global__ void __launch_bounds__(256) k_cg(CG a) {
-    // Reduction slot groups alternate (3 (k & 1) for the k-th reduction), so a
-    // block that runs ahead never overwrites partials another block is summing.
-    int rk = 0, rg = 0;
-    const Geo g = a.g;
-    const int F = a.F, n = g.n;
+// a / b to a few units of FP64 rounding, b > 0: the FP32 reciprocal refined by one
+// Newton step (relative error e -> e^2, 2^-46) and one on the quotient. Seven
+// dependent FP64 operations. Outside the range of the seed the plain quotient.
+__device__ __forceinline__ double quot(double a, double b) {
+    if (!(b > 1e-30 && b < 1e30)) return a / b;
+    double r = (double)(1.0f / (float)b);
+    r = fma(fma(-b, r, 1.0), r, r);
+    const double q = a * r;
+    return fma(fma(-b, q, a), r, q);
+}
+
+// Totals of the per-block particle sums of one row (sum v A or sum v |A|) by
+// the whole block, the same order on every run; thread 0 has it.
+__device__ __forceinline__ double particle_sum(const double *psum, int nblk, int row) {
+    __shared__ double sh[8];
+    const double *src = psum + (ll)row * nblk;
+    double s = 0;
+#pragma unroll 4
+    for (int i = threadIdx.x; i < nblk; i += 256) s += src[i];
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = s;
+    __syncthreads();
+    s = ((sh[0] + sh[1]) + (sh[2] + sh[3])) + ((sh[4] + sh[5]) + (sh[6] + sh[7]));
+    __syncthreads();
+    return s;
+}
+
+struct Q4 {
+    float v[4];
+};
+__device__ __forceinline__ Q4 ld4(const float *p) {
+    const float4 t = *(const float4 *)p;
+    return Q4{{t.x, t.y, t.z, t.w}};
+}
+__device__ __forceinline__ void st4(float *p, const Q4 &q) { *(float4 *)p = make_float4(q.v[0], q.v[1], q.v[2], q.v[3]); }
+
+// VEC consecutive nodes of a row (VEC = 4: 16-byte accesses, n % 4 == 0).
+template <int VEC>
+__device__ __forceinline__ void ldn(const float *p, float (&v)[VEC]) {
+    if (VEC == 4) {
+        const Q4 q = ld4(p);
+#pragma unroll
+        for (int j = 0; j < VEC; ++j) v[j] = q.v[j & 3];
+    } else {
+        v[0] = *p;
+    }
+}
+template <int VEC>
+__device__ __forceinline__ void stn(float *p, const float (&v)[VEC]) {
+    if (VEC == 4) *(float4 *)p = make_float4(v[0], v[1 % VEC], v[2 % VEC], v[3 % VEC]);
+    else *p = v[0];
+}
+
+// Compensated stencil sums (hi, lo) of the VEC nodes starting at flat index i0
+// (unscaled: the caller multiplies by h/6, h^2/36 or h^2/12) of the vector that
+// val gives, val.get(index, out) for VEC nodes from an aligned index and
+// val.one(index) for one; ctr: its values there. The additions are those of
+// stencil<>, in the same order.
+template <int DIM, int P1, int VEC, class Val>
+__device__ __forceinline__ void stencil_of(const Val &val, int n, int i0, float (&hi)[VEC], float (&lo)[VEC],
+                                           float (&ctr)[VEC]) {
+    if (DIM == 1) {
+        val.get(i0, ctr);
+        const float l = val.one(i0 == 0 ? n - 1 : i0 - 1), r = val.one(i0 + VEC == n ? 0 : i0 + VEC);
+#pragma unroll
+        for (int j = 0; j < VEC; ++j) {
+            Dot2 acc;
+            acc.add(4.0f * ctr[j]);
+            acc.add(j == 0 ? l : ctr[j == 0 ? 0 : j - 1]);
+            acc.add(j == VEC - 1 ? r : ctr[j == VEC - 1 ? 0 : j + 1]);
+            hi[j] = acc.hi;
+            lo[j] = acc.lo;
+        }
+        return;
+    }
+    const int iy = (int)((unsigned)i0 / (unsigned)n), ix = i0 - iy * n;
+    const int r0 = (iy == 0 ? n - 1 : iy - 1) * n, r1 = iy * n, r2 = (iy + 1 == n ? 0 : iy + 1) * n;
+    const int xl = ix == 0 ? n - 1 : ix - 1, xr = ix + VEC == n ? 0 : ix + VEC;
+    float a[VEC], c[VEC];
+    val.get(r0 + ix, a);
+    val.get(r1 + ix, ctr);
+    val.get(r2 + ix, c);
+    const float a_l = val.one(r0 + xl), a_r = P1 ? 0.0f : val.one(r0 + xr), b_l = val.one(r1 + xl),
+                b_r = val.one(r1 + xr), c_l = P1 ? 0.0f : val.one(r2 + xl), c_r = val.one(r2 + xr);
+#pragma unroll
+    for (int j = 0; j < VEC; ++j) {
+        const int jm = j == 0 ? 0 : j - 1, jp = j == VEC - 1 ? 0 : j + 1;
+        const float am = j == 0 ? a_l : a[jm], ap = j == VEC - 1 ? a_r : a[jp];
+        const float bm = j == 0 ? b_l : ctr[jm], bp = j == VEC - 1 ? b_r : ctr[jp];
+        const float cm = j == 0 ? c_l : c[jm], cp = j == VEC - 1 ? c_r : c[jp];
+        Dot2 acc;
+        if (P1) {
+            acc.add(6.0f * ctr[j]);
+            acc.add(bm);
+            acc.add(bp);
+            acc.add(a[j]);
+            acc.add(c[j]);
+            acc.add(am);
+            acc.add(cp);
+        } else {
+            acc.add(16.0f * ctr[j]);
+            acc.add(4.0f * bm);
+            acc.add(4.0f * bp);
+            acc.add(4.0f * a[j]);
+            acc.add(4.0f * c[j]);
+            acc.add(am);
+            acc.add(ap);
+            acc.add(cm);
+            acc.add(cp);
+        }
+        hi[j] = acc.hi;
+        lo[j] = acc.lo;
+    }
+}
+
+// A stored vector.
+template <int VEC>
+struct Plain {
+    const float *v;
+    __device__ __forceinline__ void get(int o, float (&q)[VEC]) const { ldn<VEC>(v + o, q); }
+    __device__ __forceinline__ float one(int o) const { return v[o]; }
+};
+// The scaled start with its exact mean, S x + sh (sh alone without a start).
+template <int VEC>
+struct Start {
+    const float *x;
+    float S, sh;
+    __device__ __forceinline__ void get(int o, float (&q)[VEC]) const {
+#pragma unroll
+        for (int j = 0; j < VEC; ++j) q[j] = 0.0f;
+        if (x) ldn<VEC>(x + o, q);
+#pragma unroll
+        for (int j = 0; j < VEC; ++j) q[j] = fmaf(q[j], S, sh);
+    }
+    __device__ __forceinline__ float one(int o) const { return fmaf(x ? x[o] : 0.0f, S, sh); }
+};
+// The next residual of a CG pass, r - alpha (w + beta s).
+template <int VEC>
+struct NextR {
+    const float *r, *w, *s;
+    float al, be;
+    bool first;  // no s yet: it is w
+    __device__ __forceinline__ void get(int o, float (&q)[VEC]) const {
+        float t[VEC], u[VEC];
+        ldn<VEC>(r + o, q);
+        ldn<VEC>(w + o, t);
+        if (!first) {
+            ldn<VEC>(s + o, u);
+#pragma unroll
+            for (int j = 0; j < VEC; ++j) t[j] = fmaf(be, u[j], t[j]);
+        }
+#pragma unroll
+        for (int j = 0; j < VEC; ++j) q[j] = fmaf(-al, t[j], q[j]);
+    }
+    __device__ __forceinline__ float one(int o) const {
+        float t = w[o];
+        if (!first) t = fmaf(be, s[o], t);
+        return fmaf(-al, t, r[o]);
+    }
+};
+
+// Per-field state of a mesh solve, the same on every block.
+struct SolveState {
+    double bb[PM_MAXF], rr[PM_MAXF], rr0[PM_MAXF], pMp[PM_MAXF], sumb[PM_MAXF], tr[PM_MAXF], sx[PM_MAXF];
+    float S[PM_MAXF], sh[PM_MAXF], al[PM_MAXF], be[PM_MAXF];
+    int act[PM_MAXF], first[PM_MAXF], its[PM_MAXF], steps[PM_MAXF];
+};
+
+// Right-hand side as float, its sum and sum of |b|, sum of the start; the field
+// scale S (a power of two that brings the mean |b| to order one: exact scaling,
+// FP32 inner products of any field stay in range) and the shift that sets the
+// mean of S x + sh to the exact one. Ends with a block barrier.
+template <int DIM, int VEC>
+__device__ __forceinline__ bool solve_begin(const CG &a, SolveState &V, BlockSums &B, unsigned &passed) {
+    const Geo &g = a.g;
+    const int F = a.F;
+    const unsigned nv = (unsigned)(g.ncell / VEC);
     const ll nn = g.ncell;
-    const ll tid = (ll)blockIdx.x * blockDim.x + threadIdx.x, nth = (ll)gridDim.x * blockDim.x;
+    const unsigned tid = blockIdx.x * blockDim.x + threadIdx.x, nth = gridDim.x * blockDim.x;
+    const float hd32 = DIM == 1 ? g.h : g.h * g.h;
+    const double hd = DIM == 1 ? (double)g.h : (double)g.h * g.h;
+    for (int f = 0; f < F; ++f) {
+        const ll fo = (ll)f * nn;
+        // the fixed-point scale 2^-E in two factors, so that neither overflows (E is
+        // at most 120 + 149) and only the second product can round, as in ldexpf
+        const int E = a.bfix ? fixed_point_exp(__uint_as_float(a.maxabs[f]), hd32) : 0;
+        const float s1 = ldexpf(1.0f, -(E / 2)), s2 = ldexpf(1.0f, E / 2 - E);
+        Dot2 sb, sa, sx;
+        for (unsigned i = tid; i < nv; i += nth) {
+            const ll o = fo + (ll)i * VEC;
+            float bv[VEC], xv[VEC];
+            if (a.bfix) {
+                ll q[VEC];
+                if (VEC == 4) {
+                    const longlong2 u = *(const longlong2 *)(a.bfix + o), v = *(const longlong2 *)(a.bfix + o + 2);
+                    q[0] = u.x, q[1 % VEC] = u.y, q[2 % VEC] = v.x, q[3 % VEC] = v.y;
+                } else {
+                    q[0] = a.bfix[o];
+                }
+#pragma unroll
+                for (int j = 0; j < VEC; ++j) bv[j] = (float)q[j] * s1 * s2;
+            } else {
+                ldn<VEC>(a.bsrc + o, bv);
+            }
+            stn<VEC>(a.b + o, bv);
+            if (a.has_start) ldn<VEC>(a.x + o, xv);
+#pragma unroll
+            for (int j = 0; j < VEC; ++j) {
+                sb.add(bv[j]);
+                sa.add(fabsf(bv[j]));
+                if (a.has_start) sx.add(xv[j]);
+            }
+        }
+        put_sum(B, 0, f, sb);
+        put_sum(B, 1, f, sa);
+        put_sum(B, 2, f, sx);
+    }
+    flush_sums(B, 3, F, a.red, 0);
+    if (!grid_sync(a.bar, a.status, passed)) return false;
+    const int f = threadIdx.x >> 5;
+    if (f < F) {
+        const double sumb = grid_sum(a.red, F, 0, f), suma = grid_sum(a.red, F, 1, f), sumx = grid_sum(a.red, F, 2, f);
+        if ((threadIdx.x & 31) == 0) {
+            const float S = solve_scale(suma / (double)nn);
+            V.S[f] = S;
+            V.sumb[f] = sumb;
+            V.sh[f] = (float)((double)S * (sumb / ((double)nn * hd) - (a.has_start ? sumx / (double)nn : 0.0)));
+            V.its[f] = 0;
+        }
+    }
+    __syncthreads();
+    return true;
+}
+
+// True residual r = S b - M xw into r (and, if out, the unscaled result into
+// out), sums of r^2 and xw; with START, xw = S x + sh is formed and stored and
+// the second sum is that of (S b)^2. Ends before the reduction's barrier.
+template <int DIM, int P1, int VEC, bool START>
+__device__ __forceinline__ void residual_pass(const CG &a, SolveState &V, BlockSums &B, float *r, float *out, int slot) {
+    const Geo &g = a.g;
+    const int F = a.F, n = g.n;
+    const unsigned nv = (unsigned)(g.ncell / VEC);
+    const ll nn = g.ncell;
+    const unsigned tid = blockIdx.x * blockDim.x + threadIdx.x, nth = gridDim.x * blockDim.x;
+    const float c = DIM == 1 ? g.h / 6.0f : (P1 ? g.h * g.h / 12.0f : g.h * g.h / 36.0f);
+    for (int f = 0; f < F; ++f) {
+        const ll fo = (ll)f * nn;
+        const float S = V.S[f], inv = 1.0f / S;  // powers of two: exact
+        const Start<VEC> st{a.has_start ? a.x + fo : nullptr, S, V.sh[f]};
+        const Plain<VEC> xw{a.xw + fo};
+        Dot2 s, t;
+        for (unsigned i = tid; i < nv; i += nth) {
+            const int i0 = (int)(i * VEC);
+            float hi[VEC], lo[VEC], ct[VEC], bv[VEC], rv[VEC];
+            if (START) stencil_of<DIM, P1, VEC>(st, n, i0, hi, lo, ct);
+            else stencil_of<DIM, P1, VEC>(xw, n, i0, hi, lo, ct);
+            ldn<VEC>(a.b + fo + i0, bv);
+#pragma unroll
+            for (int j = 0; j < VEC; ++j) {
+                bv[j] *= S;
+                rv[j] = fmaf(-c, hi[j], bv[j]) - c * lo[j];
+                s.fma_acc(rv[j], rv[j]);
+                if (START) t.fma_acc(bv[j], bv[j]);
+                else t.add(ct[j]);
+            }
+            stn<VEC>(r + fo + i0, rv);
+            if (START) stn<VEC>(a.xw + fo + i0, ct);
+            if (out) {
+#pragma unroll
+                for (int j = 0; j < VEC; ++j) ct[j] *= inv;
+                stn<VEC>(out + fo + i0, ct);
+            }
+        }
+        put_sum(B, 0, f, s);
+        put_sum(B, 1, f, t);
+    }
+    flush_sums(B, 2, F, a.red, slot);
+}
+
+// The report of a solve whose closing residual pass is summed (V.tr, V.sx).
+__device__ __forceinline__ void solve_report(const CG &a, const SolveState &V, double hd) {
+    // the particle sums, a row to a block from the last block down
+    if (a.psum)
+        for (int row = gridDim.x - 1 - blockIdx.x; row < 2 * a.F; row += gridDim.x) {
+            const double ps = particle_sum(a.psum, a.nblk_psum, row);
+            if (threadIdx.x == 0) a.scal[(row >> 1) * 16 + (row & 1 ? S_SUMABS : S_SUMPART)] = ps;
+        }
+    if (blockIdx.x != 0) return;
+    const int f = threadIdx.x >> 1, k = threadIdx.x & 1;  // k: residual at exit, at the start
+    if (f >= a.F) return;
+    const double res = V.bb[f] > 0.0 ? sqrt((k ? V.rr0[f] : V.tr[f]) / V.bb[f]) : 0.0;
+    if (k) {
+        a.scal[f * 16 + S_INIT] = res;
+        return;
+    }
+    a.scal[f * 16 + S_ITERS] = V.its[f];
+    a.scal[f * 16 + S_RESID] = res;
+    a.scal[f * 16 + S_SUMMESH] = V.sx[f] * hd / (double)V.S[f];
+    if (!a.psum) {
+        a.scal[f * 16 + S_SUMPART] = V.sumb[f];
+        a.scal[f * 16 + S_SUMABS] = 0.0;
+    }
+    if (res > a.rtol) atomicOr(a.status, ST_NOTCONV);
+}
+
+// Conjugate gradients with one pass and one grid barrier per iteration. With
+// w = M r at hand, (r, r) and (w, r) give both step lengths (Chronopoulos and
+// Gear): beta = rr / rr_old, alpha = rr / pMp, pMp = (w, r) - beta^2 pMp_old, and
+//   s = w + beta s (= M p),  p = r + beta p,  x += alpha p,  r -= alpha s,  w = M r
+// is one pass: each node forms the next r at its stencil's nodes from the old r,
+// w and s (the same FMAs everywhere, so every copy has the same bits), and r, s
+// and w alternate between two buffers. The separate passes for M p, x and r,
+// and p took three barriers. Whole solves, before and now: 128 nodes in 1D (7
+// iterations, one block) 105 -> 42 us; 256^2 (13) 232 -> 97 us; 512^2, 3 fields
+// (19) 669 -> 284 us; 2048^2, 4 fields (19) 4046 -> 2766 us, 40 bytes per node and
+// iteration at 4.6 TB/s.
+// Consecutive reductions use slot groups {0, 1, 2}, {3, 4}, {5} and then
+// alternate {0, 1} and {2, 3}, so that a block that runs ahead never overwrites
+// partials another block is summing.
+template <int DIM, int P1, int VEC>
+__global__ void __launch_bounds__(256) k_cg(CG a) {
+    __shared__ SolveState V;
+    __shared__ BlockSums B;
+    unsigned passed = 0;
+    const Geo &g = a.g;
+    const int F = a.F, n = g.n;
+    const unsigned nv = (unsigned)(g.ncell / VEC);
+    const ll nn = g.ncell;
+    const unsigned tid = blockIdx.x * blockDim.x + threadIdx.x, nth = gridDim.x * blockDim.x;
     const float c = DIM == 1 ? g.h / 6.0f : (P1 ? g.h * g.h / 12.0f : g.h * g.h / 36.0f);
     const double hd = DIM == 1 ? (double)g.h : (double)g.h * g.h;
-    double v[PM_MAXF], w[PM_MAXF];
-    double bb[PM_MAXF], rr[PM_MAXF], alpha[PM_MAXF], beta[PM_MAXF];
-    bool act[PM_MAXF];
-    int it_f[PM_MAXF];
-    // --- phase 0: right-hand side as float, its sum and sum of |b|, sum of start
-    for (int f = 0; f < F; ++f) {
-        Dot2 sb, sa, sx;
-        const float hd32 = DIM == 1 ? g.h : g.h * g.h;
-        const int E = a.bfix ? fixed_point_exp(__uint_as_float(a.maxabs[f]), hd32) : 0;
-        for (ll i = tid; i < nn; i += nth) {
-            float bv = a.bfix ? ldexpf((float)a.bfix[(ll)f * nn + i], -E) : a.bsrc[(ll)f * nn + i];
-            a.b[(ll)f * nn + i] = bv;
-            sb.add(bv);
-            sa.add(fabsf(bv));
-            if (a.has_start) sx.add(a.x[(ll)f * nn + i]);
-        }
-        v[f] = (double)sb.hi + (double)sb.lo;
-        w[f] = (double)sa.hi + (double)sa.lo;
-        alpha[f] = (double)sx.hi + (double)sx.lo;
-    }
-    rg = 3 * (rk++ & 1);
-    block_partial(v, F, a.red, rg);
-    block_partial(w, F, a.red, rg + 1);
-    block_partial(alpha, F, a.red, rg + 2);
-    if (!grid_sync(a.bar, a.status)) return;
-    double sumb[PM_MAXF], sumx[PM_MAXF], suma[PM_MAXF];
-    grid_total(a.red, F, rg, sumb);
-    grid_total(a.red, F, rg + 1, suma);
-    grid_total(a.red, F, rg + 2, sumx);
-    // The system is solved for S b with S a power of two that brings the mean
-    // |b| to order one (exact scaling: FP32 inner products of any field stay
-    // in range); x is scaled by S on entry and by 1/S on exit. Then the exact
-    // mean mode: mean(x) = sum b / (nn h^dim), and the norm of S b.
-    float S[PM_MAXF];
-    for (int f = 0; f < F; ++f) {
-        S[f] = solve_scale(suma[f] / (double)nn);
-        const double shift = (double)S[f] * (sumb[f] / ((double)nn * hd) - (a.has_start ? sumx[f] / (double)nn : 0.0));
-        const float sh = (float)shift;
-        Dot2 s2;
-        for (ll i = tid; i < nn; i += nth) {
-            const float xv = a.has_start ? a.x[(ll)f * nn + i] * S[f] : 0.0f;
-            a.x[(ll)f * nn + i] = xv + sh;
-            const float bv = a.b[(ll)f * nn + i] * S[f];
-            a.b[(ll)f * nn + i] = bv;
-            s2.fma_acc(bv, bv);
-        }
-        w[f] = (double)s2.hi + (double)s2.lo;
-    }
-    rg = 3 * (rk++ & 1);
-    block_partial(w, F, a.red, rg);
-    if (!grid_sync(a.bar, a.status)) return;
-    grid_total(a.red, F, rg, bb);
-    // --- r = b - M x, p = r
-    for (int f = 0; f < F; ++f) {
-        Dot2 s;
-        const float *xf = a.x + (ll)f * nn;
-        for (ll i = tid; i < nn; i += nth) {
-            float hi, lo;
-            stencil<DIM, P1>(xf, n, i, hi, lo);
-            float rv = fmaf(-c, hi, a.b[(ll)f * nn + i]) - c * lo;
-            a.r[(ll)f * nn + i] = rv;
-            a.p[(ll)f * nn + i] = rv;
-            s.fma_acc(rv, rv);
-        }
-        v[f] = (double)s.hi + (double)s.lo;
-    }
-    rg = 3 * (rk++ & 1);
-    block_partial(v, F, a.red, rg);
-    if (!grid_sync(a.bar, a.status)) return;
-    grid_total(a.red, F, rg, rr);
     const double tol2 = a.rtol * a.rtol;
-    for (int f = 0; f < F; ++f) {
-        act[f] = rr[f] > tol2 * bb[f] && bb[f] > 0.0;
-        it_f[f] = 0;
-        if (blockIdx.x == 0 && threadIdx.x == 0)
-            a.scal[f * 16 + S_INIT] = bb[f] > 0.0 ? sqrt(rr[f] / bb[f]) : 0.0;
+    const int wf = threadIdx.x >> 5;  // warp f sums field f's partials, its lane 0 keeps the state
+    const bool lane0 = (threadIdx.x & 31) == 0;
+    if (!solve_begin<DIM, VEC>(a, V, B, passed)) return;
+    residual_pass<DIM, P1, VEC, true>(a, V, B, a.r[0], nullptr, 3);
+    if (!grid_sync(a.bar, a.status, passed)) return;
+    if (wf < F) {
+        const double rr = grid_sum(a.red, F, 3, wf), bb = grid_sum(a.red, F, 4, wf);
+        if (lane0) {
+            V.rr[wf] = V.rr0[wf] = rr;
+            V.bb[wf] = bb;
+            V.act[wf] = V.first[wf] = bb > 0.0 && rr > tol2 * bb;
+        }
     }
-    int restarts = 0;
-    for (int it = 0; it < a.max_iter; ++it) {
+    __syncthreads();
+    int cur = 0, it = 0, slot = 5;
+    for (int restarts = 0;; ++restarts) {
         bool any = false;
-        for (int f = 0; f < F; ++f) any |= act[f];
-        if (!any) {
-            // recursive residuals converged: check the true residual once
+        for (int f = 0; f < F; ++f) any |= V.act[f] != 0;
+        if (any && it < a.max_iter) {
+            // w = M r, (w, r) of the fields that (re)start
             for (int f = 0; f < F; ++f) {
-                Dot2 s;
-                const float *xf = a.x + (ll)f * nn;
-                for (ll i = tid; i < nn; i += nth) {
-                    float hi, lo;
-                    stencil<DIM, P1>(xf, n, i, hi, lo);
-                    float rv = fmaf(-c, hi, a.b[(ll)f * nn + i]) - c * lo;
-                    s.fma_acc(rv, rv);
+                if (!V.act[f]) continue;
+                const ll fo = (ll)f * nn;
+                const Plain<VEC> rp{a.r[cur] + fo};
+                Dot2 d;
+                for (unsigned i = tid; i < nv; i += nth) {
+                    float hi[VEC], lo[VEC], ct[VEC];
+                    stencil_of<DIM, P1, VEC>(rp, n, (int)(i * VEC), hi, lo, ct);
+#pragma unroll
+                    for (int j = 0; j < VEC; ++j) {
+                        hi[j] = fmaf(c, hi[j], c * lo[j]);
+                        d.fma_acc(hi[j], ct[j]);
+                    }
+                    stn<VEC>(a.w[cur] + fo + i * VEC, hi);
                 }
-                v[f] = (double)s.hi + (double)s.lo;
+                put_sum(B, 0, f, d);
             }
-            rg = 3 * (rk++ & 1);
-            block_partial(v, F, a.red, rg);
-            if (!grid_sync(a.bar, a.status)) return;
-            double tr[PM_MAXF];
-            grid_total(a.red, F, rg, tr);
-            bool again = false;
-            for (int f = 0; f < F; ++f)
-                if (bb[f] > 0.0 && tr[f] > tol2 * bb[f]) { act[f] = true; again = true; }
-            if (!again || restarts >= 3) break;
-            ++restarts;
-            // restart the drifted fields from their true residual
-            for (int f = 0; f < F; ++f) {
-                if (!act[f]) continue;
-                Dot2 s;
-                const float *xf = a.x + (ll)f * nn;
-                for (ll i = tid; i < nn; i += nth) {
-                    float hi, lo;
-                    stencil<DIM, P1>(xf, n, i, hi, lo);
-                    float rv = fmaf(-c, hi, a.b[(ll)f * nn + i]) - c * lo;
-                    a.r[(ll)f * nn + i] = rv;
-                    a.p[(ll)f * nn + i] = rv;
-                    s.fma_acc(rv, rv);
+            flush_pairs(B, 1, F, a.red, slot);
+            if (!grid_sync(a.bar, a.status, passed)) return;
+            if (wf < F && V.act[wf]) {
+                double t[1];
+                grid_pairs<1>(a.red, F, slot, wf, t);
+                if (lane0) {
+                    const double wr = t[0];
+                    V.pMp[wf] = wr;
+                    V.al[wf] = (float)quot(V.rr[wf], wr);
+                    V.be[wf] = 0.0f;
+                    V.first[wf] = 1;
+                    if (!(wr > 0.0)) V.act[wf] = 0;  // r below the range of its products
                 }
-                v[f] = (double)s.hi + (double)s.lo;
             }
-            rg = 3 * (rk++ & 1);
-            block_partial(v, F, a.red, rg);
-            if (!grid_sync(a.bar, a.status)) return;
-            grid_total(a.red, F, rg, w);
-            for (int f = 0; f < F; ++f)
-                if (act[f]) rr[f] = w[f];
-        }
-        // q = M p, (p, q)
-        for (int f = 0; f < F; ++f) {
-            v[f] = 0.0;
-            if (!act[f]) continue;
-            Dot2 s;
-            const float *pf = a.p + (ll)f * nn;
-            for (ll i = tid; i < nn; i += nth) {
-                float hi, lo;
-                stencil<DIM, P1>(pf, n, i, hi, lo);
-                float qv = fmaf(c, hi, c * lo);
-                a.q[(ll)f * nn + i] = qv;
-                s.fma_acc(pf[i], qv);
+            __syncthreads();
+            slot = slot == 5 ? 0 : slot ^ 2;
+            while (any && it < a.max_iter) {
+                const int nxt = cur ^ 1;
+                for (int f = 0; f < F; ++f) {
+                    if (!V.act[f]) continue;
+                    const ll fo = (ll)f * nn;
+                    const float al = V.al[f], be = V.be[f];
+                    const bool first = V.first[f] != 0;
+                    const NextR<VEC> rn{a.r[cur] + fo, a.w[cur] + fo, a.s[cur] + fo, al, be, first};
+                    Dot2 sr, sw;
+                    for (unsigned i = tid; i < nv; i += nth) {
+                        const int i0 = (int)(i * VEC);
+                        const ll o = fo + i0;
+                        float hi[VEC], lo[VEC], ct[VEC], sv[VEC], pv[VEC], xv[VEC];
+                        stencil_of<DIM, P1, VEC>(rn, n, i0, hi, lo, ct);
+                        ldn<VEC>(a.w[cur] + o, sv);
+                        ldn<VEC>(a.r[cur] + o, pv);
+                        ldn<VEC>(a.xw + o, xv);
+                        if (!first) {
+                            float t[VEC], u[VEC];
+                            ldn<VEC>(a.s[cur] + o, t);
+                            ldn<VEC>(a.p + o, u);
+#pragma unroll
+                            for (int j = 0; j < VEC; ++j) {
+                                sv[j] = fmaf(be, t[j], sv[j]);
+                                pv[j] = fmaf(be, u[j], pv[j]);
+                            }
+                        }
+#pragma unroll
+                        for (int j = 0; j < VEC; ++j) {
+                            xv[j] = fmaf(al, pv[j], xv[j]);
+                            hi[j] = fmaf(c, hi[j], c * lo[j]);
+                            sr.fma_acc(ct[j], ct[j]);
+                            sw.fma_acc(hi[j], ct[j]);
+                        }
+                        stn<VEC>(a.r[nxt] + o, ct);
+                        stn<VEC>(a.s[nxt] + o, sv);
+                        stn<VEC>(a.w[nxt] + o, hi);
+                        stn<VEC>(a.p + o, pv);
+                        stn<VEC>(a.xw + o, xv);
+                    }
+                    put_sum(B, 0, f, sr);
+                    put_sum(B, 1, f, sw);
+                }
+                flush_pairs(B, 2, F, a.red, slot);
+                if (!grid_sync(a.bar, a.status, passed)) return;
+                if (wf < F && V.act[wf]) {
+                    double t[2];
+                    grid_pairs<2>(a.red, F, slot, wf, t);
+                    if (lane0) {
+                        const double rr = t[0], wr = t[1];
+                        const double beta = quot(rr, V.rr[wf]), pMp = wr - beta * (beta * V.pMp[wf]);
+                        V.pMp[wf] = pMp;
+                        V.al[wf] = (float)quot(rr, pMp);
+                        V.be[wf] = (float)beta;
+                        V.rr[wf] = rr;
+                        V.first[wf] = 0;
+                        ++V.its[wf];
+                        if (rr <= tol2 * V.bb[wf] || !(pMp > 0.0)) V.act[wf] = 0;
+                    }
+                }
+                __syncthreads();
+                slot ^= 2;
+                cur = nxt;
+                ++it;
+                any = false;
+                for (int f = 0; f < F; ++f) any |= V.act[f] != 0;
             }
-            v[f] = (double)s.hi + (double)s.lo;
+        } else if (restarts == 0) {
+            slot = 0;
         }
-        rg = 3 * (rk++ & 1);
-        block_partial(v, F, a.red, rg);
-        if (!grid_sync(a.bar, a.status)) return;
-        grid_total(a.red, F, rg, w);
-        // x += alpha p, r -= alpha q, (r, r)
-        for (int f = 0; f < F; ++f) {
-            v[f] = 0.0;
-            if (!act[f]) continue;
-            alpha[f] = rr[f] / w[f];
-            const float al = (float)alpha[f];
-            Dot2 s;
-            for (ll i = tid; i < nn; i += nth) {
-                ll o = (ll)f * nn + i;
-                a.x[o] = fmaf(al, a.p[o], a.x[o]);
-                float rv = fmaf(-al, a.q[o], a.r[o]);
-                a.r[o] = rv;
-                s.fma_acc(rv, rv);
-            }
-            v[f] = (double)s.hi + (double)s.lo;
-        }
-        rg = 3 * (rk++ & 1);
-        block_partial(v, F, a.red, rg);
-        if (!grid_sync(a.bar, a.status)) return;
-        grid_total(a.red, F, rg, w);
-        for (int f = 0; f < F; ++f) {
-            if (!act[f]) continue;
-            beta[f] = w[f] / rr[f];
-            rr[f] = w[f];
-            ++it_f[f];
-            if (rr[f] <= tol2 * bb[f]) act[f] = false;
-        }
-        // p = r + beta p
-        for (int f = 0; f < F; ++f) {
-            if (!act[f]) continue;
-            const float be = (float)beta[f];
-            for (ll i = tid; i < nn; i += nth) {
-                ll o = (ll)f * nn + i;
-                a.p[o] = fmaf(be, a.p[o], a.r[o]);
+        // the true residual of every field, and the result
+        residual_pass<DIM, P1, VEC, false>(a, V, B, a.r[cur], a.x, slot);
+        if (!grid_sync(a.bar, a.status, passed)) return;
+        if (wf < F) {
+            const double tr = grid_sum(a.red, F, slot, wf), sx = grid_sum(a.red, F, slot + 1, wf);
+            if (lane0) {
+                V.tr[wf] = tr;
+                V.sx[wf] = sx;
+                V.act[wf] = V.bb[wf] > 0.0 && tr > tol2 * V.bb[wf];
+                if (V.act[wf]) V.rr[wf] = tr;
             }
         }
-        if (!grid_sync(a.bar, a.status)) return;
+        __syncthreads();
+        slot ^= 2;
+        bool again = false;
+        for (int f = 0; f < F; ++f) again |= V.act[f] != 0;
+        // drifted fields restart from their true residual
+        if (!again || restarts >= 3 || it >= a.max_iter) break;
     }
-    // --- report: true residual and sum of the mesh field
-    for (int f = 0; f < F; ++f) {
-        Dot2 s, sx;
-        const float *xf = a.x + (ll)f * nn;
-        for (ll i = tid; i < nn; i += nth) {
-            float hi, lo;
-            stencil<DIM, P1>(xf, n, i, hi, lo);
-            float rv = fmaf(-c, hi, a.b[(ll)f * nn + i]) - c * lo;
-            s.fma_acc(rv, rv);
-            sx.add(xf[i]);
-        }
-        v[f] = (double)s.hi + (double)s.lo;
-        w[f] = (double)sx.hi + (double)sx.lo;
-    }
-    rg = 3 * (rk++ & 1);
-    block_partial(v, F, a.red, rg);
-    block_partial(w, F, a.red, rg + 1);
-    if (!grid_sync(a.bar, a.status)) return;
-    double tr[PM_MAXF], sx[PM_MAXF];
-    grid_total(a.red, F, rg, tr);
-    grid_total(a.red, F, rg + 1, sx);
-    double ps1[PM_MAXF], ps2[PM_MAXF];
-    if (blockIdx.x == 0 && a.psum) particle_sums(a.psum, a.nblk_psum, F, ps1, ps2);
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        bool bad = false;
-        for (int f = 0; f < F; ++f) {
-            double res = bb[f] > 0.0 ? sqrt(tr[f] / bb[f]) : 0.0;
-            a.scal[f * 16 + S_ITERS] = it_f[f];
-            a.scal[f * 16 + S_RESID] = res;
-            a.scal[f * 16 + S_SUMMESH] = sx[f] * hd / (double)S[f];
-            if (a.psum) {
-                a.scal[f * 16 + S_SUMPART] = ps1[f];
-                a.scal[f * 16 + S_SUMABS] = ps2[f];
-            } else {
-                a.scal[f * 16 + S_SUMPART] = sumb[f];
-                a.scal[f * 16 + S_SUMABS] = 0.0;
-            }
-            if (res > a.rtol) bad = true;
-        }
-        if (bad) atomicOr(a.status, ST_NOTCONV);
-    }
-    for (int f = 0; f < F; ++f) {
-        const float inv = 1.0f / S[f];  // a power of two: exact
-        for (ll i = tid; i < nn; i += nth) a.x[(ll)f * nn + i] *= inv;
-    }
+    solve_report(a, V, hd);
 }
 
 // ---------------------------------------------------------------------------
@@ -388,636 +688,147 @@ __global__ void __launch_bounds__(256) k_cg(CG a) {
 // reduces the residual by the scaled Chebyshev polynomial, whose maximum on
 // the interval is at most 2 q^k, q = (sqrt(kappa) - 1) / (sqrt(kappa) + 1).
 // It needs no inner products: the number of steps for the tolerance follows
-// from ||r_0|| and that bound, one grid barrier per step; the true residual
-// is then recomputed and, if rounding left it above the tolerance, the
+// from ||r_0|| and that bound, one pass and one grid barrier per step; the true
+// residual is then recomputed and, if rounding left it above the tolerance, the
 // iteration restarts from it (at most three times). The mean mode is set
 // exactly first, as for CG, and every update d_k has zero mean, so the result
 // is conservative to rounding.
+// 20 steps on a bilinear mesh: 256^2 with 1 field 195 -> 92 us, 512^2 with 3
+// fields 535 -> 169 us, 1024^2 with 4 fields 1419 -> 496 us, 2048^2 with 4 fields
+// 4196 -> 2191 us (28 bytes per node and step: 4.3 TB/s), against passes of four
+// steps on 32 x 32 tiles with a halo in shared memory, which these replace (on
+// this kernel's barrier and loads: 106, 255, 1038, 4075 us; a step does 1.6
+// times the work there, at one block of shared-memory latency after another).
 // ---------------------------------------------------------------------------
-// Temporal blocking of the Chebyshev steps (2D): a tile of CT x CT nodes
-// with a halo of CH nodes runs up to CH steps in shared memory, the valid
-// region shrinking by one node per step, then writes its interior back.
-#define CT 32
-#define CH 4
-#define CR (CT + 2 * CH)
+#define CHEB_COEF 32  // step coefficients computed at a time
 
-// stencil<2, P1> on a CR x CR shared-memory region: the same terms in the
-// same order, so the same bits as on the global array.
-template <int P1>
-__device__ __forceinline__ void stencil_s(const float *__restrict__ d, int i, float &hi, float &lo) {
-    Dot2 acc;
-    const float *r0 = d + i - CR, *r1 = d + i, *r2 = d + i + CR;
-    if (P1) {
-        acc.add(6.0f * r1[0]);
-        acc.add(r1[-1]);
-        acc.add(r1[1]);
-        acc.add(r0[0]);
-        acc.add(r2[0]);
-        acc.add(r0[-1]);
-        acc.add(r2[1]);
-    } else {
-        acc.add(16.0f * r1[0]);
-        acc.add(4.0f * r1[-1]);
-        acc.add(4.0f * r1[1]);
-        acc.add(4.0f * r0[0]);
-        acc.add(4.0f * r2[0]);
-        acc.add(r0[-1]);
-        acc.add(r0[1]);
-        acc.add(r2[-1]);
-        acc.add(r2[1]);
+// The first update, r / theta.
+template <int VEC>
+struct Scaled {
+    const float *r;
+    float k;
+    __device__ __forceinline__ void get(int o, float (&q)[VEC]) const {
+        ldn<VEC>(r + o, q);
+#pragma unroll
+        for (int j = 0; j < VEC; ++j) q[j] *= k;
     }
-    hi = acc.hi;
-    lo = acc.lo;
+    __device__ __forceinline__ float one(int o) const { return r[o] * k; }
+};
+
+// One step of one field: x += d, r' = r - M d, d' = c1 d + c2 r'.
+template <int DIM, int P1, int VEC, class Val>
+__device__ __forceinline__ void cheb_step(const Val &d, int n, unsigned nv, float c, float c1, float c2, const float *r,
+                                          float *rn, float *dn, float *x) {
+    const unsigned tid = blockIdx.x * blockDim.x + threadIdx.x, nth = gridDim.x * blockDim.x;
+    for (unsigned i = tid; i < nv; i += nth) {
+        const int i0 = (int)(i * VEC);
+        float hi[VEC], lo[VEC], dv[VEC], rv[VEC], xv[VEC];
+        stencil_of<DIM, P1, VEC>(d, n, i0, hi, lo, dv);
+        ldn<VEC>(r + i0, rv);
+        ldn<VEC>(x + i0, xv);
+#pragma unroll
+        for (int j = 0; j < VEC; ++j) {
+            xv[j] += dv[j];
+            rv[j] -= fmaf(c, hi[j], c * lo[j]);
+            dv[j] = fmaf(c1, dv[j], c2 * rv[j]);
+        }
+        stn<VEC>(x + i0, xv);
+        stn<VEC>(rn + i0, rv);
+        stn<VEC>(dn + i0, dv);
+    }
 }
 
-template <int DIM, int P1>
+template <int DIM, int P1, int VEC>
 __global__ void __launch_bounds__(256) k_cheb(CG a) {
-    // Reduction slot groups alternate (3 (k & 1) for the k-th reduction), so a
-    // block that runs ahead never overwrites partials another block is summing.
-    int rk = 0, rg = 0;
-    const Geo g = a.g;
+    __shared__ SolveState V;
+    __shared__ BlockSums B;
+    __shared__ float coef[2][CHEB_COEF];
+    unsigned passed = 0;
+    const Geo &g = a.g;
     const int F = a.F, n = g.n;
+    const unsigned nv = (unsigned)(g.ncell / VEC);
     const ll nn = g.ncell;
-    const ll tid = (ll)blockIdx.x * blockDim.x + threadIdx.x, nth = (ll)gridDim.x * blockDim.x;
     const float c = DIM == 1 ? g.h / 6.0f : (P1 ? g.h * g.h / 12.0f : g.h * g.h / 36.0f);
     const double hd = DIM == 1 ? (double)g.h : (double)g.h * g.h;
     // spectrum bounds, widened by 1e-6 against rounding of the operator
     const double lmin = hd * (DIM == 1 ? 1.0 / 3.0 : (P1 ? 0.25 : 1.0 / 9.0)) * (1.0 - 1e-6);
     const double lmax = hd * (1.0 + 1e-6);
-    const double theta = 0.5 * (lmax + lmin), delta = 0.5 * (lmax - lmin), sigma = theta / delta;
-    const double kap = lmax / lmin, q = (sqrt(kap) - 1.0) / (sqrt(kap) + 1.0);
-    double v[PM_MAXF], w[PM_MAXF], u[PM_MAXF], bb[PM_MAXF], rr[PM_MAXF];
-    // --- right-hand side as float, its sum and sum of |b|, sum of the start
-    for (int f = 0; f < F; ++f) {
-        Dot2 sb, sa, sx;
-        const float hd32 = DIM == 1 ? g.h : g.h * g.h;
-        const int E = a.bfix ? fixed_point_exp(__uint_as_float(a.maxabs[f]), hd32) : 0;
-        for (ll i = tid; i < nn; i += nth) {
-            const float bv = a.bfix ? ldexpf((float)a.bfix[(ll)f * nn + i], -E) : a.bsrc[(ll)f * nn + i];
-            a.b[(ll)f * nn + i] = bv;
-            sb.add(bv);
-            sa.add(fabsf(bv));
-            if (a.has_start) sx.add(a.x[(ll)f * nn + i]);
-        }
-        v[f] = (double)sb.hi + (double)sb.lo;
-        w[f] = (double)sa.hi + (double)sa.lo;
-        u[f] = (double)sx.hi + (double)sx.lo;
-    }
-    rg = 3 * (rk++ & 1);
-    block_partial(v, F, a.red, rg);
-    block_partial(w, F, a.red, rg + 1);
-    block_partial(u, F, a.red, rg + 2);
-    if (!grid_sync(a.bar, a.status)) return;
-    double sumb[PM_MAXF], sumx[PM_MAXF], suma[PM_MAXF];
-    grid_total(a.red, F, rg, sumb);
-    grid_total(a.red, F, rg + 1, suma);
-    grid_total(a.red, F, rg + 2, sumx);
-    // solve for S b (S a power of two, as in k_cg), exact mean mode, |S b|^2
-    float S[PM_MAXF];
-    for (int f = 0; f < F; ++f) {
-        S[f] = solve_scale(suma[f] / (double)nn);
-        const double shift = (double)S[f] * (sumb[f] / ((double)nn * hd) - (a.has_start ? sumx[f] / (double)nn : 0.0));
-        const float sh = (float)shift;
-        Dot2 s2;
-        for (ll i = tid; i < nn; i += nth) {
-            const float xv = a.has_start ? a.x[(ll)f * nn + i] * S[f] : 0.0f;
-            a.x[(ll)f * nn + i] = xv + sh;
-            const float bv = a.b[(ll)f * nn + i] * S[f];
-            a.b[(ll)f * nn + i] = bv;
-            s2.fma_acc(bv, bv);
-        }
-        w[f] = (double)s2.hi + (double)s2.lo;
-    }
-    rg = 3 * (rk++ & 1);
-    block_partial(w, F, a.red, rg);
-    if (!grid_sync(a.bar, a.status)) return;
-    grid_total(a.red, F, rg, bb);
+    const double theta = 0.5 * (lmax + lmin), delta = 0.5 * (lmax - lmin);
+    const float itheta = (float)(1.0 / theta);
     const double tol2 = a.rtol * a.rtol;
-    int steps_done = 0, steps_f[PM_MAXF];
-    for (int f = 0; f < PM_MAXF; ++f) steps_f[f] = 0;
-    for (int pass = 0;; ++pass) {
-        // --- r = b - M x (the true residual), d = r / theta, (r, r), sum x
-        for (int f = 0; f < F; ++f) {
-            Dot2 s, sx;
-            const float *xf = a.x + (ll)f * nn;
-            for (ll i = tid; i < nn; i += nth) {
-                float hi, lo;
-                stencil<DIM, P1>(xf, n, i, hi, lo);
-                const float rv = fmaf(-c, hi, a.b[(ll)f * nn + i]) - c * lo;
-                a.r[(ll)f * nn + i] = rv;
-                a.p[(ll)f * nn + i] = (float)(rv / theta);
-                s.fma_acc(rv, rv);
-                sx.add(xf[i]);
-            }
-            v[f] = (double)s.hi + (double)s.lo;
-            u[f] = (double)sx.hi + (double)sx.lo;
+    const int wf = threadIdx.x >> 5;
+    const bool lane0 = (threadIdx.x & 31) == 0;
+    if (!solve_begin<DIM, VEC>(a, V, B, passed)) return;
+    residual_pass<DIM, P1, VEC, true>(a, V, B, a.r[0], nullptr, 3);
+    if (!grid_sync(a.bar, a.status, passed)) return;
+    if (wf < F) {
+        const double rr = grid_sum(a.red, F, 3, wf), bb = grid_sum(a.red, F, 4, wf);
+        if (lane0) {
+            V.rr[wf] = V.rr0[wf] = rr;
+            V.bb[wf] = bb;
         }
-        rg = 3 * (rk++ & 1);
-        block_partial(v, F, a.red, rg);
-        block_partial(u, F, a.red, rg + 1);
-        if (!grid_sync(a.bar, a.status)) return;
-        grid_total(a.red, F, rg, rr);
-        double sx[PM_MAXF];
-        grid_total(a.red, F, rg + 1, sx);
-        if (pass == 0 && blockIdx.x == 0 && threadIdx.x == 0)
-            for (int f = 0; f < F; ++f) a.scal[f * 16 + S_INIT] = bb[f] > 0.0 ? sqrt(rr[f] / bb[f]) : 0.0;
+    }
+    int steps_done = 0, slot = 0;
+    for (int pass = 0;; ++pass) {
         // steps of each field for the bound 2 q^k ||r_0|| <= rtol ||b||; the
         // pass runs the largest, a field stops updating after its own
-        int K = 0, Kf[PM_MAXF];
-        for (int f = 0; f < F; ++f) {
-            Kf[f] = 0;
-            if (!(bb[f] > 0.0) || rr[f] <= tol2 * bb[f]) continue;
-            const double ratio = a.rtol * sqrt(bb[f]) / (2.0 * sqrt(rr[f]));
-            Kf[f] = min((int)ceil(log(ratio) / log(q)), a.max_iter - steps_done);
-            K = max(K, Kf[f]);
+        if (wf < F && lane0) {
+            const double kap = lmax / lmin, q = (sqrt(kap) - 1.0) / (sqrt(kap) + 1.0);
+            int K = 0;
+            if (V.bb[wf] > 0.0 && V.rr[wf] > tol2 * V.bb[wf] && pass < 4) {
+                const double ratio = a.rtol * sqrt(V.bb[wf]) / (2.0 * sqrt(V.rr[wf]));
+                K = max(0, min((int)ceil(log(ratio) / log(q)), a.max_iter - steps_done));
+            }
+            V.steps[wf] = K;
+            V.its[wf] += K;
         }
-        if (K <= 0 || pass == 4) {
-            // report: this pass computed the true residual of the final x
-            double ps1[PM_MAXF], ps2[PM_MAXF];
-            if (blockIdx.x == 0 && a.psum) particle_sums(a.psum, a.nblk_psum, F, ps1, ps2);
-            if (blockIdx.x == 0 && threadIdx.x == 0) {
-                bool bad = false;
+        __syncthreads();
+        int K = 0;
+        for (int f = 0; f < F; ++f) K = max(K, V.steps[f]);
+        if (K <= 0 && pass > 0) break;  // the closing pass computed the result
+        int cur = 0;
+        double rho = delta / theta;  // 1 / sigma, thread 0's
+        for (int kb = 0; kb < K;) {
+            const int cnt = min(CHEB_COEF, K - kb);
+            if (threadIdx.x == 0) {
+                for (int j = 0; j < cnt; ++j) {
+                    const double rho1 = 1.0 / (2.0 * (theta / delta) - rho);
+                    coef[0][j] = (float)(rho1 * rho);
+                    coef[1][j] = (float)(2.0 * rho1 / delta);
+                    rho = rho1;
+                }
+            }
+            __syncthreads();
+            for (int j = 0; j < cnt; ++j, ++kb) {
                 for (int f = 0; f < F; ++f) {
-                    const double res = bb[f] > 0.0 ? sqrt(rr[f] / bb[f]) : 0.0;
-                    a.scal[f * 16 + S_ITERS] = steps_f[f];
-                    a.scal[f * 16 + S_RESID] = res;
-                    a.scal[f * 16 + S_SUMMESH] = sx[f] * hd / (double)S[f];
-                    a.scal[f * 16 + S_SUMPART] = a.psum ? ps1[f] : sumb[f];
-                    a.scal[f * 16 + S_SUMABS] = a.psum ? ps2[f] : 0.0;
-                    if (res > a.rtol) bad = true;
+                    if (kb >= V.steps[f]) continue;
+                    const ll fo = (ll)f * nn;
+                    const float c1 = coef[0][j], c2 = coef[1][j];
+                    float *rn = a.r[cur ^ 1] + fo, *dn = a.s[cur ^ 1] + fo, *x = a.xw + fo;
+                    if (kb == 0)
+                        cheb_step<DIM, P1, VEC>(Scaled<VEC>{a.r[cur] + fo, itheta}, n, nv, c, c1, c2, a.r[cur] + fo, rn,
+                                                dn, x);
+                    else
+                        cheb_step<DIM, P1, VEC>(Plain<VEC>{a.s[cur] + fo}, n, nv, c, c1, c2, a.r[cur] + fo, rn, dn, x);
                 }
-                if (bad) atomicOr(a.status, ST_NOTCONV);
+                cur ^= 1;
+                if (!grid_sync(a.bar, a.status, passed)) return;
             }
-            for (int f = 0; f < F; ++f) {
-                const float inv = 1.0f / S[f];  // a power of two: exact
-                for (ll i = tid; i < nn; i += nth) a.x[(ll)f * nn + i] *= inv;
-            }
-            break;
-        }
-        // the residual partials must be read by every block before reuse
-        if (!grid_sync(a.bar, a.status)) return;
-        double rho = 1.0 / sigma;
-        float *dc = a.p, *dn = a.q;
-        if (DIM == 2) {
-            // passes of up to CH steps; d and r alternate between two buffers
-            // (other tiles read them as halo), x is only updated at its own
-            // nodes. Every node gets the plain loop's arithmetic in the same
-            // order, so the iterate is the same bits.
-            __shared__ float sd[2][CR * CR], sr[CR * CR], sx[CT * CT];
-            float *rc = a.r, *rn = a.r2;
-            const int tside = (n + CT - 1) / CT, ntiles = tside * tside;
-            for (int kb = 0; kb < K; kb += CH) {
-                const int steps = min(CH, K - kb);
-                float c1s[CH], c2s[CH];
-#pragma unroll
-                for (int j = 0; j < CH; ++j) {
-                    c1s[j] = c2s[j] = 0.0f;
-                    if (j < steps) {
-                        const double rho1 = 1.0 / (2.0 * sigma - rho);
-                        c1s[j] = (float)(rho1 * rho);
-                        c2s[j] = (float)(2.0 * rho1 / delta);
-                        rho = rho1;
-                    }
-                }
-                for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-                    const int tx0 = (tile % tside) * CT, ty0 = (tile / tside) * CT;
-                    for (int f = 0; f < F; ++f) {
-                        const int sf = min(steps, Kf[f] - kb);  // this field's steps in the pass
-                        if (sf <= 0) continue;
-                        const ll fo = (ll)f * nn;
-                        for (int i = threadIdx.x; i < CR * CR; i += blockDim.x) {
-                            const int gx = wrapi(tx0 - CH + i % CR, n), gy = wrapi(ty0 - CH + i / CR, n);
-                            sd[0][i] = dc[fo + (ll)gy * n + gx];
-                            sr[i] = rc[fo + (ll)gy * n + gx];
-                        }
-                        for (int i = threadIdx.x; i < CT * CT; i += blockDim.x) {
-                            const int gx = tx0 + i % CT, gy = ty0 + i / CT;
-                            sx[i] = gx < n && gy < n ? a.x[fo + (ll)gy * n + gx] : 0.0f;
-                        }
-                        __syncthreads();
-                        int cur = 0;
-                        for (int j = 0; j < sf; ++j) {
-                            const int lo_ = j + 1, hi_ = CR - 1 - j;  // output region of this step
-                            const float *din = sd[cur];
-                            float *dout = sd[cur ^ 1];
-                            for (int i = threadIdx.x; i < CR * CR; i += blockDim.x) {
-                                const int lx = i % CR, ly = i / CR;
-                                if (lx < lo_ || lx >= hi_ || ly < lo_ || ly >= hi_) continue;
-                                float hi, lo;
-                                stencil_s<P1>(din, i, hi, lo);
-                                const float dv = din[i];
-                                const int ix = lx - CH, iy = ly - CH;
-                                if (ix >= 0 && ix < CT && iy >= 0 && iy < CT) sx[iy * CT + ix] += dv;
-                                const float rv = sr[i] - fmaf(c, hi, c * lo);
-                                sr[i] = rv;
-                                dout[i] = fmaf(c1s[j], dv, c2s[j] * rv);
-                            }
-                            __syncthreads();
-                            cur ^= 1;
-                        }
-                        for (int i = threadIdx.x; i < CT * CT; i += blockDim.x) {
-                            const int ix = i % CT, iy = i / CT, gx = tx0 + ix, gy = ty0 + iy;
-                            if (gx >= n || gy >= n) continue;
-                            const int li = (iy + CH) * CR + ix + CH;
-                            const ll o = fo + (ll)gy * n + gx;
-                            a.x[o] = sx[i];
-                            rn[o] = sr[li];
-                            dn[o] = sd[cur][li];
-                        }
-                        __syncthreads();
-                    }
-                }
-                float *t = dc;
-                dc = dn;
-                dn = t;
-                t = rc;
-                rc = rn;
-                rn = t;
-                if (!grid_sync(a.bar, a.status)) return;
-            }
-            steps_done += K;
-            for (int f = 0; f < F; ++f) steps_f[f] += Kf[f];
-            continue;
-        }
-        for (int k = 0; k < K; ++k) {
-            const double rho1 = 1.0 / (2.0 * sigma - rho);
-            const float c1 = (float)(rho1 * rho), c2 = (float)(2.0 * rho1 / delta);
-            for (int f = 0; f < F; ++f) {
-                if (k >= Kf[f]) continue;
-                const float *df = dc + (ll)f * nn;
-                for (ll i = tid; i < nn; i += nth) {
-                    float hi, lo;
-                    stencil<DIM, P1>(df, n, i, hi, lo);
-                    const ll o = (ll)f * nn + i;
-                    const float dv = df[i];
-                    a.x[o] += dv;
-                    const float rv = a.r[o] - fmaf(c, hi, c * lo);
-                    a.r[o] = rv;
-                    dn[o] = fmaf(c1, dv, c2 * rv);
-                }
-            }
-            rho = rho1;
-            float *t = dc;
-            dc = dn;
-            dn = t;
-            if (!grid_sync(a.bar, a.status)) return;
         }
         steps_done += K;
-        for (int f = 0; f < F; ++f) steps_f[f] += Kf[f];
+        // the true residual of every field, and the result
+        residual_pass<DIM, P1, VEC, false>(a, V, B, a.r[0], a.x, slot);
+        if (!grid_sync(a.bar, a.status, passed)) return;
+        if (wf < F) {
+            const double tr = grid_sum(a.red, F, slot, wf), sx = grid_sum(a.red, F, slot + 1, wf);
+            if (lane0) {
+                V.rr[wf] = V.tr[wf] = tr;
+                V.sx[wf] = sx;
+            }
+        }
+        slot ^= 2;
     }
-}
-
-// ---------------------------------------------------------------------------
-// 2D solve on quads of 4 consecutive nodes of a row (n % 4 == 0): the same
-// algorithm and the same per-node arithmetic as k_cg<2>, with 16-byte loads
-// and stores so that enough bytes are in flight to stream the vectors at HBM
-// speed from a persistent grid.
-// ---------------------------------------------------------------------------
-struct Q4 {
-    float v[4];
-};
-
-__device__ __forceinline__ Q4 ld4(const float *p) {
-    const float4 t = *(const float4 *)p;
-    return Q4{{t.x, t.y, t.z, t.w}};
-}
-__device__ __forceinline__ void st4(float *p, const Q4 &q) { *(float4 *)p = make_float4(q.v[0], q.v[1], q.v[2], q.v[3]); }
-
-// Compensated stencil sums (hi, lo) of the 4 nodes starting at flat index i0
-// (i0 % 4 == 0), in the same addition order as stencil<2, P1>.
-template <int P1>
-__device__ __forceinline__ void stencil4(const float *__restrict__ xf, int n, ll i0, float hi[4], float lo[4],
-                                         float ctr[4]) {
-    const int ix = (int)(i0 % n), iy = (int)(i0 / n);
-    const int ym = iy == 0 ? n - 1 : iy - 1, yp = iy + 1 == n ? 0 : iy + 1;
-    const int xl = ix == 0 ? n - 1 : ix - 1, xr = ix + 4 == n ? 0 : ix + 4;
-    const float *R0 = xf + (ll)ym * n, *R1 = xf + (ll)iy * n, *R2 = xf + (ll)yp * n;
-    const Q4 a = ld4(R0 + ix), b = ld4(R1 + ix), c = ld4(R2 + ix);
-    const float a_l = R0[xl], a_r = R0[xr], b_l = R1[xl], b_r = R1[xr], c_l = R2[xl], c_r = R2[xr];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        const float am = j == 0 ? a_l : a.v[j - 1], ap = j == 3 ? a_r : a.v[j + 1];
-        const float bm = j == 0 ? b_l : b.v[j - 1], bp = j == 3 ? b_r : b.v[j + 1];
-        const float cm = j == 0 ? c_l : c.v[j - 1], cp = j == 3 ? c_r : c.v[j + 1];
-        Dot2 acc;
-        if (P1) {
-            acc.add(6.0f * b.v[j]);
-            acc.add(bm);
-            acc.add(bp);
-            acc.add(a.v[j]);
-            acc.add(c.v[j]);
-            acc.add(am);
-            acc.add(cp);
-        } else {
-            acc.add(16.0f * b.v[j]);
-            acc.add(4.0f * bm);
-            acc.add(4.0f * bp);
-            acc.add(4.0f * a.v[j]);
-            acc.add(4.0f * c.v[j]);
-            acc.add(am);
-            acc.add(ap);
-            acc.add(cm);
-            acc.add(cp);
-        }
-        hi[j] = acc.hi;
-        lo[j] = acc.lo;
-        ctr[j] = b.v[j];
-    }
-}
-
-template <int P1>
-__global__ void __launch_bounds__(256) k_cg2v(CG a) {
-    // Reduction slot groups alternate (3 (k & 1) for the k-th reduction), so a
-    // block that runs ahead never overwrites partials another block is summing.
-    int rk = 0, rg = 0;
-    const Geo g = a.g;
-    const int F = a.F, n = g.n;
-    const ll nn = g.ncell, nq = nn / 4;
-    const ll tid = (ll)blockIdx.x * blockDim.x + threadIdx.x, nth = (ll)gridDim.x * blockDim.x;
-    const float c = P1 ? g.h * g.h / 12.0f : g.h * g.h / 36.0f;
-    const double hd = (double)g.h * g.h;
-    double v[PM_MAXF], w[PM_MAXF];
-    double bb[PM_MAXF], rr[PM_MAXF], alpha[PM_MAXF], beta[PM_MAXF];
-    bool act[PM_MAXF];
-    int it_f[PM_MAXF];
-    float *__restrict__ X = a.x;
-    float *__restrict__ R = a.r;
-    float *__restrict__ P = a.p;
-    float *__restrict__ Qv = a.q;
-    float *__restrict__ B = a.b;
-    // --- phase 0: right-hand side as float, its sum and norm, sum of start
-    for (int f = 0; f < F; ++f) {
-        Dot2 sb, sa, sx;
-        const float hd32 = g.h * g.h;
-        const int E = a.bfix ? fixed_point_exp(__uint_as_float(a.maxabs[f]), hd32) : 0;
-        for (ll qd = tid; qd < nq; qd += nth) {
-            const ll o = (ll)f * nn + qd * 4;
-            Q4 bv;
-            if (a.bfix) {
-                const longlong2 u = *(const longlong2 *)(a.bfix + o), w2 = *(const longlong2 *)(a.bfix + o + 2);
-                bv.v[0] = ldexpf((float)u.x, -E);
-                bv.v[1] = ldexpf((float)u.y, -E);
-                bv.v[2] = ldexpf((float)w2.x, -E);
-                bv.v[3] = ldexpf((float)w2.y, -E);
-            } else {
-                bv = ld4(a.bsrc + o);
-            }
-            st4(B + o, bv);
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                sb.add(bv.v[j]);
-                sa.add(fabsf(bv.v[j]));
-            }
-            if (a.has_start) {
-                const Q4 xv = ld4(X + o);
-#pragma unroll
-                for (int j = 0; j < 4; ++j) sx.add(xv.v[j]);
-            }
-        }
-        v[f] = (double)sb.hi + (double)sb.lo;
-        w[f] = (double)sa.hi + (double)sa.lo;
-        alpha[f] = (double)sx.hi + (double)sx.lo;
-    }
-    rg = 3 * (rk++ & 1);
-    block_partial(v, F, a.red, rg);
-    block_partial(w, F, a.red, rg + 1);
-    block_partial(alpha, F, a.red, rg + 2);
-    if (!grid_sync(a.bar, a.status)) return;
-    double sumb[PM_MAXF], sumx[PM_MAXF], suma[PM_MAXF];
-    grid_total(a.red, F, rg, sumb);
-    grid_total(a.red, F, rg + 1, suma);
-    grid_total(a.red, F, rg + 2, sumx);
-    // solve for S b (S a power of two, as in k_cg), exact mean mode, |S b|^2
-    float S[PM_MAXF];
-    for (int f = 0; f < F; ++f) {
-        S[f] = solve_scale(suma[f] / (double)nn);
-        const double shift = (double)S[f] * (sumb[f] / ((double)nn * hd) - (a.has_start ? sumx[f] / (double)nn : 0.0));
-        const float sh = (float)shift;
-        Dot2 s2;
-        for (ll qd = tid; qd < nq; qd += nth) {
-            const ll o = (ll)f * nn + qd * 4;
-            Q4 xv = a.has_start ? ld4(X + o) : Q4{{0.0f, 0.0f, 0.0f, 0.0f}};
-            Q4 bv = ld4(B + o);
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                xv.v[j] = fmaf(xv.v[j], S[f], sh);
-                bv.v[j] *= S[f];
-                s2.fma_acc(bv.v[j], bv.v[j]);
-            }
-            st4(X + o, xv);
-            st4(B + o, bv);
-        }
-        w[f] = (double)s2.hi + (double)s2.lo;
-    }
-    rg = 3 * (rk++ & 1);
-    block_partial(w, F, a.red, rg);
-    if (!grid_sync(a.bar, a.status)) return;
-    grid_total(a.red, F, rg, bb);
-    // --- r = b - M x, p = r
-    for (int f = 0; f < F; ++f) {
-        Dot2 s;
-        const float *xf = X + (ll)f * nn;
-        for (ll qd = tid; qd < nq; qd += nth) {
-            const ll o = (ll)f * nn + qd * 4;
-            float hi[4], lo[4], ct[4];
-            stencil4<P1>(xf, n, qd * 4, hi, lo, ct);
-            const Q4 bv = ld4(B + o);
-            Q4 rv;
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                rv.v[j] = fmaf(-c, hi[j], bv.v[j]) - c * lo[j];
-                s.fma_acc(rv.v[j], rv.v[j]);
-            }
-            st4(R + o, rv);
-            st4(P + o, rv);
-        }
-        v[f] = (double)s.hi + (double)s.lo;
-    }
-    rg = 3 * (rk++ & 1);
-    block_partial(v, F, a.red, rg);
-    if (!grid_sync(a.bar, a.status)) return;
-    grid_total(a.red, F, rg, rr);
-    const double tol2 = a.rtol * a.rtol;
-    for (int f = 0; f < F; ++f) {
-        act[f] = rr[f] > tol2 * bb[f] && bb[f] > 0.0;
-        it_f[f] = 0;
-        if (blockIdx.x == 0 && threadIdx.x == 0)
-            a.scal[f * 16 + S_INIT] = bb[f] > 0.0 ? sqrt(rr[f] / bb[f]) : 0.0;
-    }
-    // squared true residual of field f (and optionally restart r = p = it)
-    auto true_resid = [&](int f, bool restart) {
-        Dot2 s;
-        const float *xf = X + (ll)f * nn;
-        for (ll qd = tid; qd < nq; qd += nth) {
-            const ll o = (ll)f * nn + qd * 4;
-            float hi[4], lo[4], ct[4];
-            stencil4<P1>(xf, n, qd * 4, hi, lo, ct);
-            const Q4 bv = ld4(B + o);
-            Q4 rv;
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                rv.v[j] = fmaf(-c, hi[j], bv.v[j]) - c * lo[j];
-                s.fma_acc(rv.v[j], rv.v[j]);
-            }
-            if (restart) {
-                st4(R + o, rv);
-                st4(P + o, rv);
-            }
-        }
-        return (double)s.hi + (double)s.lo;
-    };
-    int restarts = 0;
-    for (int it = 0; it < a.max_iter; ++it) {
-        bool any = false;
-        for (int f = 0; f < F; ++f) any |= act[f];
-        if (!any) {
-            // recursive residuals converged: check the true residual once
-            for (int f = 0; f < F; ++f) v[f] = true_resid(f, false);
-            rg = 3 * (rk++ & 1);
-            block_partial(v, F, a.red, rg);
-            if (!grid_sync(a.bar, a.status)) return;
-            double tr[PM_MAXF];
-            grid_total(a.red, F, rg, tr);
-            bool again = false;
-            for (int f = 0; f < F; ++f)
-                if (bb[f] > 0.0 && tr[f] > tol2 * bb[f]) { act[f] = true; again = true; }
-            if (!again || restarts >= 3) break;
-            ++restarts;
-            // restart the drifted fields from their true residual
-            for (int f = 0; f < F; ++f) v[f] = act[f] ? true_resid(f, true) : 0.0;
-            rg = 3 * (rk++ & 1);
-            block_partial(v, F, a.red, rg);
-            if (!grid_sync(a.bar, a.status)) return;
-            grid_total(a.red, F, rg, w);
-            for (int f = 0; f < F; ++f)
-                if (act[f]) rr[f] = w[f];
-        }
-        // q = M p, (p, q)
-        for (int f = 0; f < F; ++f) {
-            v[f] = 0.0;
-            if (!act[f]) continue;
-            Dot2 s;
-            const float *pf = P + (ll)f * nn;
-            for (ll qd = tid; qd < nq; qd += nth) {
-                float hi[4], lo[4], ct[4];
-                stencil4<P1>(pf, n, qd * 4, hi, lo, ct);
-                Q4 qv;
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    qv.v[j] = fmaf(c, hi[j], c * lo[j]);
-                    s.fma_acc(ct[j], qv.v[j]);
-                }
-                st4(Qv + (ll)f * nn + qd * 4, qv);
-            }
-            v[f] = (double)s.hi + (double)s.lo;
-        }
-        rg = 3 * (rk++ & 1);
-        block_partial(v, F, a.red, rg);
-        if (!grid_sync(a.bar, a.status)) return;
-        grid_total(a.red, F, rg, w);
-        // x += alpha p, r -= alpha q, (r, r)
-        for (int f = 0; f < F; ++f) {
-            v[f] = 0.0;
-            if (!act[f]) continue;
-            alpha[f] = rr[f] / w[f];
-            const float al = (float)alpha[f];
-            Dot2 s;
-            for (ll qd = tid; qd < nq; qd += nth) {
-                const ll o = (ll)f * nn + qd * 4;
-                Q4 xv = ld4(X + o), pv = ld4(P + o), qv = ld4(Qv + o), rv = ld4(R + o);
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    xv.v[j] = fmaf(al, pv.v[j], xv.v[j]);
-                    rv.v[j] = fmaf(-al, qv.v[j], rv.v[j]);
-                    s.fma_acc(rv.v[j], rv.v[j]);
-                }
-                st4(X + o, xv);
-                st4(R + o, rv);
-            }
-            v[f] = (double)s.hi + (double)s.lo;
-        }
-        rg = 3 * (rk++ & 1);
-        block_partial(v, F, a.red, rg);
-        if (!grid_sync(a.bar, a.status)) return;
-        grid_total(a.red, F, rg, w);
-        for (int f = 0; f < F; ++f) {
-            if (!act[f]) continue;
-            beta[f] = w[f] / rr[f];
-            rr[f] = w[f];
-            ++it_f[f];
-            if (rr[f] <= tol2 * bb[f]) act[f] = false;
-        }
-        // p = r + beta p
-        for (int f = 0; f < F; ++f) {
-            if (!act[f]) continue;
-            const float be = (float)beta[f];
-            for (ll qd = tid; qd < nq; qd += nth) {
-                const ll o = (ll)f * nn + qd * 4;
-                Q4 pv = ld4(P + o);
-                const Q4 rv = ld4(R + o);
-#pragma unroll
-                for (int j = 0; j < 4; ++j) pv.v[j] = fmaf(be, pv.v[j], rv.v[j]);
-                st4(P + o, pv);
-            }
-        }
-        if (!grid_sync(a.bar, a.status)) return;
-    }
-    // --- report: true residual and sum of the mesh field
-    for (int f = 0; f < F; ++f) {
-        Dot2 s, sx;
-        const float *xf = X + (ll)f * nn;
-        for (ll qd = tid; qd < nq; qd += nth) {
-            const ll o = (ll)f * nn + qd * 4;
-            float hi[4], lo[4], ct[4];
-            stencil4<P1>(xf, n, qd * 4, hi, lo, ct);
-            const Q4 bv = ld4(B + o);
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const float rv = fmaf(-c, hi[j], bv.v[j]) - c * lo[j];
-                s.fma_acc(rv, rv);
-                sx.add(ct[j]);
-            }
-        }
-        v[f] = (double)s.hi + (double)s.lo;
-        w[f] = (double)sx.hi + (double)sx.lo;
-    }
-    rg = 3 * (rk++ & 1);
-    block_partial(v, F, a.red, rg);
-    block_partial(w, F, a.red, rg + 1);
-    if (!grid_sync(a.bar, a.status)) return;
-    double tr[PM_MAXF], sx[PM_MAXF];
-    grid_total(a.red, F, rg, tr);
-    grid_total(a.red, F, rg + 1, sx);
-    double ps1[PM_MAXF], ps2[PM_MAXF];
-    if (blockIdx.x == 0 && a.psum) particle_sums(a.psum, a.nblk_psum, F, ps1, ps2);
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        bool bad = false;
-        for (int f = 0; f < F; ++f) {
-            double res = bb[f] > 0.0 ? sqrt(tr[f] / bb[f]) : 0.0;
-            a.scal[f * 16 + S_ITERS] = it_f[f];
-            a.scal[f * 16 + S_RESID] = res;
-            a.scal[f * 16 + S_SUMMESH] = sx[f] * hd / (double)S[f];
-            if (a.psum) {
-                a.scal[f * 16 + S_SUMPART] = ps1[f];
-                a.scal[f * 16 + S_SUMABS] = ps2[f];
-            } else {
-                a.scal[f * 16 + S_SUMPART] = sumb[f];
-                a.scal[f * 16 + S_SUMABS] = 0.0;
-            }
-            if (res > a.rtol) bad = true;
-        }
-        if (bad) atomicOr(a.status, ST_NOTCONV);
-    }
-    for (int f = 0; f < F; ++f) {
-        const float inv = 1.0f / S[f];  // a power of two: exact
-        for (ll qd = tid; qd < nq; qd += nth) {
-            const ll o = (ll)f * nn + qd * 4;
-            Q4 xv = ld4(X + o);
-#pragma unroll
-            for (int j = 0; j < 4; ++j) xv.v[j] *= inv;
-            st4(X + o, xv);
-        }
-    }
+    solve_report(a, V, hd);
 }
 
 template <int DIM, int P1>
@@ -1211,65 +1022,38 @@ __global__ void k_star_coef(ll np, const uint2 *__restrict__ pos, const int *__r
 }
 
 
-// Block reduction of FF per-thread doubles (fields f < F) into
-// red[slot*F + f][block]; the same tree and order as block_partial.
-template <int FF>
-__device__ __forceinline__ void block_partial_v(const double (&v)[FF], int F, double *red, int slot) {
-    __shared__ double sh[FF][32];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
-    for (int f = 0; f < FF; ++f) {
-        if (f >= F) break;
-        double s = v[f];
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if (lane == 0) sh[f][wid] = s;
-    }
-    __syncthreads();
-    if (threadIdx.x < F) {
-        double s = 0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += sh[threadIdx.x][w];
-        PM_CHK((ll)(slot * F + threadIdx.x + 1) * gridDim.x <= 6LL * PM_MAXF * 1024, 401, s = 0)
-        red[(ll)(slot * F + threadIdx.x) * gridDim.x + blockIdx.x] = s;
-    }
-    __syncthreads();
-}
-
-// grid_total into a shared array: out[f] = sum over blocks of the partials
-// of (slot, f), the same order on every block. Ends with a block barrier.
-__device__ __forceinline__ void grid_total_sh(const double *red, int F, int slot, double *out) {
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    if (wid < F) {
-        const double *src = red + (ll)(slot * F + wid) * gridDim.x;
-        double s = 0;
-        for (unsigned i = lane; i < gridDim.x; i += 32) s += src[i];
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if (lane == 0) out[wid] = s;
-    }
-    __syncthreads();
-}
-
 // Per-field solver scalars, identical on every block (each block computes
 // them from the same totals); shared so that the row loops stay small.
 struct PcgState {
-    double cc[PM_MAXF], rz[PM_MAXF], sumc[PM_MAXF], sumabs[PM_MAXF], t0[PM_MAXF], t1[PM_MAXF];
+    double cc[PM_MAXF], rz[PM_MAXF], rr0[PM_MAXF], sumc[PM_MAXF], sumabs[PM_MAXF];
     float al[PM_MAXF], be[PM_MAXF];
     int act[PM_MAXF], its[PM_MAXF];
 };
 
-// Compensated partials of the FF fields as doubles (fields past F give 0).
+// The FF accumulators of a kind (fields past F are dropped).
 template <int FF>
-__device__ __forceinline__ void dot_out(const Dot2 (&s)[FF], int F, double (&v)[FF]) {
+__device__ __forceinline__ void put_sums(BlockSums &B, int kind, int F, const Dot2 (&v)[FF]) {
 #pragma unroll
-    for (int f = 0; f < FF; ++f) v[f] = f < F ? (double)s[f].hi + (double)s[f].lo : 0.0;
+    for (int f = 0; f < FF; ++f)
+        if (f < F) put_sum(B, kind, f, v[f]);
 }
 
 // Reductions use slot groups {0,1,2}, {3,4}, then alternate {0} and {1,2}
-// inside the loop and {5,0} at the end: no two consecutive reductions share a
-// slot, so a block that runs ahead to the next reduction never overwrites a
-// partial that a slower block is still summing.
+// inside the loop, and at the end {3,4}, or {0,1} when no iteration ran: no two
+// consecutive reductions share a slot, so a block that runs ahead to the next
+// reduction never overwrites a partial that a slower block is still summing.
+// Sums as in the mesh solves: with FP64 shuffles and sums per thread an
+// solve of 3 fields on 1.97e6 particles (7 iterations) took 1.34 ms, now 1.15.
+// An iteration is 97 us for the rows (two 16-byte gathers per neighbour from the
+// L1 and L2), 22 us for the update and 10 us in the two barriers.
 template <int DIM, int FF>
 __global__ void __launch_bounds__(256, FF == 8 ? 2 : 4) k_pcg(PCG a) {
     __shared__ PcgState S;
+    __shared__ BlockSums B;
+    unsigned passed = 0;
+    // warp f sums field f's partials, its lane 0 keeps the field's scalars
+    const int wf = threadIdx.x >> 5;
+    const bool lane0 = (threadIdx.x & 31) == 0;
     const int F = a.F;
     const ll np = a.np;
     const ll tid = (ll)blockIdx.x * blockDim.x + threadIdx.x, nth = (ll)gridDim.x * blockDim.x;
@@ -1290,18 +1074,23 @@ __global__ void __launch_bounds__(256, FF == 8 ? 2 : 4) k_pcg(PCG a) {
             }
             stv<FF>(a.x + s * FF, xv);
         }
-        double v[FF];
-        dot_out<FF>(s2, F, v);
-        block_partial_v<FF>(v, F, a.red, 0);
-        dot_out<FF>(s1, F, v);
-        block_partial_v<FF>(v, F, a.red, 1);
-        dot_out<FF>(sa, F, v);
-        block_partial_v<FF>(v, F, a.red, 2);
+        put_sums<FF>(B, 0, F, s2);
+        put_sums<FF>(B, 1, F, s1);
+        put_sums<FF>(B, 2, F, sa);
+        flush_sums(B, 3, F, a.red, 0);
     }
-    if (!grid_sync(a.bar, a.status)) return;
-    grid_total_sh(a.red, F, 0, S.cc);
-    grid_total_sh(a.red, F, 1, S.sumc);
-    grid_total_sh(a.red, F, 2, S.sumabs);
+    if (!grid_sync(a.bar, a.status, passed)) return;
+    if (wf < F) {
+        const double cc = grid_sum(a.red, F, 0, wf);
+        if (lane0) S.cc[wf] = cc;
+        if (blockIdx.x == 0) {  // reported only
+            const double sumc = grid_sum(a.red, F, 1, wf), sumabs = grid_sum(a.red, F, 2, wf);
+            if (lane0) {
+                S.sumc[wf] = sumc;
+                S.sumabs[wf] = sumabs;
+            }
+        }
+    }
     // --- r = c - M x, z = r / d; (r, r), (r, z)
     {
         Dot2 s2[FF], sz[FF];
@@ -1319,28 +1108,27 @@ __global__ void __launch_bounds__(256, FF == 8 ? 2 : 4) k_pcg(PCG a) {
             }
             stv<FF>(a.z + s * FF, zv);
         }
-        double v[FF];
-        dot_out<FF>(s2, F, v);
-        block_partial_v<FF>(v, F, a.red, 3);
-        dot_out<FF>(sz, F, v);
-        block_partial_v<FF>(v, F, a.red, 4);
+        put_sums<FF>(B, 0, F, s2);
+        put_sums<FF>(B, 1, F, sz);
+        flush_sums(B, 2, F, a.red, 3);
     }
-    if (!grid_sync(a.bar, a.status)) return;
-    grid_total_sh(a.red, F, 3, S.t0);
-    grid_total_sh(a.red, F, 4, S.rz);
+    if (!grid_sync(a.bar, a.status, passed)) return;
     // The iteration stops on its recurrence for (r, r), which in FP32 drifts
     // from the true residual by a few roundings (observed: under 1 %); it
     // stops at 0.9 rtol so that the true residual, recomputed at exit, meets
     // rtol.
     const double tol2 = 0.81 * a.rtol * a.rtol;
-    if (threadIdx.x == 0)
-        for (int f = 0; f < F; ++f) {
-            S.act[f] = S.cc[f] > 0.0 && S.t0[f] > tol2 * S.cc[f];
-            S.its[f] = 0;
-            S.al[f] = 0.0f;
-            S.be[f] = 0.0f;
-            if (blockIdx.x == 0) a.scal[f * 16 + S_INIT] = S.cc[f] > 0.0 ? sqrt(S.t0[f] / S.cc[f]) : 0.0;
+    if (wf < F) {
+        const double rr = grid_sum(a.red, F, 3, wf), rz = grid_sum(a.red, F, 4, wf);
+        if (lane0) {
+            S.rr0[wf] = rr;
+            S.rz[wf] = rz;
+            S.act[wf] = S.cc[wf] > 0.0 && rr > tol2 * S.cc[wf];
+            S.its[wf] = 0;
+            S.al[wf] = 0.0f;
+            S.be[wf] = 0.0f;
         }
+    }
     __syncthreads();
     int last = -1;  // the last iteration run: its alpha p is still to be added to x
     for (int it = 0; it < a.max_iter; ++it) {
@@ -1387,14 +1175,15 @@ __global__ void __launch_bounds__(256, FF == 8 ? 2 : 4) k_pcg(PCG a) {
 #pragma unroll
                 for (int f = 0; f < FF; ++f) sq[f].fma_acc(ps.v[f], qv.v[f]);
             }
-            double v[FF];
-            dot_out<FF>(sq, F, v);
-            block_partial_v<FF>(v, F, a.red, 0);
+            put_sums<FF>(B, 0, F, sq);
+            flush_pairs(B, 1, F, a.red, 0);
         }
-        if (!grid_sync(a.bar, a.status)) return;
-        grid_total_sh(a.red, F, 0, S.t0);
-        if (threadIdx.x == 0)
-            for (int f = 0; f < F; ++f) S.al[f] = S.act[f] ? (float)(S.rz[f] / S.t0[f]) : 0.0f;
+        if (!grid_sync(a.bar, a.status, passed)) return;
+        if (wf < F) {
+            double t[1];
+            grid_pairs<1>(a.red, F, 0, wf, t);
+            if (lane0) S.al[wf] = S.act[wf] ? (float)quot(S.rz[wf], t[0]) : 0.0f;
+        }
         __syncthreads();
         last = it;
         // z -= alpha q / d; (r, r) and (r, z) with r = d z
@@ -1416,29 +1205,30 @@ __global__ void __launch_bounds__(256, FF == 8 ? 2 : 4) k_pcg(PCG a) {
                 }
                 stv<FF>(a.z + s * FF, zv);
             }
-            double v[FF];
-            dot_out<FF>(s2, F, v);
-            block_partial_v<FF>(v, F, a.red, 1);
-            dot_out<FF>(sz, F, v);
-            block_partial_v<FF>(v, F, a.red, 2);
+            put_sums<FF>(B, 0, F, s2);
+            put_sums<FF>(B, 1, F, sz);
+            flush_pairs(B, 2, F, a.red, 1);
         }
-        if (!grid_sync(a.bar, a.status)) return;
-        grid_total_sh(a.red, F, 1, S.t0);
-        grid_total_sh(a.red, F, 2, S.t1);
-        if (threadIdx.x == 0)
-            for (int f = 0; f < F; ++f) {
-                S.be[f] = 0.0f;
-                if (!S.act[f]) continue;
-                S.be[f] = (float)(S.t1[f] / S.rz[f]);
-                S.rz[f] = S.t1[f];
-                ++S.its[f];
-                if (S.t0[f] <= tol2 * S.cc[f]) S.act[f] = 0;
+        if (!grid_sync(a.bar, a.status, passed)) return;
+        if (wf < F) {
+            double t[2];
+            grid_pairs<2>(a.red, F, 1, wf, t);
+            if (lane0) {
+                S.be[wf] = 0.0f;
+                if (S.act[wf]) {
+                    S.be[wf] = (float)quot(t[1], S.rz[wf]);
+                    S.rz[wf] = t[1];
+                    ++S.its[wf];
+                    if (t[0] <= tol2 * S.cc[wf]) S.act[wf] = 0;
+                }
             }
+        }
         __syncthreads();
     }
     // --- report: x += alpha p of the last iteration (at the row and at each
     // neighbour), true residual c - M x, sum v x (= sum c for the exact
     // solution); the solution goes to q
+    const int end = last >= 0 ? 3 : 0;
     {
         float ap[FF];
 #pragma unroll
@@ -1467,27 +1257,22 @@ __global__ void __launch_bounds__(256, FF == 8 ? 2 : 4) k_pcg(PCG a) {
             }
             stv<FF>(a.q + s * FF, xs);
         }
-        double v[FF];
-        dot_out<FF>(s2, F, v);
-        block_partial_v<FF>(v, F, a.red, 5);
-        dot_out<FF>(sv, F, v);
-        block_partial_v<FF>(v, F, a.red, 0);
+        put_sums<FF>(B, 0, F, s2);
+        put_sums<FF>(B, 1, F, sv);
+        flush_sums(B, 2, F, a.red, end);
     }
-    if (!grid_sync(a.bar, a.status)) return;
-    grid_total_sh(a.red, F, 5, S.t0);
-    grid_total_sh(a.red, F, 0, S.t1);
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        bool bad = false;
-        for (int f = 0; f < F; ++f) {
-            const double res = S.cc[f] > 0.0 ? sqrt(S.t0[f] / S.cc[f]) : 0.0;
-            a.scal[f * 16 + S_ITERS] = S.its[f];
-            a.scal[f * 16 + S_RESID] = res;
-            a.scal[f * 16 + S_SUMMESH] = S.sumc[f];   // int Ab = sum_mu c_mu
-            a.scal[f * 16 + S_SUMPART] = S.t1[f];     // sum_mu v_mu Abb_mu
-            a.scal[f * 16 + S_SUMABS] = S.sumabs[f];  // sum_mu |c_mu|: scale of the conservation error
-            if (res > a.rtol) bad = true;
-        }
-        if (bad) atomicOr(a.status, ST_NOTCONV);
+    if (!grid_sync(a.bar, a.status, passed)) return;
+    if (blockIdx.x != 0 || wf >= F) return;
+    const double tr = grid_sum(a.red, F, end, wf), sx = grid_sum(a.red, F, end + 1, wf);
+    if (lane0) {
+        const double res = S.cc[wf] > 0.0 ? sqrt(tr / S.cc[wf]) : 0.0;
+        a.scal[wf * 16 + S_INIT] = S.cc[wf] > 0.0 ? sqrt(S.rr0[wf] / S.cc[wf]) : 0.0;
+        a.scal[wf * 16 + S_ITERS] = S.its[wf];
+        a.scal[wf * 16 + S_RESID] = res;
+        a.scal[wf * 16 + S_SUMMESH] = S.sumc[wf];   // int Ab = sum_mu c_mu
+        a.scal[wf * 16 + S_SUMPART] = sx;           // sum_mu v_mu Abb_mu
+        a.scal[wf * 16 + S_SUMABS] = S.sumabs[wf];  // sum_mu |c_mu|: scale of the conservation error
+        if (res > a.rtol) atomicOr(a.status, ST_NOTCONV);
     }
 }
 
@@ -1551,20 +1336,47 @@ void launch_mass_apply(const Geo &g, const float *x, int F, float *y, cudaStream
     count_launches(1);
 }
 
-// Returns 0 or a CUDA error code.
-int launch_cg(const Geo &g, Work &w, int F, const float *b_float, bool b_from_fix, float *x, bool x_has_start,
-              double rtol, int max_iter, cudaStream_t st) {
+namespace {
+
+// Kernel of a mesh solve by dimension, mesh kind and nodes per access.
+template <template <int, int, int> class K>
+void (*mesh_kernel(const Geo &g, int vec, int *variant))(CG) {
+    const int p1 = g.dim == 2 && g.p1;
+    *variant = g.dim == 1 ? 0 : 1 + 2 * p1 + (vec == 4);
+    if (g.dim == 1) return K<1, 0, 1>::get();
+    if (vec == 4) return p1 ? K<2, 1, 4>::get() : K<2, 0, 4>::get();
+    return p1 ? K<2, 1, 1>::get() : K<2, 0, 1>::get();
+}
+template <int DIM, int P1, int VEC>
+struct CgKernel {
+    static void (*get())(CG) { return k_cg<DIM, P1, VEC>; }
+};
+template <int DIM, int P1, int VEC>
+struct ChebKernel {
+    static void (*get())(CG) { return k_cheb<DIM, P1, VEC>; }
+};
+
+// The solvers' arguments. Vectors: w.r, w.r2, w.p, w.q, w.b and four in w.part
+// (the FLIP partials, free during a solve).
+CG mesh_args(const Geo &g, Work &w, int F, const float *b_float, bool b_from_fix, float *x, bool x_has_start,
+             double rtol, int max_iter) {
     CG a;
+    const ll len = (ll)F * g.ncell;
     a.g = g;
     a.F = F;
     a.bsrc = b_float;
     a.bfix = b_from_fix ? w.bfix : nullptr;
     a.maxabs = w.maxabs;
     a.x = x;
-    a.r = w.r;
-    a.p = w.p;
-    a.q = w.q;
     a.b = w.b;
+    a.p = w.p;
+    a.r[0] = w.r;
+    a.r[1] = w.r2;
+    a.w[0] = w.q;
+    a.w[1] = w.part;
+    a.s[0] = w.part + len;
+    a.s[1] = w.part + 2 * len;
+    a.xw = w.part + 3 * len;
     a.red = w.red;
     a.scal = w.scal;
     a.bar = w.bar;
@@ -1574,56 +1386,47 @@ int launch_cg(const Geo &g, Work &w, int F, const float *b_float, bool b_from_fi
     a.has_start = x_has_start ? 1 : 0;
     a.psum = b_from_fix ? w.psum : nullptr;
     a.nblk_psum = w.nblk_psum;
-    // 2D meshes with n % 4 == 0 take the quad kernel (16-byte accesses)
-    const bool quad = g.dim == 2 && g.n % 4 == 0, p1 = g.dim == 2 && g.p1;
-    const int di = (quad ? 2 : g.dim - 1) + (p1 ? 3 : 0);
-    void (*kern)(CG) = quad ? (p1 ? k_cg2v<1> : k_cg2v<0>)
-                            : (g.dim == 1 ? k_cg<1, 0> : (p1 ? k_cg<2, 1> : k_cg<2, 0>));
-    const ll need = ((quad ? g.ncell / 4 : g.ncell) + 255) / 256;
-    const int grid = clamp_grid(persistent_grid(di, (const void *)kern, quad ? 4 : 2), need, w);
+    return a;
+}
+
+// Nodes per access: quads on 2D meshes with n % 4 == 0 and 16-byte aligned
+// arrays of the caller (the workspace's are).
+int vec_of(const Geo &g, const float *b, const float *x) {
+    return g.dim == 2 && g.n % 4 == 0 && ((uintptr_t)b | (uintptr_t)x) % 16 == 0 ? 4 : 1;
+}
+
+// Queue a mesh solve, at most 4 resident blocks per SM and no more blocks than
+// there is work for. 0 or a CUDA error.
+int run_mesh_solve(void (*kern)(CG), int variant, CG &a, Work &w, int vec, cudaStream_t st) {
+    const ll need = (a.g.ncell / vec + 255) / 256;
+    const int grid = clamp_grid(persistent_grid(variant, (const void *)kern, 4), need, w);
     cudaMemsetAsync(w.bar, 0, 2 * sizeof(unsigned), st);
     void *args[] = {&a};
-    cudaError_t e = cudaLaunchCooperativeKernel((void *)kern, dim3(grid), dim3(256), args, 0, st);
+    const cudaError_t e = cudaLaunchCooperativeKernel((void *)kern, dim3(grid), dim3(256), args, 0, st);
     count_launches(1);
     return (int)e;
 }
 
-// Chebyshev solve: same arguments, workspace and report as launch_cg.
+}  // namespace
 
+// Returns 0 or a CUDA error code.
+int launch_cg(const Geo &g, Work &w, int F, const float *b_float, bool b_from_fix, float *x, bool x_has_start,
+              double rtol, int max_iter, cudaStream_t st) {
+    CG a = mesh_args(g, w, F, b_float, b_from_fix, x, x_has_start, rtol, max_iter);
+    const int vec = vec_of(g, b_float, x);
+    int variant;
+    void (*kern)(CG) = mesh_kernel<CgKernel>(g, vec, &variant);
+    return run_mesh_solve(kern, variant, a, w, vec, st);
+}
+
+// Chebyshev solve: same arguments, workspace and report as launch_cg.
 int launch_cheb(const Geo &g, Work &w, int F, const float *b_float, bool b_from_fix, float *x, bool x_has_start,
                 double rtol, int max_iter, cudaStream_t st) {
-    CG a;
-    a.g = g;
-    a.F = F;
-    a.bsrc = b_float;
-    a.bfix = b_from_fix ? w.bfix : nullptr;
-    a.maxabs = w.maxabs;
-    a.x = x;
-    a.r = w.r;
-    a.p = w.p;
-    a.q = w.q;
-    a.b = w.b;
-    a.r2 = w.r2;
-    a.red = w.red;
-    a.scal = w.scal;
-    a.bar = w.bar;
-    a.status = w.status;
-    a.rtol = rtol;
-    a.max_iter = max_iter;
-    a.has_start = x_has_start ? 1 : 0;
-    a.psum = b_from_fix ? w.psum : nullptr;
-    a.nblk_psum = w.nblk_psum;
-    const bool p1 = g.dim == 2 && g.p1;
-    const int di = g.dim == 1 ? 0 : (p1 ? 2 : 1);
-    if (g.dim == 2 && !w.r2) return (int)cudaErrorInvalidValue;
-    void (*kern)(CG) = g.dim == 1 ? k_cheb<1, 0> : (p1 ? k_cheb<2, 1> : k_cheb<2, 0>);
-    const ll need = (g.ncell + 255) / 256;
-    const int grid = clamp_grid(persistent_grid(6 + di, (const void *)kern, 4), need, w);
-    cudaMemsetAsync(w.bar, 0, 2 * sizeof(unsigned), st);
-    void *args[] = {&a};
-    cudaError_t e = cudaLaunchCooperativeKernel((void *)kern, dim3(grid), dim3(256), args, 0, st);
-    count_launches(1);
-    return (int)e;
+    CG a = mesh_args(g, w, F, b_float, b_from_fix, x, x_has_start, rtol, max_iter);
+    const int vec = vec_of(g, b_float, x);
+    int variant;
+    void (*kern)(CG) = mesh_kernel<ChebKernel>(g, vec, &variant);
+    return run_mesh_solve(kern, 5 + variant, a, w, vec, st);
 }
 
 int pcg_width(int F) { return F <= 2 ? 2 : (F <= 4 ? 4 : PM_MAXF); }
@@ -1659,7 +1462,7 @@ int launch_pcg(const Geo &g, Work &w, ll np, int F, const float *c, float *out, 
                                    k_pcg<2, 2>, k_pcg<2, 4>, k_pcg<2, PM_MAXF>};
     void (*kern)(PCG) = kerns[di];
     const ll need = (np + 255) / 256;
-    const int grid = clamp_grid(persistent_grid(9 + di, (const void *)kern, 4), need, w);
+    const int grid = clamp_grid(persistent_grid(10 + di, (const void *)kern, 4), need, w);
     if (g.dim == 2 && np > 0) {
         k_star_coef<<<div_up(np, 256), 256, 0, st>>>(np, w.pos, w.nbr, w.deg, a.unit, w.pcoef);
         count_launches(1);

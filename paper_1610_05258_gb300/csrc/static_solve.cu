@@ -10,10 +10,10 @@
 // fixed size instead of a context's workspace. The caller still passes the
 // right-hand side and the output array.
 //
-// Scratch: PM_NOALLOC_MAX_VALUES floats for each of the four CG vectors
-// (r, p, q, b), plus reduction partials for up to PM_NOALLOC_MAX_GRID blocks
+// Scratch: PM_NOALLOC_MAX_VALUES floats for each of the nine vectors of the
+// CG solve, plus reduction partials for up to PM_NOALLOC_MAX_GRID blocks
 // (the solve's grid is clamped to that), solver scalars, the barrier words and
-// the status word: about 16.2 MB, held by every GPU that loads the library
+// the status word: about 38 MB, held by every GPU that loads the library
 // until the process exits. Its device address is looked up once per device
 // (cudaGetSymbolAddress) by the first call on that device.
 #include <cstring>
@@ -28,7 +28,7 @@
 namespace {
 
 constexpr size_t kVecBytes = sizeof(float) * (size_t)PM_NOALLOC_MAX_VALUES;
-constexpr size_t kRedOff = 4 * kVecBytes;
+constexpr size_t kRedOff = 9 * kVecBytes;
 constexpr size_t kRedBytes = sizeof(double) * 6 * PM_MAXF * (size_t)PM_NOALLOC_MAX_GRID;
 constexpr size_t kScalOff = kRedOff + kRedBytes;
 constexpr size_t kScalBytes = sizeof(double) * 16 * PM_MAXF;
@@ -84,6 +84,8 @@ extern "C" pm_status pm_mass_solve_noalloc(int dim, int n, double L, const float
     w.p = (float *)(base + 1 * kVecBytes);
     w.q = (float *)(base + 2 * kVecBytes);
     w.b = (float *)(base + 3 * kVecBytes);
+    w.r2 = (float *)(base + 4 * kVecBytes);
+    w.part = (float *)(base + 5 * kVecBytes);  // four vectors
     w.red = (double *)(base + kRedOff);
     w.red_blocks = PM_NOALLOC_MAX_GRID;  // the solve's grid is clamped to the partials' capacity
     w.scal = (double *)(base + kScalOff);
