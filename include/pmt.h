@@ -375,11 +375,10 @@ pm_status pm_net_features(pm_ctx *ctx, const float *px, const float *py, long lo
  * Batches of independent instances (no counterpart in the paper: many
  * periodic problems of uneven mesh and particle sizes advanced together).
  *
- * All instances share one packed workspace and every phase of a step (pack,
- * sort, stars, right-hand side, start, per-instance solve on a thread-block
- * cluster) is one launch over all instances (about 18 kernels per step in
- * total), captured
- * once into a CUDA graph and replayed while the arguments stay the same.
+ * All instances share one packed workspace and every phase of a step (sort,
+ * stars, right-hand side, start, the solve with a thread-block cluster for each
+ * field of an instance) is one launch over all instances (about 17 kernels per
+ * step in total), captured once into a CUDA graph and replayed while the arguments stay the same.
  * ------------------------------------------------------------------------- */
 typedef struct pm_batch pm_batch;
 /* ninst 2D instances; instance k has an n[k] x n[k] mesh of box length L[k]
@@ -387,15 +386,15 @@ typedef struct pm_batch pm_batch;
  * Allocates the packed workspace now. stream is the caller's stream the
  * batch synchronises with. tune: 0 = choose, on the first call, by timing
  * one step for each setting (the solve's threads per CTA and CTAs per
- * instance, instances packed as given or largest first), cached per device
+ * field of an instance, instances packed as given or largest first), cached per device
  * and size class for the process; 256, 512 or 1024 = that many threads, one
- * CTA per instance, instances as given. PM_EINVAL on any other value or an
+ * CTA per field, instances as given. PM_EINVAL on any other value or an
  * invalid instance. */
 pm_status pm_batch_create(pm_batch **out, int ninst, const int *n, const double *L, const long long *max_np,
                           int max_fields, int tune, void *stream);
 void pm_batch_destroy(pm_batch *b);
 const char *pm_batch_last_error(const pm_batch *b);
-/* The solve's setting: threads per CTA, CTAs per instance (a thread-block
+/* The solve's setting: threads per CTA, CTAs per field of an instance (a thread-block
  * cluster of 1, 4 or 8 that reduces through distributed shared memory),
  * instances packed largest first (1) or as given (0), and the step time
  * measured when the autotuner chose it (0 if not tuned). Outputs may be NULL. */

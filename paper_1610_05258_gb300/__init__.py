@@ -501,7 +501,7 @@ class Batch:
             self.h = None
 
     def tuning(self):
-        """(solve threads per CTA, CTAs per instance, packed largest first, step
+        """(solve threads per CTA, CTAs per field of an instance, packed largest first, step
         ms measured when tuning)."""
         th, cl, lf, ms = ctypes.c_int(0), ctypes.c_int(0), ctypes.c_int(0), ctypes.c_double(0.0)
         self.lib.pm_batch_tuning(self.h, ctypes.byref(th), ctypes.byref(cl), ctypes.byref(lf), ctypes.byref(ms))

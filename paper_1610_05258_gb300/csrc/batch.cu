@@ -7,8 +7,7 @@
 // batch (Sec. 2.4, Eqs. proj and phi_def, as pm_assign_mass with the exact
 // inverse as start) is
 //
-//   pack       caller arrays -> packed arrays                (per particle)
-//   sort       cell keys, one scan over all cells, canonical
+//   sort       caller arrays -> cell keys, one scan over all cells, canonical
 //              order, gather with max|A| per instance         (per particle / cell)
 //   stars      periodic Delaunay stars, two retry passes       (per particle)
 //   rhs        exact right-hand side                           (per 16x16-cell tile)
@@ -16,14 +15,14 @@
 //              or the delta assignment per particle, or zero)
 //   solve      mean mode, true residual, CG if it is not yet
 //              below rtol, conservation and stability report,
-//              result written to the caller's array             (one cluster per instance)
+//              result written to the caller's array             (a cluster per field)
 //
-// about 18 launches per step whatever the number of instances, captured once
+// about 17 launches per step whatever the number of instances, captured once
 // into a CUDA graph and replayed while the arguments stay the same. Tables
 // resolve a particle, cell or tile to its instance (binary search over the
 // offsets). The autotuner times one step for each candidate setting the first
 // time a batch of a given size class runs on a device and keeps the fastest:
-// the threads per CTA and the CTAs per instance (a thread-block cluster that
+// the threads per CTA and the CTAs per field of an instance (a cluster that
 // reduces through distributed shared memory) of the solve, and the packing
 // order of the instances (as given, or largest first so that the longest
 // solves start first).
@@ -44,35 +43,59 @@ namespace cg = cooperative_groups;
 
 namespace {
 
-// Cluster-wide sum of one double per thread (every thread of the cluster
-// receives it): warp shuffle tree, the warps' sums in index order, then the
-// CTAs' sums read from each CTA's shared memory (DSMEM) in rank order, so the
-// result is the same on every CTA and every run. slot[2] alternates between
-// calls: a CTA writes slot[ph] only after every CTA has passed the barrier of
-// the previous call, which follows its reads of slot[ph] two calls back.
-template <int NT, int CS>
-__device__ __forceinline__ double cluster_sum(double v, double *sh, double *slot, int &ph) {
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+// Cluster-wide sums of K accumulators (every thread of the cluster receives
+// them): compensated FP32 in the warp and over the CTA's warps, then FP64 over
+// the CTAs' sums, which warp 0 reads from each CTA's shared memory (DSMEM): the
+// same order on every CTA and every run. slot[2] alternates between calls: a CTA
+// writes slot[ph] only after every CTA has passed the barrier of the previous
+// call, which follows its reads of slot[ph] two calls back. FP64 shuffles and
+// sums in every thread held the FP64 pipe for 8000 cycles a sum and CTA; with
+// them, one sum at a time and 64-bit node indices the solves of 24 instances of
+// 64^2 to 512^2 nodes and 3 fields took 600 us, then 427, with a cluster for each
+// field of an instance and not for all of them 221.
+struct ClusterSums {
+    DotBits warp[3][32];
+    double slot[2][3], tot[3];
+};
+template <int NT, int CS, int K>
+__device__ __forceinline__ void cluster_sums(const Dot2 (&v)[K], double (&out)[K], ClusterSums &C, int &ph) {
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    __syncthreads();
-    if (lane == 0) sh[wid] = v;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double s = 0.0;
-        for (int k = 0; k < NT / 32; ++k) s += sh[k];
-        slot[ph] = s;
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        const Dot2 t = warp_total(v[k]);
+        if (lane == 0) C.warp[k][wid].set(t);
     }
-    double tot = 0.0;
-    if (CS == 1) {
-        __syncthreads();
-        tot = slot[ph];
-    } else {
+    __syncthreads();
+    if (wid == 0) {
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            const Dot2 t = warp_total(lane < NT / 32 ? C.warp[k][lane].get() : Dot2());
+            if (lane == 0) (CS == 1 ? C.tot : C.slot[ph])[k] = total(t);
+        }
+    }
+    if (CS > 1) {
         cg::cluster_group cl = cg::this_cluster();
         cl.sync();
-        for (int r = 0; r < CS; ++r) tot += *cl.map_shared_rank(&slot[ph], r);
+        if (wid == 0) {
+#pragma unroll
+            for (int k = 0; k < K; ++k) {
+                double t = lane < CS ? *cl.map_shared_rank(&C.slot[ph][k], lane) : 0.0;
+                for (int o = CS / 2; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+                if (lane == 0) C.tot[k] = t;
+            }
+        }
     }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < K; ++k) out[k] = C.tot[k];
     ph ^= 1;
-    return tot;
+}
+template <int NT, int CS>
+__device__ __forceinline__ double cluster_sum(const Dot2 &v, ClusterSums &C, int &ph) {
+    const Dot2 a[1] = {v};
+    double t[1];
+    cluster_sums<NT, CS, 1>(a, t, C, ph);
+    return t[0];
 }
 
 // Barrier over the instance's threads (the CTA, or its cluster), ordering
@@ -83,18 +106,6 @@ __device__ __forceinline__ void instance_sync() {
         __syncthreads();
     else
         cg::this_cluster().sync();
-}
-
-__global__ void k_pack(BTab t, const float *const *__restrict__ px, const float *const *__restrict__ py,
-                       const float *const *__restrict__ vals, int F, float *__restrict__ opx,
-                       float *__restrict__ opy, float *__restrict__ ovals) {
-    const ll j = (ll)blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= t.NP) return;
-    const int k = find_slot(t.poff, t.ninst, j);
-    const ll p0 = __ldg(t.poff + k), npk = __ldg(t.poff + k + 1) - p0, l = j - p0;
-    opx[j] = px[k][l];
-    opy[j] = py[k][l];
-    for (int f = 0; f < F; ++f) ovals[(ll)f * t.NP + j] = vals[k][(ll)f * npk + l];
 }
 
 struct SolveArgs {
@@ -116,18 +127,17 @@ struct SolveArgs {
     const unsigned char *deg;
 };
 
-// One cluster of CS CTAs per instance: the same steps as the grid-wide CG kernel on one
+// One cluster of CS CTAs per field of an instance: the steps of CG on one
 // mesh (power-of-two field scale, exact mean mode from sum b, true residual
 // with the compensated stencil, CG iterations only while it is above rtol),
 // then the conservation sums and the result in the caller's array.
 template <int NT, int CS>
 __global__ void __launch_bounds__(NT) k_batch_solve(SolveArgs a) {
-    __shared__ double sh[NT / 32];
-    __shared__ double slot[2];
+    __shared__ ClusterSums C;
     int ph = 0;
     const BTab &t = a.t;
-    // instance = cluster index; this CTA's threads take every CS-th chunk of NT
-    const int k = a.order[blockIdx.x / CS];
+    // cluster -> instance and field; this CTA's threads take every CS-th chunk of NT
+    const int k = a.order[blockIdx.x / CS / a.F], f = blockIdx.x / CS % a.F;
     const int rank = CS == 1 ? 0 : (int)(blockIdx.x % CS);
     const ll t0 = (ll)rank * NT + threadIdx.x, TS = (ll)NT * CS;
     const BInst I = t.inst[k];
@@ -136,158 +146,156 @@ __global__ void __launch_bounds__(NT) k_batch_solve(SolveArgs a) {
     const float c = I.h * I.h / 36.0f;
     const double hd = (double)I.h * I.h;
     const double tol2 = a.rtol * a.rtol;
-    bool bad = false;
-    for (int f = 0; f < a.F; ++f) {
-        const ll fo = (ll)f * t.NC + co;
-        const float *bf = a.b + fo;
-        float *xf = a.x + fo, *rf = a.r + fo, *pf = a.p + fo, *qf = a.q + fo;
-        // sums of b, |b| and the start
-        Dot2 sb, sa, sx;
+    const ll fo = (ll)f * t.NC + co;
+    const float *bf = a.b + fo;
+    float *xf = a.x + fo, *rf = a.r + fo, *pf = a.p + fo, *qf = a.q + fo;
+    // sums of b, |b| and the start
+    Dot2 s0[3];
+    for (ll i = t0; i < nn; i += TS) {
+        const float bv = bf[i];
+        s0[0].add(bv);
+        s0[1].add(fabsf(bv));
+        s0[2].add(xf[i]);
+    }
+    double m0[3];
+    cluster_sums<NT, CS, 3>(s0, m0, C, ph);
+    const float S = solve_scale(m0[1] / (double)nn);
+    const float shv = (float)((double)S * (m0[0] / ((double)nn * hd) - m0[2] / (double)nn));
+    // scaled start with the exact mean mode, scaled b (into q) and |S b|^2
+    Dot2 s2[2];
+    for (ll i = t0; i < nn; i += TS) {
+        xf[i] = xf[i] * S + shv;
+        const float bv = bf[i] * S;
+        qf[i] = bv;
+        s2[1].fma_acc(bv, bv);
+    }
+    instance_sync<CS>();
+    // r = S b - M x, p = r (q keeps S b until the first iteration)
+    auto residual = [&](bool set_p) {
+        Dot2 s;
         for (ll i = t0; i < nn; i += TS) {
-            const float bv = bf[i];
-            sb.add(bv);
-            sa.add(fabsf(bv));
-            sx.add(xf[i]);
+            float hi, lo;
+            stencil<2, 0>(xf, n, i, hi, lo);
+            const float rv = fmaf(-c, hi, qf[i]) - c * lo;
+            rf[i] = rv;
+            if (set_p) pf[i] = rv;
+            s.fma_acc(rv, rv);
         }
-        const double sumb = cluster_sum<NT, CS>((double)sb.hi + (double)sb.lo, sh, slot, ph);
-        const double suma = cluster_sum<NT, CS>((double)sa.hi + (double)sa.lo, sh, slot, ph);
-        const double sumx = cluster_sum<NT, CS>((double)sx.hi + (double)sx.lo, sh, slot, ph);
-        const float S = solve_scale(suma / (double)nn);
-        const float shv = (float)((double)S * (sumb / ((double)nn * hd) - sumx / (double)nn));
-        // scaled start with the exact mean mode, scaled b (into q) and |S b|^2
-        Dot2 s2;
-        for (ll i = t0; i < nn; i += TS) {
-            xf[i] = xf[i] * S + shv;
-            const float bv = bf[i] * S;
-            qf[i] = bv;
-            s2.fma_acc(bv, bv);
-        }
-        const double bb = cluster_sum<NT, CS>((double)s2.hi + (double)s2.lo, sh, slot, ph);
-        instance_sync<CS>();
-        // r = S b - M x, p = r (q keeps S b until the first iteration)
-        auto residual = [&](bool set_p) {
+        return s;
+    };
+    s2[0] = residual(true);
+    double m2[2];
+    cluster_sums<NT, CS, 2>(s2, m2, C, ph);
+    double rr = m2[0];
+    const double bb = m2[1];
+    const double init = bb > 0.0 ? sqrt(rr / bb) : 0.0;
+    int it = 0;
+    if (bb > 0.0 && rr > tol2 * bb) {
+        // conjugate gradients on the instance (q holds M p during the
+        // iterations; S b is rebuilt from b afterwards, the scale being an
+        // exact power of two)
+        for (it = 0; it < a.max_iter && rr > tol2 * bb; ++it) {
+            Dot2 pq;
+            for (ll i = t0; i < nn; i += TS) {
+                float hi, lo;
+                stencil<2, 0>(pf, n, i, hi, lo);
+                const float qv = c * hi + c * lo;
+                qf[i] = qv;
+                pq.fma_acc(pf[i], qv);
+            }
+            const double dpq = cluster_sum<NT, CS>(pq, C, ph);
+            if (!(dpq > 0.0)) break;
+            const float al = (float)(rr / dpq);
             Dot2 s;
             for (ll i = t0; i < nn; i += TS) {
-                float hi, lo;
-                stencil<2, 0>(xf, n, i, hi, lo);
-                const float rv = fmaf(-c, hi, qf[i]) - c * lo;
+                xf[i] = fmaf(al, pf[i], xf[i]);
+                const float rv = fmaf(-al, qf[i], rf[i]);
                 rf[i] = rv;
-                if (set_p) pf[i] = rv;
                 s.fma_acc(rv, rv);
             }
-            return cluster_sum<NT, CS>((double)s.hi + (double)s.lo, sh, slot, ph);
-        };
-        double rr = residual(true);
-        const double init = bb > 0.0 ? sqrt(rr / bb) : 0.0;
-        int it = 0;
-        if (bb > 0.0 && rr > tol2 * bb) {
-            // conjugate gradients on the instance (q holds M p during the
-            // iterations; S b is rebuilt from b afterwards, the scale being an
-            // exact power of two)
-            for (it = 0; it < a.max_iter && rr > tol2 * bb; ++it) {
-                Dot2 pq;
-                for (ll i = t0; i < nn; i += TS) {
-                    float hi, lo;
-                    stencil<2, 0>(pf, n, i, hi, lo);
-                    const float qv = c * hi + c * lo;
-                    qf[i] = qv;
-                    pq.fma_acc(pf[i], qv);
-                }
-                const double dpq = cluster_sum<NT, CS>((double)pq.hi + (double)pq.lo, sh, slot, ph);
-                if (!(dpq > 0.0)) break;
-                const float al = (float)(rr / dpq);
-                Dot2 s;
-                for (ll i = t0; i < nn; i += TS) {
-                    xf[i] = fmaf(al, pf[i], xf[i]);
-                    const float rv = fmaf(-al, qf[i], rf[i]);
-                    rf[i] = rv;
-                    s.fma_acc(rv, rv);
-                }
-                const double rn = cluster_sum<NT, CS>((double)s.hi + (double)s.lo, sh, slot, ph);
-                const float be = (float)(rn / rr);
-                rr = rn;
-                for (ll i = t0; i < nn; i += TS) pf[i] = fmaf(be, pf[i], rf[i]);
-                instance_sync<CS>();
-            }
-            // true residual against S b (rebuilt in q)
-            for (ll i = t0; i < nn; i += TS) qf[i] = bf[i] * S;
+            const double rn = cluster_sum<NT, CS>(s, C, ph);
+            const float be = (float)(rn / rr);
+            rr = rn;
+            for (ll i = t0; i < nn; i += TS) pf[i] = fmaf(be, pf[i], rf[i]);
             instance_sync<CS>();
-            rr = residual(false);
         }
-        // result, conservation and stability
-        const float inv = 1.0f / S;  // a power of two: exact
-        float *o = a.out[k] + (ll)f * nn;
-        Dot2 sxx, em;
-        for (ll i = t0; i < nn; i += TS) {
-            const float xv = xf[i] * inv;
-            o[i] = xv;
-            sxx.add(xv);
-        }
-        const double sum_mesh = cluster_sum<NT, CS>((double)sxx.hi + (double)sxx.lo, sh, slot, ph) * hd;
+        // true residual against S b (rebuilt in q)
+        for (ll i = t0; i < nn; i += TS) qf[i] = bf[i] * S;
         instance_sync<CS>();
-        if (a.report) {
-            for (ll i = t0; i < nn; i += TS) {
-                float hi, lo;
-                stencil<2, 0>(o, n, i, hi, lo);
-                em.fma_acc(o[i], hi);
-                em.fma_acc(o[i], lo);
-            }
-        }
-        const double emesh = cluster_sum<NT, CS>((double)em.hi + (double)em.lo, sh, slot, ph) * ((double)I.L / n) * ((double)I.L / n) / 36.0;
-        Dot2 pa, pb;
-        const float *vf = a.vals + (ll)f * t.NP;
-        for (ll s = p0 + t0; s < p1; s += TS) {
-            const float v = a.vol[s], y = vf[s];
-            pa.fma_acc(v, y);
-            pb.fma_acc(v, fabsf(y));
-        }
-        const double sp = cluster_sum<NT, CS>((double)pa.hi + (double)pa.lo, sh, slot, ph);
-        const double spa = cluster_sum<NT, CS>((double)pb.hi + (double)pb.lo, sh, slot, ph);
-        // int A^2 over the instance's owned triangles (A^T M_p A)
-        double ep = 0.0;
-        if (a.report) {
-            Dot2 e;
-            for (ll s = p0 + t0; s < p1; s += TS) {
-                const int m = a.deg[s];
-                if (m < 3) continue;
-                const uint2 Xp = a.pos[s];
-                int ida = a.nbr[(ll)(m - 1) * t.NP + s] & 0x0fffffff;
-                int ca = (unsigned)a.nbr[(ll)(m - 1) * t.NP + s] >> 28;
-                for (int kk = 0; kk < m; ++kk) {
-                    const int eb = a.nbr[(ll)kk * t.NP + s];
-                    const int idb = eb & 0x0fffffff, cb = (unsigned)eb >> 28;
-                    if (ida > s && idb > s) {
-                        const uint2 A = a.pos[ida], B = a.pos[idb];
-                        const ll ax = (ll)A.x + (ll)(ca / 3 - 1) * 4294967296LL - Xp.x;
-                        const ll ay = (ll)A.y + (ll)(ca % 3 - 1) * 4294967296LL - Xp.y;
-                        const ll bx = (ll)B.x + (ll)(cb / 3 - 1) * 4294967296LL - Xp.x;
-                        const ll by = (ll)B.y + (ll)(cb % 3 - 1) * 4294967296LL - Xp.y;
-                        const float w2 = (float)(ax * by - ay * bx) * 5.421010862427522e-20f;
-                        const float u = vf[s], v = vf[ida], z = vf[idb];
-                        e.fma_acc(w2, u * u + v * v + z * z + u * v + v * z + z * u);
-                    }
-                    ida = idb;
-                    ca = cb;
-                }
-            }
-            ep = cluster_sum<NT, CS>((double)e.hi + (double)e.lo, sh, slot, ph) * I.L * I.L / 12.0;
-        }
-        if (t0 == 0) {
-            double *r = a.scal + ((ll)k * PM_MAXF + f) * 16;
-            const double res = bb > 0.0 ? sqrt(rr / bb) : 0.0;
-            r[0] = it;
-            r[1] = init;
-            r[2] = res;
-            r[3] = sum_mesh;
-            r[4] = sp;
-            r[5] = spa;
-            r[6] = emesh;
-            r[7] = ep;
-            if (res > a.rtol) bad = true;
-        }
-        instance_sync<CS>();
+        rr = cluster_sum<NT, CS>(residual(false), C, ph);
     }
-    if (t0 == 0 && bad) atomicOr(a.status, ST_NOTCONV);
+    // result, conservation and stability
+    const float inv = 1.0f / S;  // a power of two: exact
+    float *o = a.out[k] + (ll)f * nn;
+    Dot2 se[3];  // result, v A, v |A|
+    for (ll i = t0; i < nn; i += TS) {
+        const float xv = xf[i] * inv;
+        o[i] = xv;
+        se[0].add(xv);
+    }
+    const float *vf = a.vals + (ll)f * t.NP;
+    for (ll s = p0 + t0; s < p1; s += TS) {
+        const float v = a.vol[s], y = vf[s];
+        se[1].fma_acc(v, y);
+        se[2].fma_acc(v, fabsf(y));
+    }
+    double me[3];
+    cluster_sums<NT, CS, 3>(se, me, C, ph);
+    double emesh = 0.0;
+    if (a.report) {
+        instance_sync<CS>();
+        Dot2 em;
+        for (ll i = t0; i < nn; i += TS) {
+            float hi, lo;
+            stencil<2, 0>(o, n, i, hi, lo);
+            em.fma_acc(o[i], hi);
+            em.fma_acc(o[i], lo);
+        }
+        emesh = cluster_sum<NT, CS>(em, C, ph) * ((double)I.L / n) * ((double)I.L / n) / 36.0;
+    }
+    // int A^2 over the instance's owned triangles (A^T M_p A)
+    double ep = 0.0;
+    if (a.report) {
+        Dot2 e;
+        for (ll s = p0 + t0; s < p1; s += TS) {
+            const int m = a.deg[s];
+            if (m < 3) continue;
+            const uint2 Xp = a.pos[s];
+            int ida = a.nbr[(ll)(m - 1) * t.NP + s] & 0x0fffffff;
+            int ca = (unsigned)a.nbr[(ll)(m - 1) * t.NP + s] >> 28;
+            for (int kk = 0; kk < m; ++kk) {
+                const int eb = a.nbr[(ll)kk * t.NP + s];
+                const int idb = eb & 0x0fffffff, cb = (unsigned)eb >> 28;
+                if (ida > s && idb > s) {
+                    const uint2 A = a.pos[ida], B = a.pos[idb];
+                    const ll ax = (ll)A.x + (ll)(ca / 3 - 1) * 4294967296LL - Xp.x;
+                    const ll ay = (ll)A.y + (ll)(ca % 3 - 1) * 4294967296LL - Xp.y;
+                    const ll bx = (ll)B.x + (ll)(cb / 3 - 1) * 4294967296LL - Xp.x;
+                    const ll by = (ll)B.y + (ll)(cb % 3 - 1) * 4294967296LL - Xp.y;
+                    const float w2 = (float)(ax * by - ay * bx) * 5.421010862427522e-20f;
+                    const float u = vf[s], v = vf[ida], z = vf[idb];
+                    e.fma_acc(w2, u * u + v * v + z * z + u * v + v * z + z * u);
+                }
+                ida = idb;
+                ca = cb;
+            }
+        }
+        ep = cluster_sum<NT, CS>(e, C, ph) * I.L * I.L / 12.0;
+    }
+    if (t0 == 0) {
+        double *r = a.scal + ((ll)k * PM_MAXF + f) * 16;
+        const double res = bb > 0.0 ? sqrt(rr / bb) : 0.0;
+        r[0] = it;
+        r[1] = init;
+        r[2] = res;
+        r[3] = me[0] * hd;
+        r[4] = me[1];
+        r[5] = me[2];
+        r[6] = emesh;
+        r[7] = ep;
+        if (res > a.rtol) atomicOr(a.status, ST_NOTCONV);
+    }
+    instance_sync<CS>();
 }
 
 }  // namespace
@@ -302,7 +310,6 @@ struct pm_batch {
     // packed workspace (sized for the sum of max_np and of n^2)
     Work w{};
     ll NPmax = 0, NC = 0;
-    float *in_px = nullptr, *in_py = nullptr, *in_vals = nullptr;
     BInst *d_inst = nullptr;
     ll *d_poff = nullptr, *d_coff = nullptr;
     int *d_rtile = nullptr, *d_dtile = nullptr, *d_order = nullptr;
@@ -317,7 +324,7 @@ struct pm_batch {
     int ntiles_rhs = 0, ntiles_dir = 0;
     // tuning
     int threads = 0;     // solve block threads (256, 512, 1024); 0 = autotune
-    int cluster = 1;     // CTAs per instance in the solve (a thread-block cluster of 1, 4 or 8)
+    int cluster = 1;     // CTAs per field of an instance in the solve (a thread-block cluster of 1, 4 or 8)
     int largest_first = 0;
     int start = PM_WS_DIRECT;  // start of the solves
     double tuned_ms = 0.0;
@@ -416,7 +423,7 @@ pm_status set_layout(pm_batch *b, const ll *np, int largest_first) {
     return PM_OK;
 }
 
-// Caller pointers in slot order (device tables read by pack and solve).
+// Caller pointers in slot order (device tables read by sort and solve).
 pm_status set_pointers(pm_batch *b, const float *const *px, const float *const *py, const float *const *vals,
                        float *const *out) {
     const int K = b->ninst;
@@ -448,9 +455,9 @@ SolveKernel solve_kernel(int threads, int cs) {
     return cs == 8 ? k_batch_solve<512, 8> : (cs == 4 ? k_batch_solve<512, 4> : k_batch_solve<512, 1>);
 }
 
-cudaLaunchConfig_t solve_config(int K, int threads, int cs, cudaStream_t st, cudaLaunchAttribute *attr) {
+cudaLaunchConfig_t solve_config(int clusters, int threads, int cs, cudaStream_t st, cudaLaunchAttribute *attr) {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(K * cs);
+    cfg.gridDim = dim3(clusters * cs);
     cfg.blockDim = dim3(threads);
     cfg.stream = st;
     attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -481,9 +488,7 @@ int enqueue_step(pm_batch *b, int F, double rtol, int max_iter, int report) {
     Work &w = b->w;
     cudaStream_t st = b->main;
     cudaMemsetAsync(w.status, 0, sizeof(int), st);
-    k_pack<<<div_up(t.NP, 256), 256, 0, st>>>(t, b->d_px, b->d_py, b->d_vals, F, b->in_px, b->in_py, b->in_vals);
-    count_launches(1);
-    launch_sort_batched(t, w, b->in_px, b->in_py, b->in_vals, F, st);
+    launch_sort_batched(t, w, b->d_px, b->d_py, b->d_vals, F, st);
     launch_triangulate_batched(t, w, st);
     launch_rhs_batched(t, w, F, b->d_rtile, b->ntiles_rhs, st);
     launch_rhs_to_float_batched(t, w, F, w.b, st);
@@ -515,7 +520,7 @@ int enqueue_step(pm_batch *b, int F, double rtol, int max_iter, int report) {
     a.deg = w.deg;
     const int K = b->ninst;
     cudaLaunchAttribute attr[1];
-    cudaLaunchConfig_t cfg = solve_config(K, b->threads, b->cluster, st, attr);
+    cudaLaunchConfig_t cfg = solve_config(K * F, b->threads, b->cluster, st, attr);
     cudaError_t e = cudaLaunchKernelEx(&cfg, solve_kernel(b->threads, b->cluster), a);
     count_launches(1);
     if (e != cudaSuccess) return (int)e;
@@ -563,7 +568,6 @@ pm_status pm_batch_create(pm_batch **out, int ninst, const int *n, const double 
          balloc(&w.nbr, (ll)PM_MAXDEG * NP) && balloc(&w.bfix, F * NC) && balloc(&w.b, F * NC) &&
          balloc(&w.r, F * NC) && balloc(&w.p, F * NC) && balloc(&w.q, F * NC) &&
          balloc(&w.scal, 16LL * PM_MAXF * ninst) && balloc(&w.status, 1) && balloc(&w.nretry, 2) &&
-         balloc(&b->in_px, NP) && balloc(&b->in_py, NP) && balloc(&b->in_vals, NP * F) &&
          balloc(&b->d_inst, ninst) && balloc(&b->d_poff, ninst + 1) && balloc(&b->d_coff, ninst + 1) &&
          balloc(&b->d_rtile, ninst + 1) && balloc(&b->d_dtile, ninst + 1) && balloc(&b->d_order, ninst) &&
          balloc((unsigned char **)&b->d_taps, (ll)direct_taps_bytes() * ninst) && balloc(&b->d_px, ninst) &&
@@ -595,7 +599,7 @@ void pm_batch_destroy(pm_batch *b) {
     void *ptrs[] = {w.fx,     w.key,      w.slot,     w.count,    w.cell_start, w.scan_tmp, w.tmp,
                     w.perm,   w.pos,      w.vals,     w.maxabs,   w.deg,        w.vol,      w.nbr,
                     w.bfix,   w.b,        w.r,        w.p,        w.q,          w.scal,     w.status,
-                    w.nretry, b->in_px,   b->in_py,   b->in_vals, b->d_inst,    b->d_poff,  b->d_coff,
+                    w.nretry, b->d_inst,    b->d_poff,  b->d_coff,
                     b->d_rtile, b->d_dtile, b->d_order, b->d_taps, (void *)b->d_px, (void *)b->d_py,
                     (void *)b->d_vals, (void *)b->d_out};
     for (void *p : ptrs)
@@ -664,7 +668,7 @@ pm_status pm_batch_assign_mass(pm_batch *b, const float *const *px, const float 
     cudaStreamWaitEvent(b->main, b->fork, 0);
     bool same_np = b->np.size() == (size_t)K && std::equal(b->np.begin(), b->np.end(), np);
     // autotune once per (device, size class): the solve's threads per CTA and
-    // CTAs per instance (cluster) x the packing order
+    // CTAs per field of an instance (cluster) x the packing order
     if (!b->fixed && b->threads == 0) {
         int dev = 0;
         cudaGetDevice(&dev);

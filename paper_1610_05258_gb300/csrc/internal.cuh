@@ -277,6 +277,42 @@ struct Dot2 {
 
 #endif
 
+// Accumulators summed with another one, and over the warp (lane 0), in the same
+// compensated form.
+__device__ __forceinline__ void join(Dot2 &a, const Dot2 &b) {
+#if defined(PM_FP64_SUMS)
+    a.hi += b.hi;
+#else
+    a.add(b.hi);
+#endif
+    a.lo += b.lo;
+}
+__device__ __forceinline__ Dot2 warp_total(Dot2 a) {
+    for (int o = 16; o > 0; o >>= 1) {
+        Dot2 b;
+        b.hi = __shfl_down_sync(0xffffffffu, a.hi, o);
+        b.lo = __shfl_down_sync(0xffffffffu, a.lo, o);
+        join(a, b);
+    }
+    return a;
+}
+__device__ __forceinline__ double total(const Dot2 &a) { return (double)a.hi + (double)a.lo; }
+// An accumulator as stored in shared memory (no constructor).
+struct DotBits {
+    decltype(Dot2::hi) hi;
+    float lo;
+    __device__ __forceinline__ void set(const Dot2 &a) {
+        hi = a.hi;
+        lo = a.lo;
+    }
+    __device__ __forceinline__ Dot2 get() const {
+        Dot2 a;
+        a.hi = hi;
+        a.lo = lo;
+        return a;
+    }
+};
+
 // Compensated M x at node i of field array xf; returns (hi, lo) of the
 // unscaled stencil sum; the caller multiplies by c = h/6, h^2/36 (bilinear)
 // or h^2/12 (P1: 6 at the node, 1 at its six neighbours along the cell
@@ -290,7 +326,7 @@ __device__ __forceinline__ void stencil(const float *__restrict__ xf, int n, ll 
         acc.add(xf[xm]);
         acc.add(xf[xp]);
     } else {
-        int ix = (int)(i % n), iy = (int)(i / n);
+        const int iy = (int)((unsigned)i / (unsigned)n), ix = (int)i - iy * n;  // n^2 < 2^31
         int xm = ix == 0 ? n - 1 : ix - 1, xp = ix + 1 == n ? 0 : ix + 1;
         int ym = iy == 0 ? n - 1 : iy - 1, yp = iy + 1 == n ? 0 : iy + 1;
         const float *r0 = xf + (ll)ym * n, *r1 = xf + (ll)iy * n, *r2 = xf + (ll)yp * n;
@@ -413,7 +449,8 @@ void launch_energies(const Geo &g, Work &w, int F, const float *mesh, ll np, con
                      cudaStream_t st);
 // Batched phases (one launch each over all instances of a BTab; the Work
 // holds the packed arrays, sized for NP particles and NC cells).
-void launch_sort_batched(const BTab &t, Work &w, const float *px, const float *py, const float *vals, int F,
+void launch_sort_batched(const BTab &t, Work &w, const float *const *px, const float *const *py,
+                         const float *const *vals, int F,
                          cudaStream_t st);
 void launch_triangulate_batched(const BTab &t, Work &w, cudaStream_t st);
 // tile_start [ninst + 1]: prefix of the instances' right-hand-side tiles.

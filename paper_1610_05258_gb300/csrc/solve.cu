@@ -89,27 +89,6 @@ __device__ bool grid_sync(unsigned *bar, int *status, unsigned &passed) {
     return ok != 0;
 }
 
-// Accumulators summed with another one, and over the warp (lane 0), in the same
-// compensated form.
-__device__ __forceinline__ void join(Dot2 &a, const Dot2 &b) {
-#if defined(PM_FP64_SUMS)
-    a.hi += b.hi;
-#else
-    a.add(b.hi);
-#endif
-    a.lo += b.lo;
-}
-__device__ __forceinline__ Dot2 warp_total(Dot2 a) {
-    for (int o = 16; o > 0; o >>= 1) {
-        Dot2 b;
-        b.hi = __shfl_down_sync(0xffffffffu, a.hi, o);
-        b.lo = __shfl_down_sync(0xffffffffu, a.lo, o);
-        join(a, b);
-    }
-    return a;
-}
-__device__ __forceinline__ double total(const Dot2 &a) { return (double)a.hi + (double)a.lo; }
-
 // A sum over the grid goes through red[(slot + kind) * F + f][block]: every
 // thread puts its accumulator (the warp's total goes to shared memory), the block
 // flushes, and after a grid barrier every block sums the partials in the same
@@ -120,19 +99,21 @@ __device__ __forceinline__ double total(const Dot2 &a) { return (double)a.hi + (
 // warp, and with the FP64 sums and divisions an iteration of one block took
 // 7500 cycles, of 64 blocks 14000; now 5200 and 10000, 2250 of them the barrier.
 struct BlockSums {
-    Dot2 v[3][PM_MAXF][8];
+    DotBits v[3][PM_MAXF][8];
 };
 __device__ __forceinline__ void put_sum(BlockSums &B, int kind, int f, const Dot2 &a) {
     const Dot2 t = warp_total(a);
-    if ((threadIdx.x & 31) == 0) B.v[kind][f][threadIdx.x >> 5] = t;
+    if ((threadIdx.x & 31) == 0) B.v[kind][f][threadIdx.x >> 5].set(t);
 }
 __device__ __forceinline__ void flush_sums(const BlockSums &B, int kinds, int F, double *red, int slot) {
     __syncthreads();
     const int t = threadIdx.x;
     if (t < kinds * F) {
-        const Dot2 *v = B.v[t / F][t % F];
-        red[(ll)(slot * F + t) * gridDim.x + blockIdx.x] = ((total(v[0]) + total(v[1])) + (total(v[2]) + total(v[3]))) +
-                                                           ((total(v[4]) + total(v[5])) + (total(v[6]) + total(v[7])));
+        double v[8];
+#pragma unroll
+        for (int w = 0; w < 8; ++w) v[w] = total(B.v[t / F][t % F][w].get());
+        red[(ll)(slot * F + t) * gridDim.x + blockIdx.x] =
+            ((v[0] + v[1]) + (v[2] + v[3])) + ((v[4] + v[5]) + (v[6] + v[7]));
     }
 }
 // Total of (slot, f) over all blocks, by one warp.
@@ -167,12 +148,12 @@ __device__ __forceinline__ void flush_pairs(const BlockSums &B, int kinds, int F
     __syncthreads();
     const int t = threadIdx.x;
     if (t < kinds * F) {
-        const Dot2 *v = B.v[t / F][t % F];
-        Dot2 a = v[0], b = v[4];
+        const DotBits *v = B.v[t / F][t % F];
+        Dot2 a = v[0].get(), b = v[4].get();
 #pragma unroll
         for (int w = 1; w < 4; ++w) {
-            join(a, v[w]);
-            join(b, v[w + 4]);
+            join(a, v[w].get());
+            join(b, v[w + 4].get());
         }
         join(a, b);
         red[(ll)(slot * F + t) * gridDim.x + blockIdx.x] = pack(a);
@@ -233,7 +214,6 @@ __device__ __forceinline__ Q4 ld4(const float *p) {
     const float4 t = *(const float4 *)p;
     return Q4{{t.x, t.y, t.z, t.w}};
 }
-__device__ __forceinline__ void st4(float *p, const Q4 &q) { *(float4 *)p = make_float4(q.v[0], q.v[1], q.v[2], q.v[3]); }
 
 // VEC consecutive nodes of a row (VEC = 4: 16-byte accesses, n % 4 == 0).
 template <int VEC>
