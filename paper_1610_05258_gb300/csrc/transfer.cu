@@ -1099,51 +1099,71 @@ __global__ void k_features(Geo g, int F, const float *__restrict__ delta, const 
     }
 }
 
-// Relative residual of the delta start per field, ||b - M delta|| / ||b||,
-// from the network's input channels: channel 1 is PM_NET_RSCALE r / (h^2
-// max|A|); b is read from its fixed point. FP64 block partials [2F][nblk]
-// (sum r^2, sum b^2, both in units of (h^2 max|A|)^2), reduced by
-// k_start_resid_final into out[f].
-__global__ void __launch_bounds__(256) k_start_resid(Geo g, int F, const float *__restrict__ feat,
-                                                      const ll *__restrict__ bfix, const unsigned *__restrict__ maxabs,
-                                                      double *__restrict__ part) {
-    __shared__ double sh[2 * PM_MAXF][8];
-    const float hd = g.h * g.h;
-    double acc[2 * PM_MAXF];
-    for (int k = 0; k < 2 * F; ++k) acc[k] = 0.0;
-    for (ll i = (ll)blockIdx.x * blockDim.x + threadIdx.x; i < g.ncell; i += (ll)gridDim.x * blockDim.x) {
-        for (int f = 0; f < F; ++f) {
-            const float s = __uint_as_float(maxabs[f]);
-            const float inv = s > 0.0f ? 1.0f / (s * hd) : 0.0f;
-            const double r = (double)feat[((ll)f * 2 + 1) * g.ncell + i] * (1.0 / PM_NET_RSCALE);
-            const double b = (double)(ldexpf((float)bfix[(ll)f * g.ncell + i], -fix_exp(maxabs, f, hd)) * inv);
-            acc[2 * f] += r * r;
-            acc[2 * f + 1] += b * b;
-        }
+// Block totals of two sums into part[2 f] and part[2 f + 1] (field f =
+// blockIdx.y, a column per block).
+__device__ __forceinline__ void pair_partial(double a, double b, double *part) {
+    __shared__ double sh[2][8];
+    double v[2] = {a, b};
+    for (int o = 16; o > 0; o >>= 1) {
+        v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+        v[1] += __shfl_xor_sync(0xffffffffu, v[1], o);
     }
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    for (int k = 0; k < 2 * F; ++k) {
-        double v = acc[k];
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        if (lane == 0) sh[k][wid] = v;
+    if ((threadIdx.x & 31) == 0) {
+        sh[0][threadIdx.x >> 5] = v[0];
+        sh[1][threadIdx.x >> 5] = v[1];
     }
     __syncthreads();
-    if (threadIdx.x < 2 * F) {
-        double v = 0.0;
-        for (int w = 0; w < 8; ++w) v += sh[threadIdx.x][w];
-        part[(ll)threadIdx.x * gridDim.x + blockIdx.x] = v;
+    if (threadIdx.x < 2) {
+        const double *q = sh[threadIdx.x];
+        part[(ll)(2 * blockIdx.y + threadIdx.x) * gridDim.x + blockIdx.x] =
+            ((q[0] + q[1]) + (q[2] + q[3])) + ((q[4] + q[5]) + (q[6] + q[7]));
     }
 }
 
-__global__ void k_start_resid_final(int F, int nblk, const double *__restrict__ part, double *__restrict__ out) {
-    const int f = threadIdx.x;
-    if (f >= F) return;
-    double rr = 0.0, bb = 0.0;
-    for (int b = 0; b < nblk; ++b) {
-        rr += part[(ll)(2 * f) * nblk + b];
-        bb += part[(ll)(2 * f + 1) * nblk + b];
+// Totals of the two rows of field f = threadIdx.x / 32, by one warp.
+__device__ __forceinline__ void pair_total(const double *part, int nblk, double &a, double &b) {
+    const int f = threadIdx.x >> 5;
+    const double *pa = part + (ll)(2 * f) * nblk, *pb = pa + nblk;
+    a = b = 0.0;
+    for (int i = threadIdx.x & 31; i < nblk; i += 32) {
+        a += pa[i];
+        b += pb[i];
     }
-    out[f] = bb > 0.0 ? sqrt(rr / bb) : 0.0;
+    for (int o = 16; o > 0; o >>= 1) {
+        a += __shfl_xor_sync(0xffffffffu, a, o);
+        b += __shfl_xor_sync(0xffffffffu, b, o);
+    }
+}
+
+// Relative residual of the delta start per field, ||b - M delta|| / ||b||,
+// from the network's input channels: channel 1 is PM_NET_RSCALE r / (h^2
+// max|A|); b is read from its fixed point. Partials (sum r^2, sum b^2, both in
+// units of (h^2 max|A|)^2), reduced by k_start_resid_final into out[f]. The
+// values are of order one and the products exact pairs (an FP64 instruction
+// costs 64 times an FP32 one). One thread per field over the blocks' partials
+// made the final kernels longer than the passes: 1024^2, 4 fields, 50 MB took 67 +
+// 73 us here and 53 + 74 us for k_alpha_partial and its final; now 34 + 9 and 47 + 9 us.
+__global__ void __launch_bounds__(256) k_start_resid(Geo g, const float *__restrict__ feat,
+                                                      const ll *__restrict__ bfix, const unsigned *__restrict__ maxabs,
+                                                      double *__restrict__ part) {
+    const float hd = g.h * g.h;
+    const int f = blockIdx.y, E = fix_exp(maxabs, f, hd);
+    const float s = __uint_as_float(maxabs[f]);
+    const float inv = s > 0.0f ? 1.0f / (s * hd) : 0.0f;
+    Dot2 rr, bb;
+    for (ll i = (ll)blockIdx.x * blockDim.x + threadIdx.x; i < g.ncell; i += (ll)gridDim.x * blockDim.x) {
+        const float r = feat[((ll)f * 2 + 1) * g.ncell + i];
+        const float b = ldexpf((float)bfix[(ll)f * g.ncell + i], -E) * inv;
+        rr.fma_acc(r, r);
+        bb.fma_acc(b, b);
+    }
+    pair_partial((double)rr.hi + (double)rr.lo, (double)bb.hi + (double)bb.lo, part);
+}
+
+__global__ void k_start_resid_final(int nblk, const double *__restrict__ part, double *__restrict__ out) {
+    double rr, bb;
+    pair_total(part, nblk, rr, bb);
+    if ((threadIdx.x & 31) == 0) out[threadIdx.x >> 5] = bb > 0.0 ? sqrt(rr / bb) * (1.0 / PM_NET_RSCALE) : 0.0;
 }
 
 // Step length of the network's correction. With r0 = b - M delta (feature
@@ -1153,52 +1173,31 @@ __global__ void k_start_resid_final(int F, int nblk, const double *__restrict__ 
 //   alpha = <r0, M c> / <M c, M c> = 36 <feat1, S corr> / <S corr, S corr>
 // (M = h^2/36 S, S the 9-point stencil 1-4-1 x 1-4-1). alpha = 0 keeps the
 // delta start, so the network can never make the start worse than delta in
-// this norm. Per-block FP64 partials, then one fixed-order reduction.
+// this norm. Per-block partials, then one fixed-order reduction.
 #define ALPHA_BLOCKS 608
-__global__ void __launch_bounds__(256) k_alpha_partial(Geo g, int F, const float *__restrict__ feat,
+__global__ void __launch_bounds__(256) k_alpha_partial(Geo g, const float *__restrict__ feat,
                                                         const float *__restrict__ corr, double *__restrict__ part) {
-    __shared__ double sh[2 * PM_MAXF][8];
-    const int n = g.n;
-    double acc[2 * PM_MAXF];
-    for (int k = 0; k < 2 * F; ++k) acc[k] = 0.0;
+    const int n = g.n, f = blockIdx.y;
+    const float *c = corr + (ll)f * g.ncell, *f1 = feat + ((ll)f * 2 + 1) * g.ncell;
+    double num = 0.0, den = 0.0;  // FP64 per node: a network's output has any range
     for (ll i = (ll)blockIdx.x * blockDim.x + threadIdx.x; i < g.ncell; i += (ll)gridDim.x * blockDim.x) {
-        const int ix = (int)(i % n), iy = (int)(i / n);
+        const int iy = (int)((unsigned)i / (unsigned)n), ix = (int)i - iy * n;
         const int xm = ix == 0 ? n - 1 : ix - 1, xp = ix + 1 == n ? 0 : ix + 1;
         const int ym = iy == 0 ? n - 1 : iy - 1, yp = iy + 1 == n ? 0 : iy + 1;
-        for (int f = 0; f < F; ++f) {
-            const float *c = corr + (ll)f * g.ncell;
-            const float *r0 = c + (ll)ym * n, *r1 = c + (ll)iy * n, *r2 = c + (ll)yp * n;
-            const float z = 16.0f * r1[ix] + 4.0f * (r1[xm] + r1[xp] + r0[ix] + r2[ix]) +
-                            (r0[xm] + r0[xp] + r2[xm] + r2[xp]);
-            const float f1 = feat[((ll)f * 2 + 1) * g.ncell + i];
-            acc[2 * f] += (double)f1 * (double)z;
-            acc[2 * f + 1] += (double)z * (double)z;
-        }
+        const float *r0 = c + (ll)ym * n, *r1 = c + (ll)iy * n, *r2 = c + (ll)yp * n;
+        const float z = 16.0f * r1[ix] + 4.0f * (r1[xm] + r1[xp] + r0[ix] + r2[ix]) +
+                        (r0[xm] + r0[xp] + r2[xm] + r2[xp]);
+        num += (double)f1[i] * (double)z;
+        den += (double)z * (double)z;
     }
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    for (int k = 0; k < 2 * F; ++k) {
-        double v = acc[k];
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        if (lane == 0) sh[k][wid] = v;
-    }
-    __syncthreads();
-    if (threadIdx.x < 2 * F) {
-        double v = 0.0;
-        for (int w = 0; w < 8; ++w) v += sh[threadIdx.x][w];
-        part[(ll)threadIdx.x * gridDim.x + blockIdx.x] = v;
-    }
+    pair_partial(num, den, part);
 }
 
-__global__ void k_alpha_final(int F, int nblk, const double *__restrict__ part, double *__restrict__ alpha) {
-    const int f = threadIdx.x;
-    if (f >= F) return;
-    double num = 0.0, den = 0.0;
-    for (int b = 0; b < nblk; ++b) {
-        num += part[(ll)(2 * f) * nblk + b];
-        den += part[(ll)(2 * f + 1) * nblk + b];
-    }
+__global__ void k_alpha_final(int nblk, const double *__restrict__ part, double *__restrict__ alpha) {
+    double num, den;
+    pair_total(part, nblk, num, den);
     const double a = den > 0.0 ? 36.0 * num / den : 0.0;
-    alpha[f] = isfinite(a) ? a : 0.0;
+    if ((threadIdx.x & 31) == 0) alpha[threadIdx.x >> 5] = isfinite(a) ? a : 0.0;
 }
 
 // Warm start: mesh = delta + alpha_f (max|A_f| / PM_NET_RSCALE) * network output.
@@ -1290,16 +1289,18 @@ void launch_features(const Geo &g, Work &w, int F, const float *delta, cudaStrea
 
 void launch_start_resid(const Geo &g, Work &w, int F, double *out, cudaStream_t st) {
     double *part = w.red;  // the solver's reduction buffer (the solve has not started yet)
-    k_start_resid<<<ALPHA_BLOCKS, 256, 0, st>>>(g, F, w.feat, w.bfix, w.maxabs, part);
-    k_start_resid_final<<<1, 32, 0, st>>>(F, ALPHA_BLOCKS, part, out);
+    const int nblk = std::min(ALPHA_BLOCKS, div_up(g.ncell, 256));
+    k_start_resid<<<dim3(nblk, F), 256, 0, st>>>(g, w.feat, w.bfix, w.maxabs, part);
+    k_start_resid_final<<<1, 32 * F, 0, st>>>(nblk, part, out);
     count_launches(2);
 }
 
 void launch_apply_correction(const Geo &g, Work &w, int F, float *mesh, cudaStream_t st) {
     // scratch: the solver's reduction buffer (the solve has not started yet)
     double *part = w.red, *alpha = w.red + 2LL * PM_MAXF * ALPHA_BLOCKS;
-    k_alpha_partial<<<ALPHA_BLOCKS, 256, 0, st>>>(g, F, w.feat, w.corr, part);
-    k_alpha_final<<<1, 32, 0, st>>>(F, ALPHA_BLOCKS, part, alpha);
+    const int nblk = std::min(ALPHA_BLOCKS, div_up(g.ncell, 256));
+    k_alpha_partial<<<dim3(nblk, F), 256, 0, st>>>(g, w.feat, w.corr, part);
+    k_alpha_final<<<1, 32 * F, 0, st>>>(nblk, part, alpha);
     k_apply_corr<<<div_up(g.ncell, 256), 256, 0, st>>>(g, F, w.corr, w.maxabs, alpha, mesh);
     count_launches(3);
 }
