@@ -309,22 +309,25 @@ def run_reference(args):
 # ---------------------------------------------------------------------------
 # Roofline of the triangulation (the dominant kernel of the 2D steps): it is
 # bound by ALU issue, not by memory. Its algorithmic operation count per
-# launch is the arithmetic of the clipping algorithm on the actual particle
-# set: the kernel's counting build (pm_profile mode 2) counts, over all
-# particles, the candidates examined, the candidates passing the distance
-# bound, the in-circle vertex tests, the clips and the cell sizes after each
-# clip; each is weighted by the FP32/INT32 arithmetic instructions of that
-# step as written (an FMA counts as one): distance test 10, margin set-up 5,
-# vertex test 5, clip with two circumcentres and error bounds 80, radius bound
-# 9 per vertex. Divergence, address arithmetic, loads and stores are not
-# counted.
+# launch is the arithmetic of building the stars on the actual particle set:
+# the kernels' counting build (pm_profile mode 2) counts, over all particles,
+# the candidates examined, the candidates passing the distance bound, the
+# tests of a candidate against a hull edge or cell vertex, the insertions into
+# a star (clips) and the star sizes after each; each is weighted by the
+# FP32/INT32 arithmetic instructions of that step in the exact clipping passes
+# (an FMA counts as one): distance test 10, margin set-up 5, vertex test 5,
+# clip with two circumcentres and error bounds 80, radius bound 9 per vertex.
+# The hull passes, which build most stars, insert with less than that, so the
+# count is an upper estimate for them. Divergence, address arithmetic, loads
+# and stores are not counted.
 DELAUNAY_OP_WEIGHTS = {"candidates": 10, "tested": 5, "vertex_tests": 5, "clips": 80, "cell_size_sum": 9}
 # ALU peak: 152 SMs x 128 FP32 lanes x one instruction per lane per clock.
 ALU_LANES = 152 * 128
 # DRAM traffic of one k_delaunay launch per particle: dram__bytes_read.sum +
 # dram__bytes_write.sum of one ncu capture on the 1024^2 mixture (4,194,304
 # particles: 100.11 MB read + 106.89 MB written), scaled to a launch by its
-# particle count (the kernel's traffic grows in proportion to it).
+# particle count (the kernel's traffic grows in proportion to it). The capture
+# is of the clipping main pass; the hull pass moves 216 MB there.
 DELAUNAY_DRAM_BYTES_PER_PARTICLE = (100.109568e6 + 106.889216e6) / 4194304
 
 
