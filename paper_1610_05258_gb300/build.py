@@ -51,7 +51,7 @@ def build(force: bool = False, verbose: bool = False, variant: str = "") -> str:
     flags = FLAGS + VARIANTS[variant]
     os.makedirs(out, exist_ok=True)
     srcs = sorted(glob.glob(os.path.join(CSRC, "*.cu")))
-    headers = sorted(glob.glob(os.path.join(CSRC, "*.cuh"))) + [os.path.join(ROOT, "include", "pmt.h")]
+    headers = sorted(glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(CSRC, "*.h"))) + [os.path.join(ROOT, "include", "pmt.h")]
     nvcc = _nvcc()
     jobs = []
     objs = []

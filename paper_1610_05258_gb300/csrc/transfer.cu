@@ -10,6 +10,7 @@
 // 64-bit fixed-point integers (2^E scaled, E from max |A| per field), whose
 // sum does not depend on the order of the atomic additions.
 #include "internal.cuh"
+#include "pack.h"
 
 #define PM_VIRT_LIMIT 0x0ffffff0
 
@@ -554,13 +555,14 @@ struct TriQ {
 
 // What the pieces of a triangle share, for the 32 triangles at work: p's offset
 // in its cell, the reciprocals of the edge vectors' components, 1 / (twice the
-// area), p's cell (x | y << 16), the box corner relative to it (the same) and
+// area), p's cell, the box corner relative to it and
 // the box width; for up to 4 fields also A at p and its gradient.
 template <int FF, int MODE>
 struct TriD {
     static constexpr int NG = MODE == 0 && FF <= 4 ? FF : 1;
     float us[32], ws[32], rx[3][32], ry[3][32], idet[32];
-    int cell[32], box[32], w[32];
+    unsigned cell[32], box[32];  // packed (pack.h)
+    int w[32];
     float a0[NG][32], gx[NG][32], gy[NG][32];
 };
 
@@ -728,8 +730,8 @@ __device__ __forceinline__ void rhs2d_tile(const Geo &g, ll np, const uint2 *__r
                 D.rx[2][lane] = __frcp_rn(us - vx2);
                 D.ry[2][lane] = __frcp_rn(ws - vy2);
                 D.idet[lane] = idet;
-                D.cell[lane] = cell_of(Xt.x, n) | (cell_of(Xt.y, n) << 16);
-                D.box[lane] = (bi & 0xffff) | (bj << 16);
+                D.cell[lane] = pack_cell(cell_of(Xt.x, n), cell_of(Xt.y, n));
+                D.box[lane] = pack_offset(bi, bj);
                 D.w[lane] = w;
                 if (GRAD) {
                     const int ta = Q.a[lane], tb = Q.b[lane];
@@ -764,10 +766,11 @@ __device__ __forceinline__ void rhs2d_tile(const Geo &g, ll np, const uint2 *__r
                 if (j >= T_all) continue;
                 const float us = D.us[src], ws = D.ws[src];
                 const float vx1 = Q.ax[src], vy1 = Q.ay[src], vx2 = Q.bx[src], vy2 = Q.by[src];
-                const int box = D.box[src], cell = D.cell[src], wdt = D.w[src];
+                const unsigned box = D.box[src], cell = D.cell[src];
+                const int wdt = D.w[src];
                 // rem / wdt, exact in float for fewer than 2^21 pieces
                 const int row = rem < (1 << 21) ? (int)(((float)rem + 0.5f) * __frcp_rn((float)wdt)) : rem / wdt;
-                const int ci = (int)(short)(box & 0xffff) + (rem - row * wdt), cj = (box >> 16) + row;
+                const int ci = offset_x(box) + (rem - row * wdt), cj = offset_y(box) + row;
                 const float fci = (float)ci, fcj = (float)cj;
                 const float xmin = fminf(us, fminf(vx1, vx2)), xmax = fmaxf(us, fmaxf(vx1, vx2));
                 const float ymin = fminf(ws, fminf(vy1, vy2)), ymax = fmaxf(ws, fmaxf(vy1, vy2));
@@ -784,7 +787,7 @@ __device__ __forceinline__ void rhs2d_tile(const Geo &g, ll np, const uint2 *__r
                 float K0[4], K1[4], K2[4];
                 corner_integrals<P1>(Mm, tx, ty, ox, oy, K0, K1, K2);
                 const float idet = D.idet[src], dsx = ox + fci - us, dty = oy + fcj - ws;
-                const int gcx = (cell & 0xffff) + ci, gcy = (cell >> 16) + cj;  // unwrapped cell
+                const int gcx = cell_x(cell) + ci, gcy = cell_y(cell) + cj;  // unwrapped cell
                 if (MODE == 1) {
                     // W_k[f] = sum over corners of Ab_c * (K0, K1, K2)_c
                     float W0[FF], W1[FF], W2[FF];
