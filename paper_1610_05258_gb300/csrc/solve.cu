@@ -25,6 +25,8 @@
 // on large ones.
 #include <cooperative_groups.h>
 
+#include <algorithm>
+#include <cmath>
 #include <mutex>
 
 #include "internal.cuh"
@@ -863,6 +865,9 @@ struct PCG {
     double rtol;
     int max_iter;
     float unit;  // L / 2^32: torus units -> length
+    const unsigned *meshmax;  // [F] max |Ab| bit patterns
+    double vmean;             // mean particle volume
+    float vs;                 // 1 / vmean, to a power of two
 };
 
 template <int FF>
@@ -1006,7 +1011,7 @@ __global__ void k_star_coef(ll np, const uint2 *__restrict__ pos, const int *__r
 // them from the same totals); shared so that the row loops stay small.
 struct PcgState {
     double cc[PM_MAXF], rz[PM_MAXF], rr0[PM_MAXF], sumc[PM_MAXF], sumabs[PM_MAXF];
-    float al[PM_MAXF], be[PM_MAXF];
+    float al[PM_MAXF], be[PM_MAXF], ap[PM_MAXF], S[PM_MAXF];  // ap: alpha in units of x
     int act[PM_MAXF], its[PM_MAXF];
 };
 
@@ -1018,6 +1023,11 @@ __device__ __forceinline__ void put_sums(BlockSums &B, int kind, int F, const Do
         if (f < F) put_sum(B, kind, f, v[f]);
 }
 
+// The iteration runs on S c, S the field's power of two with S max|Ab| (mean
+// volume) of order one (|c_mu| <= max|Ab| v_mu), and its inner products with z and
+// p take the factor vs: the totals over all particles stay in the range of FP32
+// whatever the field's amplitude and the box. Power-of-two factors are exact, so
+// the results are those of the unscaled iteration bit for bit. x is unscaled.
 // Reductions use slot groups {0,1,2}, {3,4}, then alternate {0} and {1,2}
 // inside the loop, and at the end {3,4}, or {0,1} when no iteration ran: no two
 // consecutive reductions share a slot, so a block that runs ahead to the next
@@ -1038,6 +1048,8 @@ __global__ void __launch_bounds__(256, FF == 8 ? 2 : 4) k_pcg(PCG a) {
     const ll np = a.np;
     const ll tid = (ll)blockIdx.x * blockDim.x + threadIdx.x, nth = (ll)gridDim.x * blockDim.x;
     const float dfac = DIM == 2 ? 0.5f : 2.0f / 3.0f;  // Jacobi diagonal = dfac v
+    if (threadIdx.x < F) S.S[threadIdx.x] = solve_scale(a.vmean * (double)__uint_as_float(a.meshmax[threadIdx.x]));
+    __syncthreads();
     // --- lumped start x = c / v; (c, c), sum c, sum |c|
     {
         Dot2 s2[FF], s1[FF], sa[FF];
@@ -1048,9 +1060,10 @@ __global__ void __launch_bounds__(256, FF == 8 ? 2 : 4) k_pcg(PCG a) {
             for (int f = 0; f < FF; ++f) {
                 cv.v[f] = f < F ? a.c[(ll)f * np + s] : 0.0f;
                 xv.v[f] = vv > 0.0f ? cv.v[f] / vv : 0.0f;
-                s2[f].fma_acc(cv.v[f], cv.v[f]);
-                s1[f].add(cv.v[f]);
-                sa[f].add(fabsf(cv.v[f]));
+                const float cs = f < F ? cv.v[f] * S.S[f] : 0.0f;
+                s2[f].fma_acc(cs, cs);
+                s1[f].add(cs);
+                sa[f].add(fabsf(cs));
             }
             stv<FF>(a.x + s * FF, xv);
         }
@@ -1062,7 +1075,9 @@ __global__ void __launch_bounds__(256, FF == 8 ? 2 : 4) k_pcg(PCG a) {
     if (!grid_sync(a.bar, a.status, passed)) return;
     if (wf < F) {
         const double cc = grid_sum(a.red, F, 0, wf);
-        if (lane0) S.cc[wf] = cc;
+        // a field so small that its residual drowns in FP32's denormals keeps the
+        // lumped start, as a zero field does
+        if (lane0) S.cc[wf] = a.vmean * (double)__uint_as_float(a.meshmax[wf]) > 0x1p-110 ? cc : 0.0;
         if (blockIdx.x == 0) {  // reported only
             const double sumc = grid_sum(a.red, F, 1, wf), sumabs = grid_sum(a.red, F, 2, wf);
             if (lane0) {
@@ -1071,7 +1086,7 @@ __global__ void __launch_bounds__(256, FF == 8 ? 2 : 4) k_pcg(PCG a) {
             }
         }
     }
-    // --- r = c - M x, z = r / d; (r, r), (r, z)
+    // --- r = S (c - M x), z = r / d; (r, r), (r, z)
     {
         Dot2 s2[FF], sz[FF];
         for (ll s = tid; s < np; s += nth) {
@@ -1081,10 +1096,10 @@ __global__ void __launch_bounds__(256, FF == 8 ? 2 : 4) k_pcg(PCG a) {
             VF<FF> zv;
 #pragma unroll
             for (int f = 0; f < FF; ++f) {
-                const float rv = (f < F ? a.c[(ll)f * np + s] : 0.0f) - mx.v[f];
+                const float rv = f < F ? (a.c[(ll)f * np + s] - mx.v[f]) * S.S[f] : 0.0f;
                 zv.v[f] = d > 0.0f ? rv / d : 0.0f;
                 s2[f].fma_acc(rv, rv);
-                sz[f].fma_acc(rv, zv.v[f]);
+                sz[f].fma_acc(rv, zv.v[f] * a.vs);
             }
             stv<FF>(a.z + s * FF, zv);
         }
@@ -1105,7 +1120,7 @@ __global__ void __launch_bounds__(256, FF == 8 ? 2 : 4) k_pcg(PCG a) {
             S.rz[wf] = rz;
             S.act[wf] = S.cc[wf] > 0.0 && rr > tol2 * S.cc[wf];
             S.its[wf] = 0;
-            S.al[wf] = 0.0f;
+            S.al[wf] = S.ap[wf] = 0.0f;
             S.be[wf] = 0.0f;
         }
     }
@@ -1123,7 +1138,7 @@ __global__ void __launch_bounds__(256, FF == 8 ? 2 : 4) k_pcg(PCG a) {
 #pragma unroll
         for (int f = 0; f < FF; ++f) {
             be[f] = f < F ? S.be[f] : 0.0f;
-            ap[f] = f < F ? S.al[f] : 0.0f;
+            ap[f] = f < F ? S.ap[f] : 0.0f;
         }
         const bool first = it == 0;
         {
@@ -1153,7 +1168,7 @@ __global__ void __launch_bounds__(256, FF == 8 ? 2 : 4) k_pcg(PCG a) {
                 stv<FF>(pout + s * FF, ps);
                 stv<FF>(a.q + s * FF, qv);
 #pragma unroll
-                for (int f = 0; f < FF; ++f) sq[f].fma_acc(ps.v[f], qv.v[f]);
+                for (int f = 0; f < FF; ++f) sq[f].fma_acc(ps.v[f] * a.vs, qv.v[f]);
             }
             put_sums<FF>(B, 0, F, sq);
             flush_pairs(B, 1, F, a.red, 0);
@@ -1162,7 +1177,10 @@ __global__ void __launch_bounds__(256, FF == 8 ? 2 : 4) k_pcg(PCG a) {
         if (wf < F) {
             double t[1];
             grid_pairs<1>(a.red, F, 0, wf, t);
-            if (lane0) S.al[wf] = S.act[wf] ? (float)quot(S.rz[wf], t[0]) : 0.0f;
+            if (lane0) {
+                S.al[wf] = S.act[wf] ? (float)quot(S.rz[wf], t[0]) : 0.0f;
+                S.ap[wf] = S.al[wf] / S.S[wf];
+            }
         }
         __syncthreads();
         last = it;
@@ -1181,7 +1199,7 @@ __global__ void __launch_bounds__(256, FF == 8 ? 2 : 4) k_pcg(PCG a) {
                     zv.v[f] = d > 0.0f ? fmaf(-al[f], qv.v[f] / d, zv.v[f]) : 0.0f;
                     const float rv = d * zv.v[f];
                     s2[f].fma_acc(rv, rv);
-                    sz[f].fma_acc(rv, zv.v[f]);
+                    sz[f].fma_acc(rv, zv.v[f] * a.vs);
                 }
                 stv<FF>(a.z + s * FF, zv);
             }
@@ -1212,7 +1230,7 @@ __global__ void __launch_bounds__(256, FF == 8 ? 2 : 4) k_pcg(PCG a) {
     {
         float ap[FF];
 #pragma unroll
-        for (int f = 0; f < FF; ++f) ap[f] = (f < F && last >= 0) ? S.al[f] : 0.0f;
+        for (int f = 0; f < FF; ++f) ap[f] = (f < F && last >= 0) ? S.ap[f] : 0.0f;
         const float *pl = a.p[(last >= 0 ? last : 0) & 1];
         const bool pend = last >= 0;
         auto xval = [&](ll i) {
@@ -1231,9 +1249,10 @@ __global__ void __launch_bounds__(256, FF == 8 ? 2 : 4) k_pcg(PCG a) {
             const float vv = a.vol[s];
 #pragma unroll
             for (int f = 0; f < FF; ++f) {
-                const float rv = (f < F ? a.c[(ll)f * np + s] : 0.0f) - mx.v[f];
+                const float Sf = f < F ? S.S[f] : 0.0f;
+                const float rv = f < F ? (a.c[(ll)f * np + s] - mx.v[f]) * Sf : 0.0f;
                 s2[f].fma_acc(rv, rv);
-                sv[f].fma_acc(vv, xs.v[f]);
+                sv[f].fma_acc(vv, xs.v[f] * Sf);
             }
             stv<FF>(a.q + s * FF, xs);
         }
@@ -1245,14 +1264,14 @@ __global__ void __launch_bounds__(256, FF == 8 ? 2 : 4) k_pcg(PCG a) {
     if (blockIdx.x != 0 || wf >= F) return;
     const double tr = grid_sum(a.red, F, end, wf), sx = grid_sum(a.red, F, end + 1, wf);
     if (lane0) {
-        const double res = S.cc[wf] > 0.0 ? sqrt(tr / S.cc[wf]) : 0.0;
+        const double res = S.cc[wf] > 0.0 ? sqrt(tr / S.cc[wf]) : 0.0, inv = 1.0 / (double)S.S[wf];
         a.scal[wf * 16 + S_INIT] = S.cc[wf] > 0.0 ? sqrt(S.rr0[wf] / S.cc[wf]) : 0.0;
         a.scal[wf * 16 + S_ITERS] = S.its[wf];
         a.scal[wf * 16 + S_RESID] = res;
-        a.scal[wf * 16 + S_SUMMESH] = S.sumc[wf];   // int Ab = sum_mu c_mu
-        a.scal[wf * 16 + S_SUMPART] = sx;           // sum_mu v_mu Abb_mu
-        a.scal[wf * 16 + S_SUMABS] = S.sumabs[wf];  // sum_mu |c_mu|: scale of the conservation error
-        if (res > a.rtol) atomicOr(a.status, ST_NOTCONV);
+        a.scal[wf * 16 + S_SUMMESH] = S.sumc[wf] * inv;   // int Ab = sum_mu c_mu
+        a.scal[wf * 16 + S_SUMPART] = sx * inv;           // sum_mu v_mu Abb_mu
+        a.scal[wf * 16 + S_SUMABS] = S.sumabs[wf] * inv;  // sum_mu |c_mu|: scale of the conservation error
+        if (!(res <= a.rtol)) atomicOr(a.status, ST_NOTCONV);  // also when it is not a number
     }
 }
 
@@ -1436,6 +1455,9 @@ int launch_pcg(const Geo &g, Work &w, ll np, int F, const float *c, float *out, 
     a.rtol = rtol;
     a.max_iter = max_iter;
     a.unit = (float)(g.L / 4294967296.0);
+    a.meshmax = w.meshmax;
+    a.vmean = (g.dim == 2 ? g.L * g.L : g.L) / (double)(np > 0 ? np : 1);
+    a.vs = std::ldexp(1.0f, std::min(120, std::max(-120, -std::ilogb(a.vmean))));
     const int fi = FF == 2 ? 0 : (FF == 4 ? 1 : 2);
     const int di = (g.dim - 1) * 3 + fi;
     void (*const kerns[6])(PCG) = {k_pcg<1, 2>, k_pcg<1, 4>, k_pcg<1, PM_MAXF>,
