@@ -867,7 +867,7 @@ struct PCG {
     float unit;  // L / 2^32: torus units -> length
     const unsigned *meshmax;  // [F] max |Ab| bit patterns
     double vmean;             // mean particle volume
-    float vs;                 // 1 / vmean, to a power of two
+    float vs;                 // vmean to a power of two
 };
 
 template <int FF>
@@ -1457,7 +1457,7 @@ int launch_pcg(const Geo &g, Work &w, ll np, int F, const float *c, float *out, 
     a.unit = (float)(g.L / 4294967296.0);
     a.meshmax = w.meshmax;
     a.vmean = (g.dim == 2 ? g.L * g.L : g.L) / (double)(np > 0 ? np : 1);
-    a.vs = std::ldexp(1.0f, std::min(120, std::max(-120, -std::ilogb(a.vmean))));
+    a.vs = std::ldexp(1.0f, std::min(120, std::max(-120, std::ilogb(a.vmean))));
     const int fi = FF == 2 ? 0 : (FF == 4 ? 1 : 2);
     const int di = (g.dim - 1) * 3 + fi;
     void (*const kerns[6])(PCG) = {k_pcg<1, 2>, k_pcg<1, 4>, k_pcg<1, PM_MAXF>,

@@ -9,7 +9,8 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("F", [1, 3, 5])
-@pytest.mark.parametrize("L,k", [(1.0, 70), (1.0, -60), (2.0**10, 60), (2.0**30, 17), (2.0**-20, 10), (2.0**-20, -30)])
+@pytest.mark.parametrize("L,k", [(1.0, 70), (1.0, -60), (2.0**10, 60), (2.0**30, 17), (2.0**-20, 10), (2.0**-20, -30),
+                                 (2.0**-28, 0), (2.0**-28, 80)])
 def test_projection_scales_exactly_2d(L, k, F):
     import torch
 
