@@ -429,7 +429,7 @@ pm_status pm_batch_assign_mass(pm_batch *b, const float *const *px, const float 
  * of cudaMalloc/cudaFree. Same result as pm_mass_solve() (conjugate gradients
  * on M x[f] = b[f], mean mode set exactly, true residual checked), but it
  * needs no context: its scratch is one file-scope device array of about
- * 38 MB that every GPU loading the library holds until exit. The caller
+ * 39 MB that every GPU loading the library holds until exit. The caller
  * passes b [F][n^dim] and x [F][n^dim] (device); x is the start vector when
  * use_x0 != 0, else the solve starts from zero. Limit: F * n^dim <= 2^20
  * values (e.g. F = 1 at 1024^2, F = 4 at 512^2); larger sizes, dim not 1 or 2,

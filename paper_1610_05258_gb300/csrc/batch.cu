@@ -44,7 +44,7 @@ namespace cg = cooperative_groups;
 namespace {
 
 // Cluster-wide sums of K accumulators (every thread of the cluster receives
-// them): compensated FP32 in the warp and over the CTA's warps, then FP64 over
+// them): Sum3 in the warp, then FP64 over the CTA's warps and over
 // the CTAs' sums, which warp 0 reads from each CTA's shared memory (DSMEM): the
 // same order on every CTA and every run. slot[2] alternates between calls: a CTA
 // writes slot[ph] only after every CTA has passed the barrier of the previous
@@ -54,7 +54,7 @@ namespace {
 // 64^2 to 512^2 nodes and 3 fields took 600 us, then 427, with a cluster for each
 // field of an instance and not for all of them 221.
 struct ClusterSums {
-    DotBits warp[3][32];
+    Sum3 warp[3][32];
     double slot[2][3], tot[3];
 };
 template <int NT, int CS, int K>
@@ -62,15 +62,16 @@ __device__ __forceinline__ void cluster_sums(const Dot2 (&v)[K], double (&out)[K
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
 #pragma unroll
     for (int k = 0; k < K; ++k) {
-        const Dot2 t = warp_total(v[k]);
-        if (lane == 0) C.warp[k][wid].set(t);
+        const Sum3 t = fold_warp(warp_parts(v[k]));
+        if (lane == 0) C.warp[k][wid] = t;
     }
     __syncthreads();
     if (wid == 0) {
 #pragma unroll
         for (int k = 0; k < K; ++k) {
-            const Dot2 t = warp_total(lane < NT / 32 ? C.warp[k][lane].get() : Dot2());
-            if (lane == 0) (CS == 1 ? C.tot : C.slot[ph])[k] = total(t);
+            double t = lane < NT / 32 ? total(C.warp[k][lane]) : 0.0;
+            for (int o = NT / 64; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+            if (lane == 0) (CS == 1 ? C.tot : C.slot[ph])[k] = t;
         }
     }
     if (CS > 1) {

@@ -161,8 +161,9 @@ struct Work {
     double *epart;      // [2 PM_MAXF][energy_blocks()] block partials of the stability diagnostics
     // solver
     float *r, *p, *q, *b;  // [F][ncell]
-    double *red;           // reduction partials [slots][grid]
-    int red_blocks;        // grid capacity of red (blocks per slot); persistent solves never exceed it
+    double *red;           // reduction partials [6 PM_MAXF][grid]
+    float4 *red4;          // reduction partials of the iterations [4 PM_MAXF][grid]
+    int red_blocks;        // grid capacity of both (blocks per slot); persistent solves never exceed it
     double *scal;          // solver scalars per field
     unsigned *bar;         // grid barrier words (2)
     int *status;           // device status word
@@ -201,6 +202,17 @@ __device__ __forceinline__ int cell_of(uint32_t X, int n) { return (int)(((ull)X
 __device__ __forceinline__ uint32_t cell_frac(uint32_t X, int n) { return (uint32_t)((ull)X * (ull)n); }
 __device__ __forceinline__ float frac_f(uint32_t X, int n) { return (float)cell_frac(X, n) * 2.3283064365386963e-10f; }
 __device__ __forceinline__ int wrapi(int i, int n) { int r = i % n; return r < 0 ? r + n : r; }
+
+// Error-free product and sum (for compensated dot products).
+__device__ __forceinline__ void two_prod(float a, float b, float &p, float &e) {
+    p = __fmul_rn(a, b);
+    e = fmaf(a, b, -p);
+}
+__device__ __forceinline__ void two_sum(float a, float b, float &s, float &e) {
+    s = __fadd_rn(a, b);
+    float z = __fsub_rn(s, a);
+    e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, z)), __fsub_rn(b, z));
+}
 
 // Accumulators. The library's arithmetic is the compensated one (PM_SUMS
 // unset): FP32 values with error-free transformations. Two other builds exist
@@ -246,16 +258,6 @@ struct KSum {
     __device__ __forceinline__ float get() const { return s + c; }
 };
 
-// Error-free product and sum (for compensated dot products).
-__device__ __forceinline__ void two_prod(float a, float b, float &p, float &e) {
-    p = __fmul_rn(a, b);
-    e = fmaf(a, b, -p);
-}
-__device__ __forceinline__ void two_sum(float a, float b, float &s, float &e) {
-    s = __fadd_rn(a, b);
-    float z = __fsub_rn(s, a);
-    e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, z)), __fsub_rn(b, z));
-}
 // Dot2-style accumulator: sum of products carried as (hi, lo).
 struct Dot2 {
     float hi, lo;
@@ -277,41 +279,66 @@ struct Dot2 {
 
 #endif
 
-// Accumulators summed with another one, and over the warp (lane 0), in the same
-// compensated form.
-__device__ __forceinline__ void join(Dot2 &a, const Dot2 &b) {
-#if defined(PM_FP64_SUMS)
-    a.hi += b.hi;
-#else
-    a.add(b.hi);
-#endif
-    a.lo += b.lo;
-}
-__device__ __forceinline__ Dot2 warp_total(Dot2 a) {
-    for (int o = 16; o > 0; o >>= 1) {
-        Dot2 b;
-        b.hi = __shfl_down_sync(0xffffffffu, a.hi, o);
-        b.lo = __shfl_down_sync(0xffffffffu, a.lo, o);
-        join(a, b);
-    }
-    return a;
-}
-__device__ __forceinline__ double total(const Dot2 &a) { return (double)a.hi + (double)a.lo; }
-// An accumulator as stored in shared memory (no constructor).
-struct DotBits {
-    decltype(Dot2::hi) hi;
-    float lo;
-    __device__ __forceinline__ void set(const Dot2 &a) {
-        hi = a.hi;
-        lo = a.lo;
-    }
-    __device__ __forceinline__ Dot2 get() const {
-        Dot2 a;
-        a.hi = hi;
-        a.lo = lo;
-        return a;
-    }
+// A sum over many threads, (a + b + c) 2^e: three floats of falling size, added
+// without error but in the last (about 70 bits), and a common exponent apart. It
+// holds what FP64 holds, in precision and range, at the rate of FP32: an FP64
+// instruction takes the pipe for 16 cycles a warp here.
+struct Sum3 {
+    float a, b, c;
+    int e;
 };
+__device__ __forceinline__ float pow2f(int k) { return __int_as_float((127 + max(k, -126)) << 23); }  // k <= 127
+__device__ __forceinline__ void add_parts(Sum3 &x, float a, float b, float c) {
+    float e1, e2, e3;
+    two_sum(x.a, a, x.a, e1);
+    two_sum(x.b, b, x.b, e2);
+    two_sum(x.b, e1, x.b, e3);
+    x.c = (x.c + c) + (e2 + e3);
+}
+// x += y; of two exponents the larger one stays (what the other's scaling drops
+// lies below 2^-126 of the sum).
+__device__ __forceinline__ void join(Sum3 &x, const Sum3 &y) {
+    const int e = max(x.e, y.e);
+    const float sx = pow2f(x.e - e), sy = pow2f(y.e - e);
+    x.a *= sx, x.b *= sx, x.c *= sx, x.e = e;
+    add_parts(x, y.a * sy, y.b * sy, y.c * sy);
+}
+// x += x of the lane `o` further on.
+__device__ __forceinline__ void fold_down(Sum3 &x, int o) {
+    const float a = __shfl_down_sync(0xffffffffu, x.a, o), b = __shfl_down_sync(0xffffffffu, x.b, o),
+                c = __shfl_down_sync(0xffffffffu, x.c, o);
+    add_parts(x, a, b, c);
+}
+__device__ __forceinline__ Sum3 scaled_parts(const Dot2 &d, float s, int e) {
+    const float hi = (float)d.hi;
+    return Sum3{hi * s, ((float)(d.hi - hi) + d.lo) * s, 0.0f, e};
+}
+// Totals of the warp's x (lane 0), or of its x and y at once (lane 0 and lane 16).
+__device__ __forceinline__ Sum3 fold_warp(Sum3 x) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) fold_down(x, o);
+    return x;
+}
+__device__ __forceinline__ Sum3 fold_warp(const Sum3 &x, const Sum3 &y) {
+    const bool up = (threadIdx.x & 16) != 0;
+    Sum3 t = up ? y : x;
+    const float a = __shfl_xor_sync(0xffffffffu, up ? x.a : y.a, 16), b = __shfl_xor_sync(0xffffffffu, up ? x.b : y.b, 16),
+                c = __shfl_xor_sync(0xffffffffu, up ? x.c : y.c, 16);
+    add_parts(t, a, b, c);
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) fold_down(t, o);
+    return t;
+}
+// The warp's accumulators ready to be folded, their largest at order one.
+__device__ __forceinline__ Sum3 warp_parts(const Dot2 &d) {
+    const Sum3 p = scaled_parts(d, 1.0f, 0);
+    const unsigned m = __reduce_max_sync(0xffffffffu, __float_as_uint(fmaxf(fabsf(p.a), fabsf(p.b))));
+    const int e = min(max((int)(m >> 23) - 127, -126), 126);
+    return scaled_parts(d, pow2f(-e), e);
+}
+__device__ __forceinline__ double total(const Sum3 &t) {
+    return (((double)t.a + (double)t.b) + (double)t.c) * __hiloint2double((1023 + t.e) << 20, 0);
+}
 
 // Compensated M x at node i of field array xf; returns (hi, lo) of the
 // unscaled stencil sum; the caller multiplies by c = h/6, h^2/36 (bilinear)

@@ -10,19 +10,18 @@
 //
 // The mesh solves are ONE persistent cooperative kernel each (k_cg, k_cheb):
 // every block owns a strided share of the nodes of all F fields, and the
-// reductions go through per-block FP64 partials that every block then sums in
-// the same fixed order (deterministic and identical on all blocks, so all
+// reductions go through the blocks' totals, which every block then sums in the
+// same fixed order (deterministic and identical on all blocks, so all
 // blocks take the same branch). Per-node products are accumulated per thread
-// and per warp in compensated FP32 before entering FP64. Before iterating, the
-// mean mode of x is set exactly from sum_j b_j (1 is an eigenvector of the
-// circulant M with eigenvalue h^dim, and the iterations keep the mean of the
-// start vector), which makes the result conservative (Eq. cons) to rounding at
-// any iteration count.
+// in compensated FP32, and the threads' sums lose nothing against FP64 (Sum3).
+// Before iterating, the mean mode of x is set exactly from sum_j b_j (1 is an
+// eigenvector of the circulant M with eigenvalue h^dim, and the iterations keep
+// the mean of the start vector), which makes the result conservative (Eq. cons)
+// to rounding at any iteration count.
 //
 // What bounds them is the grid barrier with its reduction on small meshes
 // (FP64 runs at 1/64 of FP32 here, so one thread per field computes the step
-// lengths, and FP64 starts at the warp totals) and the passes over the vectors
-// on large ones.
+// lengths) and the passes over the vectors on large ones.
 #include <cooperative_groups.h>
 
 #include <algorithm>
@@ -46,6 +45,7 @@ struct CG {
     float *r[2], *s[2], *w[2];  // CG: residual, M p, M r, alternating between passes
                                 // Chebyshev: r and d (in s)
     double *red;            // [6 * PM_MAXF][grid]
+    float4 *red4;           // [4 * PM_MAXF][grid]
     double *scal;           // [F][16]
     unsigned *bar;          // [2] barrier count
     int *status;
@@ -91,31 +91,43 @@ __device__ bool grid_sync(unsigned *bar, int *status, unsigned &passed) {
     return ok != 0;
 }
 
-// A sum over the grid goes through red[(slot + kind) * F + f][block]: every
-// thread puts its accumulator (the warp's total goes to shared memory), the block
-// flushes, and after a grid barrier every block sums the partials in the same
-// order. FP64 sums (flush_sums, grid_sum) from the warp totals on where the
-// total itself is used or reported; the inner products of an iteration, which
-// only set FP32 step lengths and the stop, stay compensated FP32 pairs
-// (flush_pairs, grid_pairs): an FP64 instruction holds its pipe for 16 cycles a
-// warp, and with the FP64 sums and divisions an iteration of one block took
-// 7500 cycles, of 64 blocks 14000; now 5200 and 10000, 2250 of them the barrier.
+// A sum over the grid: every thread puts its accumulator (the warp's total goes
+// to shared memory), the block flushes its total, and after a grid barrier every
+// block sums the blocks' totals in the same order. Sum3 throughout or FP64, so
+// nothing is held in fewer bits than FP64 holds:
+//  put_sum, flush_sums, grid_sum: any range; FP64 totals of the blocks in
+//    red[(slot + kind) * F + f][block]. The start, the closing residual.
+//  put_scaled, flush_scaled, grid_scaled: the inner products of an iteration,
+//    brought to order one by powers of two, so that no exponents are carried;
+//    Sum3 in red4[(slot + kind) * F + f][block].
+// An FP64 addition takes 62 cycles here, a sum over a warp 680 in FP64 and 228 in
+// Sum3 (180 in FP32 pairs, which this replaces: whole solves by CG take the
+// same time to 5 %, 256^2 122.5 -> 125.7 us, 255^2 166 -> 147 us).
 struct BlockSums {
-    DotBits v[3][PM_MAXF][8];
+    Sum3 v[3][PM_MAXF][8];
 };
 __device__ __forceinline__ void put_sum(BlockSums &B, int kind, int f, const Dot2 &a) {
-    const Dot2 t = warp_total(a);
-    if ((threadIdx.x & 31) == 0) B.v[kind][f][threadIdx.x >> 5].set(t);
+    const Sum3 t = fold_warp(warp_parts(a));
+    if ((threadIdx.x & 31) == 0) B.v[kind][f][threadIdx.x >> 5] = t;
+}
+// Kinds 0 and 1 at once.
+__device__ __forceinline__ void put_sums(BlockSums &B, int f, const Dot2 &a0, const Dot2 &a1) {
+    const Sum3 t = fold_warp(warp_parts(a0), warp_parts(a1));
+    if ((threadIdx.x & 15) == 0) B.v[threadIdx.x >> 4 & 1][f][threadIdx.x >> 5] = t;
 }
 __device__ __forceinline__ void flush_sums(const BlockSums &B, int kinds, int F, double *red, int slot) {
     __syncthreads();
     const int t = threadIdx.x;
     if (t < kinds * F) {
-        double v[8];
+        const Sum3 *v = B.v[t / F][t % F];
+        Sum3 a = v[0], b = v[4];
 #pragma unroll
-        for (int w = 0; w < 8; ++w) v[w] = total(B.v[t / F][t % F][w].get());
-        red[(ll)(slot * F + t) * gridDim.x + blockIdx.x] =
-            ((v[0] + v[1]) + (v[2] + v[3])) + ((v[4] + v[5]) + (v[6] + v[7]));
+        for (int w = 1; w < 4; ++w) {
+            join(a, v[w]);
+            join(b, v[w + 4]);
+        }
+        join(a, b);
+        red[(ll)(slot * F + t) * gridDim.x + blockIdx.x] = total(a);
     }
 }
 // Total of (slot, f) over all blocks, by one warp.
@@ -128,69 +140,50 @@ __device__ __forceinline__ double grid_sum(const double *red, int F, int slot, i
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     return s;
 }
-#if defined(PM_FP64_SUMS)
-__device__ __forceinline__ double pack(const Dot2 &a) { return total(a); }
-__device__ __forceinline__ Dot2 unpack(double v) {
-    Dot2 a;
-    a.hi = v;
-    return a;
+__device__ __forceinline__ void put_scaled(BlockSums &B, int kind, int f, const Dot2 &a, float scale) {
+    const Sum3 t = fold_warp(scaled_parts(a, scale, 0));
+    if ((threadIdx.x & 31) == 0) B.v[kind][f][threadIdx.x >> 5] = t;
 }
-#else
-__device__ __forceinline__ double pack(const Dot2 &a) {
-    return __hiloint2double(__float_as_int(a.hi), __float_as_int(a.lo));  // bits only
+// Kinds 0 and 1 at once.
+__device__ __forceinline__ void put_scaled(BlockSums &B, int f, const Dot2 &a0, float s0, const Dot2 &a1, float s1) {
+    const Sum3 t = fold_warp(scaled_parts(a0, s0, 0), scaled_parts(a1, s1, 0));
+    if ((threadIdx.x & 15) == 0) B.v[threadIdx.x >> 4 & 1][f][threadIdx.x >> 5] = t;
 }
-__device__ __forceinline__ Dot2 unpack(double v) {
-    Dot2 a;
-    a.hi = __int_as_float(__double2hiint(v));
-    a.lo = __int_as_float(__double2loint(v));
-    return a;
-}
-#endif
-__device__ __forceinline__ void flush_pairs(const BlockSums &B, int kinds, int F, double *red, int slot) {
+__device__ __forceinline__ void flush_scaled(const BlockSums &B, int kinds, int F, float4 *red4, int slot) {
     __syncthreads();
     const int t = threadIdx.x;
     if (t < kinds * F) {
-        const DotBits *v = B.v[t / F][t % F];
-        Dot2 a = v[0].get(), b = v[4].get();
+        const Sum3 *v = B.v[t / F][t % F];
+        Sum3 a = v[0], b = v[4];
 #pragma unroll
         for (int w = 1; w < 4; ++w) {
-            join(a, v[w].get());
-            join(b, v[w + 4].get());
+            add_parts(a, v[w].a, v[w].b, v[w].c);
+            add_parts(b, v[w + 4].a, v[w + 4].b, v[w + 4].c);
         }
-        join(a, b);
-        red[(ll)(slot * F + t) * gridDim.x + blockIdx.x] = pack(a);
+        add_parts(a, b.a, b.b, b.c);
+        red4[(ll)(slot * F + t) * gridDim.x + blockIdx.x] = make_float4(a.a, a.b, a.c, 0.0f);
     }
 }
-// Totals of field f in K consecutive slots, by one warp; lane 0 has them.
+// Totals of field f in K consecutive slots (1 or 2) over all blocks, by one
+// warp, half of it for each of two slots; lane 0 has them.
 template <int K>
-__device__ __forceinline__ void grid_pairs(const double *red, int F, int slot, int f, double (&out)[K]) {
-    const int lane = threadIdx.x & 31;
-    Dot2 a[K];
-#pragma unroll 2
-    for (unsigned i = lane; i < gridDim.x; i += 32)
+__device__ __forceinline__ void grid_scaled(const float4 *red4, int F, int slot, int f, double (&out)[K]) {
+    constexpr int W = 32 / K;
+    const unsigned lane = threadIdx.x & 31;
+    const float4 *src = red4 + (ll)((slot + (int)(lane / W)) * F + f) * gridDim.x;
+    Sum3 s{0.0f, 0.0f, 0.0f, 0};
+    // eight loads in flight, also at the end: a load is an L2 latency
+    for (unsigned i = lane % W; i < gridDim.x; i += 8 * W) {
+        float4 t[8];
 #pragma unroll
-        for (int k = 0; k < K; ++k) join(a[k], unpack(__ldcg(red + (ll)((slot + k) * F + f) * gridDim.x + i)));
-    for (int o = 16; o > 0; o >>= 1)
+        for (int j = 0; j < 8; ++j) t[j] = i + j * W < gridDim.x ? __ldcg(src + i + j * W) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
 #pragma unroll
-        for (int k = 0; k < K; ++k) {
-            Dot2 b;
-            b.hi = __shfl_down_sync(0xffffffffu, a[k].hi, o);
-            b.lo = __shfl_down_sync(0xffffffffu, a[k].lo, o);
-            join(a[k], b);
-        }
+        for (int j = 0; j < 8; ++j) add_parts(s, t[j].x, t[j].y, t[j].z);
+    }
 #pragma unroll
-    for (int k = 0; k < K; ++k) out[k] = total(a[k]);
-}
-
-// a / b to a few units of FP64 rounding, b > 0: the FP32 reciprocal refined by one
-// Newton step (relative error e -> e^2, 2^-46) and one on the quotient. Seven
-// dependent FP64 operations. Outside the range of the seed the plain quotient.
-__device__ __forceinline__ double quot(double a, double b) {
-    if (!(b > 1e-30 && b < 1e30)) return a / b;
-    double r = (double)(1.0f / (float)b);
-    r = fma(fma(-b, r, 1.0), r, r);
-    const double q = a * r;
-    return fma(fma(-b, q, a), r, q);
+    for (int o = W / 2; o > 0; o >>= 1) fold_down(s, o);
+    out[0] = ((double)s.a + (double)s.b) + (double)s.c;
+    if (K == 2) out[K - 1] = __shfl_down_sync(0xffffffffu, out[0], W);
 }
 
 // Totals of the per-block particle sums of one row (sum v A or sum v |A|) by
@@ -345,7 +338,9 @@ struct NextR {
 // Per-field state of a mesh solve, the same on every block.
 struct SolveState {
     double bb[PM_MAXF], rr[PM_MAXF], rr0[PM_MAXF], pMp[PM_MAXF], sumb[PM_MAXF], tr[PM_MAXF], sx[PM_MAXF];
-    float S[PM_MAXF], sh[PM_MAXF], al[PM_MAXF], be[PM_MAXF];
+    double thr[PM_MAXF];  // the iteration's tolerance for rr
+    float S[PM_MAXF], sh[PM_MAXF], al[PM_MAXF], be[PM_MAXF], ka[PM_MAXF];
+    float kr[PM_MAXF], kw[PM_MAXF];  // powers of two that bring (r, r) and (w, r) to order one; rr and pMp hold them
     int act[PM_MAXF], first[PM_MAXF], its[PM_MAXF], steps[PM_MAXF];
 };
 
@@ -389,20 +384,21 @@ __device__ __forceinline__ bool solve_begin(const CG &a, SolveState &V, BlockSum
             if (a.has_start) ldn<VEC>(a.x + o, xv);
 #pragma unroll
             for (int j = 0; j < VEC; ++j) {
-                sb.add(bv[j]);
-                sa.add(fabsf(bv[j]));
-                if (a.has_start) sx.add(xv[j]);
+                // times 2^-10: a thread's sums stay in range where the nodes do
+                sb.add(bv[j] * 0x1p-10f);
+                sa.add(fabsf(bv[j]) * 0x1p-10f);
+                if (a.has_start) sx.add(xv[j] * 0x1p-10f);
             }
         }
-        put_sum(B, 0, f, sb);
-        put_sum(B, 1, f, sa);
+        put_sums(B, f, sb, sa);
         put_sum(B, 2, f, sx);
     }
     flush_sums(B, 3, F, a.red, 0);
     if (!grid_sync(a.bar, a.status, passed)) return false;
     const int f = threadIdx.x >> 5;
     if (f < F) {
-        const double sumb = grid_sum(a.red, F, 0, f), suma = grid_sum(a.red, F, 1, f), sumx = grid_sum(a.red, F, 2, f);
+        const double sumb = 1024.0 * grid_sum(a.red, F, 0, f), suma = 1024.0 * grid_sum(a.red, F, 1, f),
+                     sumx = 1024.0 * grid_sum(a.red, F, 2, f);
         if ((threadIdx.x & 31) == 0) {
             const float S = solve_scale(suma / (double)nn);
             V.S[f] = S;
@@ -454,8 +450,7 @@ __device__ __forceinline__ void residual_pass(const CG &a, SolveState &V, BlockS
                 stn<VEC>(out + fo + i0, ct);
             }
         }
-        put_sum(B, 0, f, s);
-        put_sum(B, 1, f, t);
+        put_sums(B, f, s, t);
     }
     flush_sums(B, 2, F, a.red, slot);
 }
@@ -486,6 +481,16 @@ __device__ __forceinline__ void solve_report(const CG &a, const SolveState &V, d
     if (res > a.rtol) atomicOr(a.status, ST_NOTCONV);
 }
 
+// Field f (re)starts from a residual of squared norm rr.
+__device__ __forceinline__ void restart_state(SolveState &V, int f, double rr, double tol2, ll nn, double hd) {
+    const float kr = solve_scale(rr / (double)nn), kw = solve_scale(rr / (double)nn * hd);
+    V.rr[f] = rr * (double)kr;
+    V.thr[f] = tol2 * V.bb[f] * (double)kr;
+    V.kr[f] = kr;
+    V.kw[f] = kw;
+    V.ka[f] = kw / kr;
+}
+
 // Conjugate gradients with one pass and one grid barrier per iteration. With
 // w = M r at hand, (r, r) and (w, r) give both step lengths (Chronopoulos and
 // Gear): beta = rr / rr_old, alpha = rr / pMp, pMp = (w, r) - beta^2 pMp_old, and
@@ -497,11 +502,11 @@ __device__ __forceinline__ void solve_report(const CG &a, const SolveState &V, d
 // iterations, one block) 105 -> 42 us; 256^2 (13) 232 -> 97 us; 512^2, 3 fields
 // (19) 669 -> 284 us; 2048^2, 4 fields (19) 4046 -> 2766 us, 40 bytes per node and
 // iteration at 4.6 TB/s.
-// Consecutive reductions use slot groups {0, 1, 2}, {3, 4}, {5} and then
-// alternate {0, 1} and {2, 3}, so that a block that runs ahead never overwrites
-// partials another block is summing.
+// Consecutive reductions never share slots, so that a block that runs ahead never
+// overwrites partials another block is summing: {0, 1, 2} and {3, 4} of red, {0}
+// and then alternately {2, 3} and {0, 1} of red4, and {0, 1} of red at the end.
 template <int DIM, int P1, int VEC>
-__global__ void __launch_bounds__(256) k_cg(CG a) {
+__global__ void __launch_bounds__(256, VEC == 4 ? 3 : 4) k_cg(CG a) {
     __shared__ SolveState V;
     __shared__ BlockSums B;
     unsigned passed = 0;
@@ -521,13 +526,14 @@ __global__ void __launch_bounds__(256) k_cg(CG a) {
     if (wf < F) {
         const double rr = grid_sum(a.red, F, 3, wf), bb = grid_sum(a.red, F, 4, wf);
         if (lane0) {
-            V.rr[wf] = V.rr0[wf] = rr;
+            V.rr0[wf] = rr;
             V.bb[wf] = bb;
+            restart_state(V, wf, rr, tol2, nn, hd);
             V.act[wf] = V.first[wf] = bb > 0.0 && rr > tol2 * bb;
         }
     }
     __syncthreads();
-    int cur = 0, it = 0, slot = 5;
+    int cur = 0, it = 0;
     for (int restarts = 0;; ++restarts) {
         bool any = false;
         for (int f = 0; f < F; ++f) any |= V.act[f] != 0;
@@ -548,24 +554,24 @@ __global__ void __launch_bounds__(256) k_cg(CG a) {
                     }
                     stn<VEC>(a.w[cur] + fo + i * VEC, hi);
                 }
-                put_sum(B, 0, f, d);
+                put_scaled(B, 0, f, d, V.kw[f]);
             }
-            flush_pairs(B, 1, F, a.red, slot);
+            flush_scaled(B, 1, F, a.red4, 0);
             if (!grid_sync(a.bar, a.status, passed)) return;
             if (wf < F && V.act[wf]) {
                 double t[1];
-                grid_pairs<1>(a.red, F, slot, wf, t);
+                grid_scaled<1>(a.red4, F, 0, wf, t);
                 if (lane0) {
                     const double wr = t[0];
                     V.pMp[wf] = wr;
-                    V.al[wf] = (float)quot(V.rr[wf], wr);
+                    V.al[wf] = (float)(V.rr[wf] / wr) * V.ka[wf];
                     V.be[wf] = 0.0f;
                     V.first[wf] = 1;
                     if (!(wr > 0.0)) V.act[wf] = 0;  // r below the range of its products
                 }
             }
             __syncthreads();
-            slot = slot == 5 ? 0 : slot ^ 2;
+            int slot = 2;
             while (any && it < a.max_iter) {
                 const int nxt = cur ^ 1;
                 for (int f = 0; f < F; ++f) {
@@ -606,24 +612,23 @@ __global__ void __launch_bounds__(256) k_cg(CG a) {
                         stn<VEC>(a.p + o, pv);
                         stn<VEC>(a.xw + o, xv);
                     }
-                    put_sum(B, 0, f, sr);
-                    put_sum(B, 1, f, sw);
+                    put_scaled(B, f, sr, V.kr[f], sw, V.kw[f]);
                 }
-                flush_pairs(B, 2, F, a.red, slot);
+                flush_scaled(B, 2, F, a.red4, slot);
                 if (!grid_sync(a.bar, a.status, passed)) return;
                 if (wf < F && V.act[wf]) {
                     double t[2];
-                    grid_pairs<2>(a.red, F, slot, wf, t);
+                    grid_scaled<2>(a.red4, F, slot, wf, t);
                     if (lane0) {
                         const double rr = t[0], wr = t[1];
-                        const double beta = quot(rr, V.rr[wf]), pMp = wr - beta * (beta * V.pMp[wf]);
+                        const double beta = rr / V.rr[wf], pMp = wr - beta * (beta * V.pMp[wf]);
                         V.pMp[wf] = pMp;
-                        V.al[wf] = (float)quot(rr, pMp);
+                        V.al[wf] = (float)(rr / pMp) * V.ka[wf];
                         V.be[wf] = (float)beta;
                         V.rr[wf] = rr;
                         V.first[wf] = 0;
                         ++V.its[wf];
-                        if (rr <= tol2 * V.bb[wf] || !(pMp > 0.0)) V.act[wf] = 0;
+                        if (rr <= V.thr[wf] || !(pMp > 0.0)) V.act[wf] = 0;
                     }
                 }
                 __syncthreads();
@@ -633,23 +638,20 @@ __global__ void __launch_bounds__(256) k_cg(CG a) {
                 any = false;
                 for (int f = 0; f < F; ++f) any |= V.act[f] != 0;
             }
-        } else if (restarts == 0) {
-            slot = 0;
         }
         // the true residual of every field, and the result
-        residual_pass<DIM, P1, VEC, false>(a, V, B, a.r[cur], a.x, slot);
+        residual_pass<DIM, P1, VEC, false>(a, V, B, a.r[cur], a.x, 0);
         if (!grid_sync(a.bar, a.status, passed)) return;
         if (wf < F) {
-            const double tr = grid_sum(a.red, F, slot, wf), sx = grid_sum(a.red, F, slot + 1, wf);
+            const double tr = grid_sum(a.red, F, 0, wf), sx = grid_sum(a.red, F, 1, wf);
             if (lane0) {
                 V.tr[wf] = tr;
                 V.sx[wf] = sx;
                 V.act[wf] = V.bb[wf] > 0.0 && tr > tol2 * V.bb[wf];
-                if (V.act[wf]) V.rr[wf] = tr;
+                if (V.act[wf]) restart_state(V, wf, tr, tol2, nn, hd);
             }
         }
         __syncthreads();
-        slot ^= 2;
         bool again = false;
         for (int f = 0; f < F; ++f) again |= V.act[f] != 0;
         // drifted fields restart from their true residual
@@ -721,7 +723,7 @@ __device__ __forceinline__ void cheb_step(const Val &d, int n, unsigned nv, floa
 }
 
 template <int DIM, int P1, int VEC>
-__global__ void __launch_bounds__(256) k_cheb(CG a) {
+__global__ void __launch_bounds__(256, DIM == 1 ? 2 : 3) k_cheb(CG a) {
     __shared__ SolveState V;
     __shared__ BlockSums B;
     __shared__ float coef[2][CHEB_COEF];
@@ -860,14 +862,15 @@ struct PCG {
     float *x, *z, *q;       // [np][FF]: iterate, D^-1 r, M_p p (the solution at exit)
     float *p[2];            // [np][FF]: search directions of even and odd iterations
     double *red, *scal;
+    float4 *red4;
     unsigned *bar;
     int *status;
     double rtol;
     int max_iter;
     float unit;  // L / 2^32: torus units -> length
     const unsigned *meshmax;  // [F] max |Ab| bit patterns
-    double vmean;             // mean particle volume
-    float vs;                 // vmean to a power of two
+    int ev;                   // binary exponent of the mean particle volume
+    float vs;                 // 2^ev
 };
 
 template <int FF>
@@ -1011,7 +1014,7 @@ __global__ void k_star_coef(ll np, const uint2 *__restrict__ pos, const int *__r
 // them from the same totals); shared so that the row loops stay small.
 struct PcgState {
     double cc[PM_MAXF], rz[PM_MAXF], rr0[PM_MAXF], sumc[PM_MAXF], sumabs[PM_MAXF];
-    float al[PM_MAXF], be[PM_MAXF], ap[PM_MAXF], S[PM_MAXF];  // ap: alpha in units of x
+    float al[PM_MAXF], be[PM_MAXF], ap[PM_MAXF], S[PM_MAXF], iS[PM_MAXF];  // ap: alpha in units of x; iS = 1 / S
     int act[PM_MAXF], its[PM_MAXF];
 };
 
@@ -1022,18 +1025,30 @@ __device__ __forceinline__ void put_sums(BlockSums &B, int kind, int F, const Do
     for (int f = 0; f < FF; ++f)
         if (f < F) put_sum(B, kind, f, v[f]);
 }
+template <int FF>
+__device__ __forceinline__ void put_order_one(BlockSums &B, int F, const Dot2 (&v)[FF]) {
+#pragma unroll
+    for (int f = 0; f < FF; ++f)
+        if (f < F) put_scaled(B, 0, f, v[f], 1.0f);
+}
+template <int FF>
+__device__ __forceinline__ void put_order_one(BlockSums &B, int F, const Dot2 (&v)[FF], const Dot2 (&u)[FF]) {
+#pragma unroll
+    for (int f = 0; f < FF; ++f)
+        if (f < F) put_scaled(B, f, v[f], 1.0f, u[f], 1.0f);
+}
 
 // The iteration runs on S c, S the field's power of two with S max|Ab| (mean
 // volume) of order one (|c_mu| <= max|Ab| v_mu), and its inner products with z and
 // p take the factor vs: the totals over all particles stay in the range of FP32
 // whatever the field's amplitude and the box. Power-of-two factors are exact, so
 // the results are those of the unscaled iteration bit for bit. x is unscaled.
-// Reductions use slot groups {0,1,2}, {3,4}, then alternate {0} and {1,2}
-// inside the loop, and at the end {3,4}, or {0,1} when no iteration ran: no two
+// Reductions use slot groups {0,1,2} and {3,4} of red, then alternate {0} and
+// {1,2} of red4 inside the loop, and at the end {0,1} of red: no two
 // consecutive reductions share a slot, so a block that runs ahead to the next
 // reduction never overwrites a partial that a slower block is still summing.
-// Sums as in the mesh solves: with FP64 shuffles and sums per thread an
-// solve of 3 fields on 1.97e6 particles (7 iterations) took 1.34 ms, now 1.15.
+// Sums as in the mesh solves: with FP64 shuffles and sums per thread a
+// solve of 3 fields on 1.97e6 particles (7 iterations) took 1.34 ms, now 1.16.
 // An iteration is 97 us for the rows (two 16-byte gathers per neighbour from the
 // L1 and L2), 22 us for the update and 10 us in the two barriers.
 template <int DIM, int FF>
@@ -1048,10 +1063,21 @@ __global__ void __launch_bounds__(256, FF == 8 ? 2 : 4) k_pcg(PCG a) {
     const ll np = a.np;
     const ll tid = (ll)blockIdx.x * blockDim.x + threadIdx.x, nth = (ll)gridDim.x * blockDim.x;
     const float dfac = DIM == 2 ? 0.5f : 2.0f / 3.0f;  // Jacobi diagonal = dfac v
-    if (threadIdx.x < F) S.S[threadIdx.x] = solve_scale(a.vmean * (double)__uint_as_float(a.meshmax[threadIdx.x]));
-    __syncthreads();
+    // binary exponent of max|Ab| (mean volume) of field f, 0 for a zero field
+    auto exponent = [&](int f) {
+        const float m = __uint_as_float(__ldg(a.meshmax + f));
+        return m > 0.0f ? min(max(ilogbf(m) + a.ev, -120), 120) : 0;
+    };
+    if (threadIdx.x < F) {
+        const int e = exponent(threadIdx.x);
+        S.S[threadIdx.x] = pow2f(-e);
+        S.iS[threadIdx.x] = pow2f(e);
+    }
     // --- lumped start x = c / v; (c, c), sum c, sum |c|
     {
+        float Sf[FF];
+#pragma unroll
+        for (int f = 0; f < FF; ++f) Sf[f] = f < F ? pow2f(-exponent(f)) : 0.0f;
         Dot2 s2[FF], s1[FF], sa[FF];
         for (ll s = tid; s < np; s += nth) {
             const float vv = a.vol[s];
@@ -1060,7 +1086,7 @@ __global__ void __launch_bounds__(256, FF == 8 ? 2 : 4) k_pcg(PCG a) {
             for (int f = 0; f < FF; ++f) {
                 cv.v[f] = f < F ? a.c[(ll)f * np + s] : 0.0f;
                 xv.v[f] = vv > 0.0f ? cv.v[f] / vv : 0.0f;
-                const float cs = f < F ? cv.v[f] * S.S[f] : 0.0f;
+                const float cs = cv.v[f] * Sf[f];
                 s2[f].fma_acc(cs, cs);
                 s1[f].add(cs);
                 sa[f].add(fabsf(cs));
@@ -1077,7 +1103,7 @@ __global__ void __launch_bounds__(256, FF == 8 ? 2 : 4) k_pcg(PCG a) {
         const double cc = grid_sum(a.red, F, 0, wf);
         // a field so small that its residual drowns in FP32's denormals keeps the
         // lumped start, as a zero field does
-        if (lane0) S.cc[wf] = a.vmean * (double)__uint_as_float(a.meshmax[wf]) > 0x1p-110 ? cc : 0.0;
+        if (lane0) S.cc[wf] = exponent(wf) > -110 ? cc : 0.0;
         if (blockIdx.x == 0) {  // reported only
             const double sumc = grid_sum(a.red, F, 1, wf), sumabs = grid_sum(a.red, F, 2, wf);
             if (lane0) {
@@ -1170,16 +1196,16 @@ __global__ void __launch_bounds__(256, FF == 8 ? 2 : 4) k_pcg(PCG a) {
 #pragma unroll
                 for (int f = 0; f < FF; ++f) sq[f].fma_acc(ps.v[f] * a.vs, qv.v[f]);
             }
-            put_sums<FF>(B, 0, F, sq);
-            flush_pairs(B, 1, F, a.red, 0);
+            put_order_one<FF>(B, F, sq);
+            flush_scaled(B, 1, F, a.red4, 0);
         }
         if (!grid_sync(a.bar, a.status, passed)) return;
         if (wf < F) {
             double t[1];
-            grid_pairs<1>(a.red, F, 0, wf, t);
+            grid_scaled<1>(a.red4, F, 0, wf, t);
             if (lane0) {
-                S.al[wf] = S.act[wf] ? (float)quot(S.rz[wf], t[0]) : 0.0f;
-                S.ap[wf] = S.al[wf] / S.S[wf];
+                S.al[wf] = S.act[wf] ? (float)(S.rz[wf] / t[0]) : 0.0f;
+                S.ap[wf] = S.al[wf] * S.iS[wf];
             }
         }
         __syncthreads();
@@ -1203,18 +1229,17 @@ __global__ void __launch_bounds__(256, FF == 8 ? 2 : 4) k_pcg(PCG a) {
                 }
                 stv<FF>(a.z + s * FF, zv);
             }
-            put_sums<FF>(B, 0, F, s2);
-            put_sums<FF>(B, 1, F, sz);
-            flush_pairs(B, 2, F, a.red, 1);
+            put_order_one<FF>(B, F, s2, sz);
+            flush_scaled(B, 2, F, a.red4, 1);
         }
         if (!grid_sync(a.bar, a.status, passed)) return;
         if (wf < F) {
             double t[2];
-            grid_pairs<2>(a.red, F, 1, wf, t);
+            grid_scaled<2>(a.red4, F, 1, wf, t);
             if (lane0) {
                 S.be[wf] = 0.0f;
                 if (S.act[wf]) {
-                    S.be[wf] = (float)quot(t[1], S.rz[wf]);
+                    S.be[wf] = (float)(t[1] / S.rz[wf]);
                     S.rz[wf] = t[1];
                     ++S.its[wf];
                     if (t[0] <= tol2 * S.cc[wf]) S.act[wf] = 0;
@@ -1226,7 +1251,6 @@ __global__ void __launch_bounds__(256, FF == 8 ? 2 : 4) k_pcg(PCG a) {
     // --- report: x += alpha p of the last iteration (at the row and at each
     // neighbour), true residual c - M x, sum v x (= sum c for the exact
     // solution); the solution goes to q
-    const int end = last >= 0 ? 3 : 0;
     {
         float ap[FF];
 #pragma unroll
@@ -1258,13 +1282,13 @@ __global__ void __launch_bounds__(256, FF == 8 ? 2 : 4) k_pcg(PCG a) {
         }
         put_sums<FF>(B, 0, F, s2);
         put_sums<FF>(B, 1, F, sv);
-        flush_sums(B, 2, F, a.red, end);
+        flush_sums(B, 2, F, a.red, 0);
     }
     if (!grid_sync(a.bar, a.status, passed)) return;
     if (blockIdx.x != 0 || wf >= F) return;
-    const double tr = grid_sum(a.red, F, end, wf), sx = grid_sum(a.red, F, end + 1, wf);
+    const double tr = grid_sum(a.red, F, 0, wf), sx = grid_sum(a.red, F, 1, wf);
     if (lane0) {
-        const double res = S.cc[wf] > 0.0 ? sqrt(tr / S.cc[wf]) : 0.0, inv = 1.0 / (double)S.S[wf];
+        const double res = S.cc[wf] > 0.0 ? sqrt(tr / S.cc[wf]) : 0.0, inv = (double)S.iS[wf];
         a.scal[wf * 16 + S_INIT] = S.cc[wf] > 0.0 ? sqrt(S.rr0[wf] / S.cc[wf]) : 0.0;
         a.scal[wf * 16 + S_ITERS] = S.its[wf];
         a.scal[wf * 16 + S_RESID] = res;
@@ -1377,6 +1401,7 @@ CG mesh_args(const Geo &g, Work &w, int F, const float *b_float, bool b_from_fix
     a.s[1] = w.part + 2 * len;
     a.xw = w.part + 3 * len;
     a.red = w.red;
+    a.red4 = w.red4;
     a.scal = w.scal;
     a.bar = w.bar;
     a.status = w.status;
@@ -1449,6 +1474,7 @@ int launch_pcg(const Geo &g, Work &w, ll np, int F, const float *c, float *out, 
     a.p[1] = w.pp2;
     a.q = w.pq;
     a.red = w.red;
+    a.red4 = w.red4;
     a.scal = w.scal;
     a.bar = w.bar;
     a.status = w.status;
@@ -1456,8 +1482,8 @@ int launch_pcg(const Geo &g, Work &w, ll np, int F, const float *c, float *out, 
     a.max_iter = max_iter;
     a.unit = (float)(g.L / 4294967296.0);
     a.meshmax = w.meshmax;
-    a.vmean = (g.dim == 2 ? g.L * g.L : g.L) / (double)(np > 0 ? np : 1);
-    a.vs = std::ldexp(1.0f, std::min(120, std::max(-120, std::ilogb(a.vmean))));
+    a.ev = std::min(1000, std::max(-1000, std::ilogb((g.dim == 2 ? g.L * g.L : g.L) / (double)(np > 0 ? np : 1))));
+    a.vs = std::ldexp(1.0f, std::min(120, std::max(-120, a.ev)));
     const int fi = FF == 2 ? 0 : (FF == 4 ? 1 : 2);
     const int di = (g.dim - 1) * 3 + fi;
     void (*const kerns[6])(PCG) = {k_pcg<1, 2>, k_pcg<1, 4>, k_pcg<1, PM_MAXF>,

@@ -13,7 +13,7 @@
 // Scratch: PM_NOALLOC_MAX_VALUES floats for each of the nine vectors of the
 // CG solve, plus reduction partials for up to PM_NOALLOC_MAX_GRID blocks
 // (the solve's grid is clamped to that), solver scalars, the barrier words and
-// the status word: about 38 MB, held by every GPU that loads the library
+// the status word: about 39 MB, held by every GPU that loads the library
 // until the process exits. Its device address is looked up once per device
 // (cudaGetSymbolAddress) by the first call on that device.
 #include <cstring>
@@ -30,7 +30,9 @@ namespace {
 constexpr size_t kVecBytes = sizeof(float) * (size_t)PM_NOALLOC_MAX_VALUES;
 constexpr size_t kRedOff = 9 * kVecBytes;
 constexpr size_t kRedBytes = sizeof(double) * 6 * PM_MAXF * (size_t)PM_NOALLOC_MAX_GRID;
-constexpr size_t kScalOff = kRedOff + kRedBytes;
+constexpr size_t kRed4Off = kRedOff + kRedBytes;
+constexpr size_t kRed4Bytes = sizeof(float4) * 4 * PM_MAXF * (size_t)PM_NOALLOC_MAX_GRID;
+constexpr size_t kScalOff = kRed4Off + kRed4Bytes;
 constexpr size_t kScalBytes = sizeof(double) * 16 * PM_MAXF;
 constexpr size_t kBarOff = kScalOff + kScalBytes;
 constexpr size_t kStatusOff = kBarOff + 256;
@@ -87,6 +89,7 @@ extern "C" pm_status pm_mass_solve_noalloc(int dim, int n, double L, const float
     w.r2 = (float *)(base + 4 * kVecBytes);
     w.part = (float *)(base + 5 * kVecBytes);  // four vectors
     w.red = (double *)(base + kRedOff);
+    w.red4 = (float4 *)(base + kRed4Off);
     w.red_blocks = PM_NOALLOC_MAX_GRID;  // the solve's grid is clamped to the partials' capacity
     w.scal = (double *)(base + kScalOff);
     w.bar = (unsigned *)(base + kBarOff);
