@@ -1142,8 +1142,8 @@ __device__ __forceinline__ void pair_total(const double *part, int nblk, double 
 // from the network's input channels: channel 1 is PM_NET_RSCALE r / (h^2
 // max|A|); b is read from its fixed point. Partials (sum r^2, sum b^2, both in
 // units of (h^2 max|A|)^2), reduced by k_start_resid_final into out[f]. The
-// values are of order one and the products exact pairs (an FP64 instruction
-// costs 64 times an FP32 one). One thread per field over the blocks' partials
+// values are of order one, the products exact pairs and their sums Sum3: no fewer
+// bits than FP64, whose instructions cost 64 times as much. One thread per field over the blocks' partials
 // made the final kernels longer than the passes: 1024^2, 4 fields, 50 MB took 67 +
 // 73 us here and 53 + 74 us for k_alpha_partial and its final; now 34 + 9 and 47 + 9 us.
 __global__ void __launch_bounds__(256) k_start_resid(Geo g, const float *__restrict__ feat,
@@ -1153,14 +1153,17 @@ __global__ void __launch_bounds__(256) k_start_resid(Geo g, const float *__restr
     const int f = blockIdx.y, E = fix_exp(maxabs, f, hd);
     const float s = __uint_as_float(maxabs[f]);
     const float inv = s > 0.0f ? 1.0f / (s * hd) : 0.0f;
-    Dot2 rr, bb;
+    Sum3 rr{0.0f, 0.0f, 0.0f, 0}, bb = rr;
     for (ll i = (ll)blockIdx.x * blockDim.x + threadIdx.x; i < g.ncell; i += (ll)gridDim.x * blockDim.x) {
         const float r = feat[((ll)f * 2 + 1) * g.ncell + i];
         const float b = ldexpf((float)bfix[(ll)f * g.ncell + i], -E) * inv;
-        rr.fma_acc(r, r);
-        bb.fma_acc(b, b);
+        float p, e;
+        two_prod(r, r, p, e);
+        add_parts(rr, p, e, 0.0f);
+        two_prod(b, b, p, e);
+        add_parts(bb, p, e, 0.0f);
     }
-    pair_partial((double)rr.hi + (double)rr.lo, (double)bb.hi + (double)bb.lo, part);
+    pair_partial(total(rr), total(bb), part);
 }
 
 __global__ void k_start_resid_final(int nblk, const double *__restrict__ part, double *__restrict__ out) {
