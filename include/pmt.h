@@ -480,7 +480,8 @@ pm_status pm_profile_read(pm_ctx *ctx, double *ms, long long *calls, int reset);
  * edge or cell vertex, vertices inserted into a star (clips), sum of the star
  * sizes after each, summed over all particles and calls since the last reset,
  * each particle counted once, in the pass that completes its star.
- * counts[5] = stars the main pass gave up to the later passes,
+ * counts[5] = stars the main pass gave up to the later passes (how many depends
+ * on timing where ties are many),
  * counts[6] = stars of the later passes with more than 12 neighbours,
  * counts[7] = tests that float arithmetic could not decide and left to the
  * exact 128-bit predicate.

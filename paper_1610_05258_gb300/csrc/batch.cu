@@ -9,7 +9,7 @@
 //
 //   sort       caller arrays -> cell keys, one scan over all cells, canonical
 //              order, gather with max|A| per instance         (per particle / cell)
-//   stars      periodic Delaunay stars, two retry passes       (per particle)
+//   stars      periodic Delaunay stars, four passes            (per particle)
 //   rhs        exact right-hand side                           (per 16x16-cell tile)
 //   start      M^-1 b by separable circulant convolutions      (per 32x32 tile;
 //              or the delta assignment per particle, or zero)
@@ -568,7 +568,7 @@ pm_status pm_batch_create(pm_batch **out, int ninst, const int *n, const double 
          balloc(&w.maxabs, (ll)PM_MAXF * ninst) && balloc(&w.deg, NP) && balloc(&w.vol, NP) &&
          balloc(&w.nbr, (ll)PM_MAXDEG * NP) && balloc(&w.bfix, F * NC) && balloc(&w.b, F * NC) &&
          balloc(&w.r, F * NC) && balloc(&w.p, F * NC) && balloc(&w.q, F * NC) &&
-         balloc(&w.scal, 16LL * PM_MAXF * ninst) && balloc(&w.status, 1) && balloc(&w.nretry, 2) &&
+         balloc(&w.scal, 16LL * PM_MAXF * ninst) && balloc(&w.status, 1) && balloc(&w.nretry, 4) &&
          balloc(&b->d_inst, ninst) && balloc(&b->d_poff, ninst + 1) && balloc(&b->d_coff, ninst + 1) &&
          balloc(&b->d_rtile, ninst + 1) && balloc(&b->d_dtile, ninst + 1) && balloc(&b->d_order, ninst) &&
          balloc((unsigned char **)&b->d_taps, (ll)direct_taps_bytes() * ninst) && balloc(&b->d_px, ninst) &&

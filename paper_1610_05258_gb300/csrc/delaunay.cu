@@ -3,16 +3,18 @@
 // the periodically ordered particles (1D); and particle volumes
 // v_mu = int psi_mu (Sec. 2.1, Eq. part_v).
 //
-// 2D: the Delaunay star of a particle p comes from three kinds of passes.
+// 2D: the Delaunay star of a particle p comes from one of four passes.
 //  * k_delaunay, one thread per particle: the star is the convex hull of the
-//    particles around p after inversion about p, found with float arithmetic
-//    whose every decision is certain (see below).
+//    particles around p after inversion about p (the manner of quickhull), found
+//    with float arithmetic whose every decision is certain (see below).
 //  * k_delaunay_wide, 8 lanes per particle, for what the first pass gives up:
 //    the same hull with a wider search, undecided tests made exactly.
-//  * k_delaunay_retry, one thread per particle, for the rest (regular lattices,
-//    stars of more than 24 neighbours, coincident particles, sets too sparse to
-//    certify): p's Voronoi cell is clipped by the bisectors of nearby
-//    particles, scanned ring by ring of mesh cells. The cell is a cyclic list of
+//  * k_delaunay_exact, one thread per particle, for many ties (lattices), and
+//    k_delaunay_last, a warp per particle, for the rest (crowds inside a cell, jumps
+//    of density, coincident particles, sets too sparse to certify, stars of more
+//    than 24 neighbours, which are refused): p's Voronoi cell is clipped by the
+//    bisectors of nearby particles, scanned ring by ring of mesh cells. The cell
+//    is a cyclic list of
 //    neighbours q_k; its vertex k is the circumcentre of (p, q_k, q_k+1). A
 //    candidate s removes vertex k iff s lies strictly inside the circle
 //    through (p, q_k, q_k+1): the in-circle predicate, equivalently
@@ -25,14 +27,17 @@
 // |r|^2 + eps^rank, rank = caller index. Because every decision is exact and
 // the perturbation is a property of the point set, the stars of all particles
 // agree, whatever pass made them: every triangle (p, a, b) appears in the stars
-// of p, a and b.
+// of p, a and b. Its order does not tell the pass either (start_key).
 //
 // Measured (16.8M clustered particles on 2048^2, all passes): 6.1 ms, against
-// 17.2 ms with the clipping alone as the main pass. Clipping ran 853 warp
-// instructions per particle with 8 of 32 lanes active, every lane at its own
-// candidate and its own polygon; the hull runs about 240 (+ 65 in the wide
-// pass, for 4 % of the particles) with 26 lanes active. Smallest calls gain
-// too, 262,144 particles from 518 to 170 us: no lane walks a long chain.
+// 17.2 ms with the clipping alone as the main pass, every lane at its own
+// candidate and its own polygon. Smallest calls gain too, 262,144 particles from
+// 518 to 170 us: no lane walks a long chain. Sets that the hull cannot take (clipping
+// alone, a hull attempt and one thread each after it, now): 1M on a square lattice
+// 427, 710, 487 us; 1M with x = u^2 2959, 4027, 2179 us; 80,000 with 20,000 inside
+// a quarter of a cell 35.7, 44.9, 5.8 ms.
+#include <algorithm>
+
 #include "internal.cuh"
 
 PM_DEBUG_DECL(delaunay)
@@ -82,11 +87,12 @@ __device__ __forceinline__ int prio(int enc, const int *__restrict__ perm) {
     return id >= PM_VIRT ? 0x7ffffff0 + (id - PM_VIRT) : __ldg(perm + id);
 }
 
-#define R1BLK 32    // threads per block of the first retry pass
-#define R1CAP 12    // polygon capacity of the first retry pass (17 warps per SM)
-#define RBLK 32     // threads per block of the last retry pass
-#define RCAP 24     // polygon capacity of the last retry pass (= PM_MAXDEG)
-#define ST_OVERFLOW 0x40000000  // internal: the cell outgrew the main pass's capacity
+#define EBLK 64     // threads per block of the exact pass
+#define EMINB 12    // resident blocks per SM (24 warps, what the polygons in shared memory leave)
+#define ECAP 9      // polygon capacity of the exact pass
+#define LBLK 128    // threads per block of the last pass, a warp per particle
+#define LCAP 31     // polygon capacity of the last pass (vertex masks are 32 bits)
+#define ST_OVERFLOW 0x40000000  // internal: the cell outgrew the exact pass's capacity
 
 // Float circumcentre c of (0, a, b) and a bound e on the error of each of its
 // components (infinite when the triangle is too flat to bound). Inputs are
@@ -223,7 +229,7 @@ __device__ __forceinline__ int clip_by(PolyS<NB> P, int &m, float &R2, int sx, i
     if (cnt >= m || __popc(starts) != 1) return ST_RANGE;
     const int i0 = __ffs(starts) - 1;  // first removed vertex; q_i0 is kept
     const int nd = cnt - 1;            // neighbours q_{i0+1..i0+nd} are removed
-    if (m - nd + 1 > CAP) return CAP < RCAP ? ST_OVERFLOW : ST_DEGREE;
+    if (m - nd + 1 > CAP) return CAP < LCAP ? ST_OVERFLOW : ST_DEGREE;
     PM_CHK(m - nd + 1 <= CAP, 204, return ST_DEGREE)
     const int4 S = make_int4(sx, sy, sidx | (code << 28), 0);
     int ipos;
@@ -295,6 +301,117 @@ __device__ __forceinline__ void ring1(int i, int &dx, int &dy) {
     dy = i < 3 ? -1 : (i < 5 ? 0 : 1);
 }
 
+// Star entry of sorted neighbour s at Xs: index and image code of its minimal
+// image; (rx, ry) its offset from p.
+__device__ __forceinline__ int star_entry(int s, uint2 Xs, uint2 Xp, int &rx, int &ry) {
+    rx = (int)(Xs.x - Xp.x);
+    ry = (int)(Xs.y - Xp.y);
+    const int ox = rx >= 0 ? (Xs.x < Xp.x ? 1 : 0) : (Xs.x > Xp.x ? -1 : 0);
+    const int oy = ry >= 0 ? (Xs.y < Xp.y ? 1 : 0) : (Xs.y > Xp.y ? -1 : 0);
+    return s | (((ox + 1) * 3 + (oy + 1)) << 28);
+}
+
+__device__ __forceinline__ float rcp_approx(float x) {
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+
+// Inversion about Xp, in units of 1 / cell (cw: torus units per cell); the
+// origin for p itself. The same bits in every kernel (explicit roundings).
+struct Inversion {
+    uint2 Xp;
+    float cw;
+    __device__ __forceinline__ float of(int rx, int ry, float &ux, float &uy) const {
+        const float sx = (float)rx, sy = (float)ry, d2 = __fmaf_rn(sx, sx, __fmul_rn(sy, sy));
+        const float iv = d2 > 0.0f ? __fmul_rn(rcp_approx(d2), cw) : 0.0f;
+        ux = __fmul_rn(sx, iv);
+        uy = __fmul_rn(sy, iv);
+        return d2;
+    }
+    __device__ __forceinline__ float operator()(uint2 X, float &ux, float &uy) const {
+        return of((int)(X.x - Xp.x), (int)(X.y - Xp.y), ux, uy);
+    }
+};
+
+// A star is stored counter-clockwise from the neighbour of largest start_key,
+// where the main pass begins its hull: the inversion farthest in x, its low 6
+// bits dropped, then the place in the main pass's list (row of cells, beyond the
+// box edge in x or not, sorted index). So a star is the same array whatever pass
+// made it.
+__device__ __forceinline__ ull start_key(const Inversion &inv, int rx, int ry, int entry, int n, int cy) {
+    float ux, uy;
+    inv.of(rx, ry, ux, uy);
+    const int code = (unsigned)entry >> 28, ox = code / 3 - 1, oy = code % 3 - 1;
+    const int dy = cell_of(inv.Xp.y + (unsigned)ry, n) + oy * n - cy;
+    return (ull)(ux > 0.0f ? __float_as_uint(ux) >> 6 : 0u) << 34 | (ull)(dy + 16) << 29 | (ull)(ox != 0) << 28 |
+           (ull)(entry & 0x0fffffff);
+}
+
+// Up to four particles around p that a hull pass found before it gave p up, -1
+// for none; kept in p's star slots until its star is written. The last pass
+// clips by them first: the cell is then near its final size, and most other
+// candidates fail the distance test.
+#define NSEED 4
+struct Seeds {
+    int s[NSEED];
+    __device__ __forceinline__ void load(const int *nbr, ll np, int p) {
+        s[0] = nbr[p];
+#pragma unroll
+        for (int k = 1; k < NSEED; ++k) s[k] = s[0] < 0 ? -1 : nbr[(ll)k * np + p];
+    }
+    __device__ __forceinline__ bool has(int i) const {
+        bool h = false;
+#pragma unroll
+        for (int k = 0; k < NSEED; ++k) h |= s[k] == i;
+        return h;
+    }
+    // seed k, if it is one and not an earlier one again
+    __device__ __forceinline__ bool take(int k, int p) const {
+        bool ok = s[k] >= 0 && s[k] != p;
+        for (int j = 0; j < k; ++j) ok = ok && s[j] != s[k];
+        return ok;
+    }
+};
+
+// The initial cell: the square cut out by four virtual points at distance
+// B = 2^30, the largest coordinate the exact predicates take. A vertex
+// involving a virtual point is at least 2^29 from p, which the scan
+// (< 2^30) can never certify, so a certified cell is bounded by real
+// particles only; a cell still touching a virtual point after the last
+// ring is reported as ST_SPARSE. Returns the bound R2 of its vertices.
+template <int NB>
+__device__ __forceinline__ float initial_cell(PolyS<NB> P) {
+    const int t = P.t, B = 1 << 30;
+    const float hb = 0.5f * (float)B;
+    const float rb = 2.0f * hb * hb * 1.0001f;
+    P.q[0][t] = make_int4(B, 0, PM_VIRT + 0, 0);
+    P.q[1][t] = make_int4(0, B, PM_VIRT + 1, 0);
+    P.q[2][t] = make_int4(-B, 0, PM_VIRT + 2, 0);
+    P.q[3][t] = make_int4(0, -B, PM_VIRT + 3, 0);
+    P.v[0][t] = make_float4(hb, hb, 0.0f, rb);
+    P.v[1][t] = make_float4(-hb, hb, 0.0f, rb);
+    P.v[2][t] = make_float4(-hb, -hb, 0.0f, rb);
+    P.v[3][t] = make_float4(hb, -hb, 0.0f, rb);
+    return rb;
+}
+
+// Clip the initial cell by the seeds.
+template <int CAP, int NB, bool COUNT>
+__device__ __forceinline__ int clip_by_seeds(PolyS<NB> P, int &m, float &R2, const Seeds &seeds, int p, uint2 Xp,
+                                             const uint2 *__restrict__ pos, int &pp, const int *__restrict__ perm,
+                                             WorkCount &wc) {
+    for (int k = 0; k < NSEED; ++k) {
+        if (!seeds.take(k, p)) continue;
+        int rx, ry;
+        const int e = star_entry(seeds.s[k], __ldg(pos + seeds.s[k]), Xp, rx, ry);
+        if ((rx | ry) == 0) return ST_DUP;
+        const int err = clip_by<CAP, NB, COUNT>(P, m, R2, rx, ry, seeds.s[k], (unsigned)e >> 28, p, pp, perm, wc);
+        if (err) return err;
+    }
+    return 0;
+}
+
 // The Voronoi cell (star) of one particle p. Candidates are taken ring by
 // ring of cells around p until the cell is certified. A neighbouring cell is
 // skipped when its box is farther than 2 max|c_k| (none of its points can cut
@@ -311,24 +428,7 @@ __device__ __forceinline__ int star_of(PolyS<NB> P, int p, const Geo &g, ll np, 
     const int t = P.t;
     const int n = g.n;
     int m = 4;
-    // Initial cell: the square cut out by four virtual points at distance
-    // B = 2^30, the largest coordinate the exact predicates take. A vertex
-    // involving a virtual point is at least 2^29 from p, which the scan
-    // (< 2^30) can never certify, so a certified cell is bounded by real
-    // particles only; a cell still touching a virtual point after the last
-    // ring is reported as ST_SPARSE.
-    const int B = 1 << 30;
-    const float hb = 0.5f * (float)B;
-    const float rb = 2.0f * hb * hb * 1.0001f;
-    P.q[0][t] = make_int4(B, 0, PM_VIRT + 0, 0);
-    P.q[1][t] = make_int4(0, B, PM_VIRT + 1, 0);
-    P.q[2][t] = make_int4(-B, 0, PM_VIRT + 2, 0);
-    P.q[3][t] = make_int4(0, -B, PM_VIRT + 3, 0);
-    P.v[0][t] = make_float4(hb, hb, 0.0f, rb);
-    P.v[1][t] = make_float4(-hb, hb, 0.0f, rb);
-    P.v[2][t] = make_float4(-hb, -hb, 0.0f, rb);
-    P.v[3][t] = make_float4(hb, -hb, 0.0f, rb);
-    float R2 = rb;
+    float R2 = initial_cell(P);
     const uint2 Xp = pos[p];
     const int cx = cell_of(Xp.x, n), cy = cell_of(Xp.y, n);
     const float cw = 4294967296.0f / (float)n;
@@ -408,10 +508,22 @@ __device__ __forceinline__ int star_of(PolyS<NB> P, int p, const Geo &g, ll np, 
         if ((P.q[k][t].z & 0x0fffffff) >= PM_VIRT) return ST_SPARSE;
     if (m > PM_MAXDEG) return ST_DEGREE;
     PM_CHK(m >= 3 && m <= PM_MAXDEG, 203, return ST_DEGREE)
-    ll area2 = 0;
-    int4 A = P.q[0][t];
+    const Inversion inv{Xp, cw};
+    int k0 = 0;
+    ull best = 0;
     for (int k = 0; k < m; ++k) {
-        int4 Bq = P.q[k + 1 == m ? 0 : k + 1][t];
+        const int4 q = P.q[k][t];
+        const ull key = start_key(inv, q.x, q.y, q.z, n, cy);
+        if (key > best) {
+            best = key;
+            k0 = k;
+        }
+    }
+    ll area2 = 0;
+    int4 A = P.q[k0][t];
+    for (int k = 0; k < m; ++k) {
+        k0 = k0 + 1 == m ? 0 : k0 + 1;
+        int4 Bq = P.q[k0][t];
         area2 += (ll)A.x * Bq.y - (ll)A.y * Bq.x;
         nbr[(ll)k * np + p] = A.z;
         A = Bq;
@@ -503,11 +615,6 @@ __device__ __forceinline__ float fma_sat(float a, float b, float c) {
     asm("fma.rn.sat.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
     return r;
 }
-__device__ __forceinline__ float rcp_approx(float x) {
-    float r;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-    return r;
-}
 __device__ __forceinline__ float sqrt_approx(float x) {
     float r;
     asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
@@ -567,55 +674,30 @@ __device__ __forceinline__ void row_range(const int *__restrict__ cell_start, in
     }
 }
 
-// Star entry of sorted neighbour s at Xs: index and image code of its minimal
-// image; (rx, ry) its offset from p.
-__device__ __forceinline__ int star_entry(int s, uint2 Xs, uint2 Xp, int &rx, int &ry) {
-    rx = (int)(Xs.x - Xp.x);
-    ry = (int)(Xs.y - Xp.y);
-    const int ox = rx >= 0 ? (Xs.x < Xp.x ? 1 : 0) : (Xs.x > Xp.x ? -1 : 0);
-    const int oy = ry >= 0 ? (Xs.y < Xp.y ? 1 : 0) : (Xs.y > Xp.y ? -1 : 0);
-    return s | (((ox + 1) * 3 + (oy + 1)) << 28);
-}
-
 // Star written; needs a wider search; needs exact tests; undecided tests.
 enum { HULL_DONE = 1, HULL_WIDER = 2, HULL_EXACT = 3, HULL_UNSURE = 4 };
-
-// Inversion about Xp, in units of 1 / cell (cw: torus units per cell); the
-// origin for p itself.
-struct Inversion {
-    uint2 Xp;
-    float cw;
-    __device__ __forceinline__ float operator()(uint2 X, float &ux, float &uy) const {
-        const float sx = (float)(int)(X.x - Xp.x), sy = (float)(int)(X.y - Xp.y), d2 = sx * sx + sy * sy;
-        const float iv = d2 > 0.0f ? rcp_approx(d2) * cw : 0.0f;
-        ux = sx * iv;
-        uy = sy * iv;
-        return d2;
-    }
-};
 
 // All lanes of the warp call this together (live: the lane has a particle).
 // ids: the block's list columns, HL + 4 rows (the last rows take the candidates
 // of a full list); stk: the stack of hull vertices (u, slot).
 template <bool COUNT>
-__device__ __forceinline__ int star_hull(int (*ids)[HBLK], float4 (*stk)[HBLK], bool live, int p, const Geo &g, ll np,
+__device__ __forceinline__ int star_hull(int (*ids)[HBLK], float4 (*stk)[HBLK], bool live, int p, uint2 Xp, int ties, const Geo &g, ll np,
                                          const uint2 *__restrict__ pos, const int *__restrict__ cell_start,
-                                         const int *__restrict__ perm, int *__restrict__ nbr,
-                                         unsigned char *__restrict__ deg, float *__restrict__ vol, float vol_scale,
-                                         WorkCount &wc) {
+                                         int *__restrict__ nbr, unsigned char *__restrict__ deg,
+                                         float *__restrict__ vol, float vol_scale, WorkCount &wc) {
     const int t = (int)threadIdx.x, n = g.n;
-    const uint2 Xp = live ? pos[p] : make_uint2(0u, 0u);
     const Inversion inv{Xp, 4294967296.0f / (float)n};
     int *const col = &ids[0][0];
     int q = t;
     float ri2 = 0.0f;
+    const bool mostly_ties = 3LL * ties > (ll)blockIdx.x * HBLK;  // of the blocks before this one (see on_lattice)
     if (live) {
         const int cx = cell_of(Xp.x, n), cy = cell_of(Xp.y, n);
         const float fx = frac_f(Xp.x, n), fy = frac_f(Xp.y, n);
         const float r = search_radius(g, cell_start, cx, cy, HN, HRMAX), rs = r * 1.0001f + 1e-6f;
         const float r2 = (r * inv.cw) * (r * inv.cw);
         ri2 = rcp_approx(r * r) * 1.0002f;
-        const int y1 = (int)floorf(fy + rs);
+        const int y1 = mostly_ties ? -100 : (int)floorf(fy + rs);
         for (int dy = (int)floorf(fy - rs); dy <= y1; ++dy) {
             int s0, s1, t0, t1;
             row_range(cell_start, n, cx, cy, dy, fx, fy, rs, s0, s1, t0, t1);
@@ -654,7 +736,10 @@ __device__ __forceinline__ int star_hull(int (*ids)[HBLK], float4 (*stk)[HBLK], 
     if (COUNT) wc.tested += cnt;
     int state = !live || cnt < 4 || cnt >= HL ? HULL_WIDER : 0;  // 0: running
     const int used = __reduce_max_sync(0xffffffffu, state == 0 ? cnt : 0);
-    if (used == 0) return state;
+    if (used == 0) {
+        if (live) nbr[p] = -1;
+        return mostly_ties ? HULL_EXACT : state;
+    }
     // The inverted candidates, in registers; slots past the lane's own list
     // hold the origin, which is never beyond an edge. The extremes in x and y
     // start the hull: the largest bit pattern as a signed integer is the
@@ -694,6 +779,8 @@ __device__ __forceinline__ int star_hull(int (*ids)[HBLK], float4 (*stk)[HBLK], 
     // U >= |u| of every candidate (the tags take at most 2^-17 off a component)
     const float ex = fmaxf(__int_as_float(xmax), -__uint_as_float(xmin)), ey = fmaxf(__int_as_float(ymax), -__uint_as_float(ymin));
     const float U27 = 2.7e-6f * 1.00003f * sqrt_approx(ex * ex + ey * ey);
+    const unsigned ext = (unsigned)(xmax & 63) | (ymin & 63u) << 8 | (xmin & 63u) << 16 | (unsigned)(ymax & 63) << 24;
+    const bool seeded = state == 0;
     int a = 0, b = 0, m = 0, depth = 0;  // edge (a, b); the stack's top, b, is row depth; row 0 closes the cycle
     ull out = 0;
     float ax = 0.0f, ay = 0.0f, bx = 0.0f, by = 0.0f;
@@ -707,7 +794,7 @@ __device__ __forceinline__ int star_hull(int (*ids)[HBLK], float4 (*stk)[HBLK], 
         by = ay;
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
-            const int v = (int)((k == 0 ? ymin : (k == 1 ? xmin : (unsigned)ymax)) & 63u);
+            const int v = (int)(ext >> (8 * (k + 1))) & 63;
             if (v != b && v != a) {
                 b = v;
                 inv(__ldg(pos + ids[b][t]), bx, by);
@@ -778,8 +865,16 @@ __device__ __forceinline__ int star_hull(int (*ids)[HBLK], float4 (*stk)[HBLK], 
     // A few undecided lanes go to the wide pass, which decides exactly; where
     // they are many (a regular lattice) the exact passes are the faster way.
     if (__popc(__ballot_sync(0xffffffffu, state == HULL_UNSURE)) > 4 && state == HULL_UNSURE) state = HULL_EXACT;
-    if (state != HULL_DONE || m < 3) return state == HULL_EXACT ? HULL_EXACT : HULL_WIDER;
-    // the star, counter-clockwise from the nearest particle
+    if (state != HULL_DONE || m < 3) {
+        if (live) {
+            const bool keep = seeded && state != HULL_EXACT;
+            nbr[p] = keep ? ids[ext & 63][t] : -1;
+            if (keep)
+                for (int k = 1; k < NSEED; ++k) nbr[(ll)k * np + p] = ids[(ext >> (8 * k)) & 63][t];
+        }
+        return state == HULL_EXACT ? HULL_EXACT : HULL_WIDER;
+    }
+    // the star, counter-clockwise from the largest x of the inversions
     ll area2 = 0;
     int fx0 = 0, fy0 = 0, px = 0, py = 0;
     for (int k = 0; k < m; ++k) {
@@ -817,25 +912,68 @@ __device__ __forceinline__ void push_list(bool add, int p, ll np, int *__restric
     }
 }
 
-// The lists of the particles that the hull passes give up: wide[] with
-// counts[0] entries (after the main pass) and exact[] with counts[1] entries.
+// The particles that a pass gives up: to the wide pass (counts[0]), to the exact
+// pass (counts[1]: ties, from the main pass), to the last pass (counts[2], from both);
+// counts[3]: the exact pass's next entry.
 struct Lists {
-    int *wide, *exact, *counts;
+    int *wide, *exact, *last, *counts;
 };
 
+// A warp goes to the exact pass without an attempt (the attempt costs a third to
+// all of the hull, and the exact pass then starts over) in two cases:
+//  - (here) its particles stand on a rectangular lattice along the axes: nearly all
+//    share a coordinate with the one before or after them, and the next row above
+//    has a particle straight above them, so every four are a tie;
+//  - (in star_hull) of the particles of the blocks before it more than a third were
+//    ties: hull and exact pass take about 270 + 450 f us for 1M particles with a
+//    fraction f of ties, the exact pass alone 420. A block reads the count as it
+//    stands, so its route may differ from run to run; its stars do not.
+__device__ __forceinline__ bool on_lattice(bool live, uint2 X, const Geo &g, const uint2 *__restrict__ pos,
+                                           const int *__restrict__ cell_start) {
+    const unsigned FULL = 0xffffffffu;
+    const uint2 N = make_uint2(__shfl_down_sync(FULL, X.x, 1), __shfl_down_sync(FULL, X.y, 1));
+    const bool row = (threadIdx.x & 31) < 31 && (X.x == N.x || X.y == N.y);
+    const unsigned rows = __ballot_sync(FULL, live && row);
+    if (__popc(rows | rows << 1) < 28) return false;
+    bool above = false;
+    if (live) {
+        const int n = g.n, cx = cell_of(X.x, n), cy = cell_of(X.y, n);
+        unsigned dmin = 0xffffffffu;
+        for (int h = 0; h < 2; ++h) {
+            const int *cs = cell_start + (ll)(cy + h == n ? 0 : cy + h) * n + cx;
+            const int s0 = __ldg(cs), s1 = min(__ldg(cs + 1), s0 + 16);
+            for (int s = s0; s < s1; ++s) {
+                const uint2 Y = __ldg(pos + s);
+                const unsigned d = Y.y - X.y;  // up, modulo the box
+                if (d == 0 || d > 0x7fffffffu) continue;
+                if (d < dmin) above = false;
+                if (d <= dmin) above |= Y.x == X.x;
+                dmin = min(dmin, d);
+            }
+        }
+    }
+    return __popc(__ballot_sync(FULL, above)) >= 24;
+}
+
 // Counters: wsum[0..4] the work of completed cells, wsum[5] the cells given
-// up by the main pass, wsum[6] those given up by the first exact pass.
+// up by the main pass, wsum[6] large stars of the later passes.
 template <bool COUNT>
 __global__ void __launch_bounds__(HBLK, HMINB) k_delaunay(Geo g, ll np, const uint2 *__restrict__ pos,
-                                                   const int *__restrict__ cell_start, const int *__restrict__ perm,
-                                                   int *__restrict__ nbr, unsigned char *__restrict__ deg,
-                                                   float *__restrict__ vol, float vol_scale, Lists L, ull *__restrict__ wsum) {
+                                                   const int *__restrict__ cell_start, int *__restrict__ nbr,
+                                                   unsigned char *__restrict__ deg, float *__restrict__ vol,
+                                                   float vol_scale, Lists L, ull *__restrict__ wsum) {
     __shared__ int ids[HL + 4][HBLK];
     __shared__ float4 stk[HDEG][HBLK];
     const ll pl = (ll)blockIdx.x * HBLK + threadIdx.x;
     const bool live = pl < np;
+    const int ties = L.counts[1];
+    const uint2 Xp = live ? pos[pl] : make_uint2(0u, 0u);
     WorkCount wc;
-    const int e = star_hull<COUNT>(ids, stk, live, (int)pl, g, np, pos, cell_start, perm, nbr, deg, vol, vol_scale, wc);
+    int e = HULL_EXACT;
+    if (!on_lattice(live, Xp, g, pos, cell_start))
+        e = star_hull<COUNT>(ids, stk, live, (int)pl, Xp, ties, g, np, pos, cell_start, nbr, deg, vol, vol_scale, wc);
+    else if (live)
+        nbr[pl] = -1;
     if (COUNT && live && e != HULL_DONE) {
         wc = WorkCount{};
         wc.over = 1;
@@ -1048,6 +1186,7 @@ __device__ __forceinline__ int star_wide(WideS &G, bool live, int p, const Geo &
                 result = HULL_EXACT;
             else
                 r = fminf(state == 1 && need2 < 1e30f ? sqrt_approx(need2) * 1.001f : 1.6f * r, rlim);
+            if (state == 1 && result != HULL_DONE && sub < NSEED) nbr[(ll)sub * np + p] = G.id[G.out[sub * m / NSEED]];
             if (result == 0 && state == 1) {  // the next search drops what lies inside this hull
                 edges = m;
                 for (int k = sub; k < m; k += 8) {
@@ -1063,11 +1202,28 @@ __device__ __forceinline__ int star_wide(WideS &G, bool live, int p, const Geo &
         __syncwarp();
     }
     const bool done = result == HULL_DONE;
+    ull key = 0;
+    int first_k = 0;
+    for (int k = sub; done && k < m; k += 8) {
+        const int s = G.id[G.out[k]];
+        int rx, ry;
+        const int e = star_entry(s, __ldg(pos + s), Xp, rx, ry);
+        const ull q = start_key(inv, rx, ry, e, n, cy);
+        if (q > key) {
+            key = q;
+            first_k = k;
+        }
+    }
+    ull best = key;
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) best = max(best, (ull)__shfl_xor_sync(FULL, best, o));
+    first_k = __shfl_sync(FULL, first_k, sh + __ffs((__ballot_sync(FULL, key == best) >> sh) & 0xffu) - 1);
     ll area2 = 0;
     for (int k = sub; done && k < m; k += 8) {
         const int s = G.id[G.out[k]], s2 = G.id[G.out[k + 1 == m ? 0 : k + 1]];
+        const int slot = k >= first_k ? k - first_k : k + m - first_k;
         int rx, ry, qx, qy;
-        nbr[(ll)k * np + p] = star_entry(s, __ldg(pos + s), Xp, rx, ry);
+        nbr[(ll)slot * np + p] = star_entry(s, __ldg(pos + s), Xp, rx, ry);
         star_entry(s2, __ldg(pos + s2), Xp, qx, qy);
         area2 += (ll)rx * qy - (ll)ry * qx;
     }
@@ -1077,7 +1233,7 @@ __device__ __forceinline__ int star_wide(WideS &G, bool live, int p, const Geo &
     if (done && sub == 0) {
         deg[p] = (unsigned char)m;
         vol[p] = (float)area2 * vol_scale;
-        if (COUNT && m > R1CAP) wc.over++;
+        if (COUNT && m > 12) wc.over++;
     }
     return done ? HULL_DONE : HULL_EXACT;
 }
@@ -1099,68 +1255,248 @@ __global__ void __launch_bounds__(WBLK) k_delaunay_wide(Geo g, ll np, const uint
         const int e = star_wide<COUNT>(G[gid], live, p, g, np, pos, cell_start, perm, nbr, deg, vol, vol_scale, wc);
         const bool over = live && e != HULL_DONE && (threadIdx.x & 7) == 0;
         if (COUNT && over) wc = before;
-        push_list(over, p, np, L.exact, L.counts + 1);
+        push_list(over, p, np, L.last, L.counts + 2);
     }
     add_counts<COUNT>(wc, wsum, 6);
 }
 
-// Exact passes over the exact list (grid-stride). The first (capacity R1CAP,
-// LAST false) marks a particle whose cell outgrows it by storing ~p in its list
-// entry; the last (capacity RCAP, LAST true) takes only the marked entries.
-template <int CAP, int NB, bool LAST, bool COUNT>
-__global__ void __launch_bounds__(NB) k_delaunay_retry(Geo g, ll np, const uint2 *__restrict__ pos,
-                                                       const int *__restrict__ cell_start,
-                                                       const int *__restrict__ perm, int *__restrict__ nbr,
-                                                       unsigned char *__restrict__ deg, float *__restrict__ vol,
-                                                       float vol_scale, int *__restrict__ status,
-                                                       int *__restrict__ retry, const int *__restrict__ nretry,
-                                                       ull *__restrict__ wsum) {
-    __shared__ int4 sq[CAP][NB];
-    __shared__ float4 sv[CAP][NB];
-    const int cnt = *nretry;
+// The mesh of a particle: one mesh, or the particle's instance of a batch (from
+// the packed offsets; stars hold packed sorted indices, < 2^28 in total).
+struct OneMesh {
+    Geo g;
+    ll np;
+    const int *cell_start;
+    float vol_scale;
+    __device__ __forceinline__ Geo geo(int) const { return g; }
+    __device__ __forceinline__ const int *cells(int) const { return cell_start; }
+    __device__ __forceinline__ float scale(int) const { return vol_scale; }
+    __device__ __forceinline__ int instance(int) const { return 0; }
+};
+struct BatchMesh {
+    BTab t;
+    ll np;
+    const int *cell_start;
+    __device__ __forceinline__ Geo geo(int k) const { return batch_geo(t, k); }
+    __device__ __forceinline__ const int *cells(int k) const { return cell_start + __ldg(t.coff + k); }
+    __device__ __forceinline__ float scale(int k) const { return t.inst[k].vol_scale; }
+    __device__ __forceinline__ int instance(int p) const { return find_slot(t.poff, t.ninst, (ll)p); }
+};
+
+// From this many particles on the exact pass takes its list, one thread each, and
+// leaves those whose cell outgrows ECAP to the last pass; a shorter list goes to
+// the last pass as it is.
+#define EXACT_MIN 4096
+
+__device__ __forceinline__ void fail_star(int err, int p, unsigned char *deg, float *vol, int *status) {
+    atomicOr(status, (err & ~ST_OVERFLOW) | (err & ST_OVERFLOW ? ST_DEGREE : 0));
+    deg[p] = 0;
+    vol[p] = 0.0f;
+}
+
+template <class Mesh, bool COUNT>
+__global__ void __launch_bounds__(EBLK, EMINB) k_delaunay_exact(Mesh M, const uint2 *__restrict__ pos,
+                                                                const int *__restrict__ perm, int *__restrict__ nbr,
+                                                                unsigned char *__restrict__ deg,
+                                                                float *__restrict__ vol, int *__restrict__ status,
+                                                                Lists L, ull *__restrict__ wsum) {
+    __shared__ int4 sq[ECAP][EBLK];
+    __shared__ float4 sv[ECAP][EBLK];
+    const int cnt = L.counts[1];
+    if (cnt < EXACT_MIN) return;
     WorkCount wc;
-    PolyS<NB> P{sq, sv, (int)threadIdx.x};
-    for (ll j = (ll)blockIdx.x * NB + threadIdx.x; j < cnt; j += (ll)gridDim.x * NB) {
-        int p = retry[j];
-        if (LAST) {
-            if (p >= 0) continue;
-            p = ~p;
+    PolyS<EBLK> P{sq, sv, (int)threadIdx.x};
+    const int lane = threadIdx.x & 31;
+    for (;;) {  // a warp takes the next 32
+        int j = 0;
+        if (lane == 0) j = atomicAdd(L.counts + 3, 32);
+        j = __shfl_sync(0xffffffffu, j, 0);
+        if (j >= cnt) break;
+        j += lane;
+        bool over = false;
+        int p = 0;
+        if (j < cnt) {
+            p = L.exact[j];
+            PM_CHK(p >= 0 && p < M.np, 206, p = 0)
+            const WorkCount before = wc;
+            const int k = M.instance(p);
+            const int err = star_of<ECAP, EBLK, COUNT>(P, p, M.geo(k), M.np, pos, M.cells(k), perm, nbr, deg, vol,
+                                                       M.scale(k), wc);
+            over = err == ST_OVERFLOW;
+            if (COUNT && over) wc = before;
+            if (err && !over) fail_star(err, p, deg, vol, status);
         }
-        PM_CHK(p >= 0 && p < np, 206, continue)
-        const WorkCount before = wc;
-        const int err = star_of<CAP, NB, COUNT>(P, p, g, np, pos, cell_start, perm, nbr, deg, vol, vol_scale, wc);
-        if (!LAST && err == ST_OVERFLOW) {
-            if (COUNT) {
-                wc = before;
-                wc.over++;
-            }
-            retry[j] = ~p;
-        } else if (err) {
-            atomicOr(status, (err & ~ST_OVERFLOW) | (err == ST_OVERFLOW ? ST_DEGREE : 0));
-            deg[p] = 0;
-            vol[p] = 0.0f;
-        }
+        push_list(over, p, M.np, L.last, L.counts + 2);
     }
-    add_counts<COUNT>(wc, wsum, 6);  // the first exact pass's give-ups (none in the last)
+    add_counts<COUNT>(wc, wsum, 6);
+}
+
+// ---------------------------------------------------------------------------
+// Last pass: the cell of a particle by a warp. The lanes read a cell's particles
+// 32 at a time and drop those that certainly cut nothing; what is left is clipped
+// by lane 0, one after another. It takes the few particles whose neighbourhood is
+// unlike the mean density (a blob inside a cell, a jump of density), where one
+// thread walks over thousands of candidates with a load latency each: 80,000
+// particles with 20,000 in a blob of a quarter of a cell, 33.5 + 7.3 ms by one
+// thread each.
+// ---------------------------------------------------------------------------
+template <bool COUNT>
+__device__ __forceinline__ int star_warp(PolyS<LBLK / 32> P, int p, const Geo &g, ll np, const uint2 *__restrict__ pos,
+                                         const int *__restrict__ cell_start, const int *__restrict__ perm,
+                                         int *__restrict__ nbr, unsigned char *__restrict__ deg,
+                                         float *__restrict__ vol, float vol_scale, WorkCount &wc) {
+    constexpr int NB = LBLK / 32;
+    const unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x & 31, t = P.t, n = g.n;
+    const uint2 Xp = pos[p];
+    const int cx = cell_of(Xp.x, n), cy = cell_of(Xp.y, n);
+    const float cw = 4294967296.0f / (float)n;
+    const float fxl = (float)cell_frac(Xp.x, n) / (float)n, fyl = (float)cell_frac(Xp.y, n) / (float)n;
+    const float edge = fminf(fminf(fxl, cw - fxl), fminf(fyl, cw - fyl));
+    const int rmax = max(0, min(PM_RCAP, n / 4 - 1));
+    Seeds seeds;
+    seeds.load(nbr, np, p);
+    int m = 4, pp = -2, err = 0;
+    float R2 = 0.0f;
+    if (lane == 0) {
+        R2 = initial_cell(P);
+        err = clip_by_seeds<LCAP, NB, COUNT>(P, m, R2, seeds, p, Xp, pos, pp, perm, wc);
+    }
+    __syncwarp();
+    m = __shfl_sync(FULL, m, 0);
+    R2 = __shfl_sync(FULL, R2, 0);
+    err = __shfl_sync(FULL, err, 0);
+    bool done = false;
+    for (int r = 0; r <= rmax && !done && !err; ++r) {
+        const int ncells = r == 0 ? 1 : 8 * r;
+        for (int c0 = 0; c0 < ncells && !err; c0 += 32) {
+            // the ring's cells, one a lane; those that can matter are visited
+            const int ci = c0 + lane;
+            int dx = 0, dy = 0;
+            if (r > 0) {
+                if (ci < 2 * r + 1) { dx = ci - r; dy = -r; }
+                else if (ci < 4 * r + 2) { dx = ci - (3 * r + 1); dy = r; }
+                else if (ci < 6 * r + 1) { dx = -r; dy = ci - (5 * r + 1); }
+                else { dx = r; dy = ci - (7 * r); }
+            }
+            int s0 = 0, s1 = 0, ox = 0, oy = 0;
+            const float bd = r == 0 ? 0.0f : box_dist2(dx, dy, fxl, fyl, cw);
+            if (ci < ncells && bd <= 4.0001f * R2) {
+                const int c = nb_cell(cx, cy, dx, dy, n, ox, oy);
+                PM_CHK(c >= 0 && c < g.ncell, 201, s0 = s1)
+                s0 = __ldg(cell_start + c);
+                s1 = __ldg(cell_start + c + 1);
+                PM_CHK(s0 >= 0 && s1 <= np && s0 <= s1, 202, s0 = s1 = 0)
+            }
+            for (unsigned cells = __ballot_sync(FULL, s0 < s1); cells && !err; cells &= cells - 1) {
+                const int src = __ffs(cells) - 1;
+                const int a = __shfl_sync(FULL, s0, src), b = __shfl_sync(FULL, s1, src);
+                const int code = (__shfl_sync(FULL, ox, src) + 1) * 3 + (__shfl_sync(FULL, oy, src) + 1);
+                if (__shfl_sync(FULL, bd, src) > 4.0001f * R2) continue;
+                for (int k = a; k < b && !err; k += 32) {
+                    const int s = k + lane;
+                    bool hit = false, dup = false;
+                    int rx = 0, ry = 0;
+                    if (s < b && s != p) {
+                        const uint2 Xs = __ldg(pos + s);
+                        rx = (int)(Xs.x - Xp.x);
+                        ry = (int)(Xs.y - Xp.y);
+                        dup = (rx | ry) == 0;
+                        hit = rx <= (1 << 30) && rx >= -(1 << 30) && ry <= (1 << 30) && ry >= -(1 << 30) && !seeds.has(s);
+                        const float fx = (float)rx, fy = (float)ry, d2 = fx * fx + fy * fy;
+                        hit = hit && d2 <= 4.0001f * R2;
+                        if (hit) {  // certainly outside every vertex's circle: no cut (as in clip_by)
+                            const float hs = 0.5f * d2, ns = 1.41422f * fmaxf(fabsf(fx), fabsf(fy)), mr = 2.4e-7f * d2;
+                            bool cut = false;
+                            for (int i = 0; i < m; ++i) {
+                                const float4 v = P.v[i][t];
+                                cut |= !(v.x * fx + v.y * fy - hs < -(v.z * ns + mr));
+                            }
+                            hit = cut;
+                        }
+                    }
+                    if (COUNT && lane == 0) wc.cand += min(32, b - k);
+                    if (__any_sync(FULL, dup)) err = ST_DUP;
+                    for (unsigned hits = __ballot_sync(FULL, hit); hits && !err; hits &= hits - 1) {
+                        const int h = __ffs(hits) - 1, hx = __shfl_sync(FULL, rx, h), hy = __shfl_sync(FULL, ry, h);
+                        if (lane == 0) {
+                            err = clip_by<LCAP, NB, COUNT>(P, m, R2, hx, hy, k + h, code, p, pp, perm, wc);
+                            if (COUNT) wc.cand--;  // counted above
+                        }
+                        err = __shfl_sync(FULL, err, 0);
+                    }
+                    __syncwarp();
+                    m = __shfl_sync(FULL, m, 0);
+                    R2 = __shfl_sync(FULL, R2, 0);
+                }
+            }
+        }
+        const float dmin = edge + (float)r * cw;
+        if (4.0001f * R2 < dmin * dmin) done = true;
+    }
+    if (err) return err;
+    if (!done) return ST_SPARSE;
+    const int4 q = P.q[lane < m ? lane : 0][t], q2 = P.q[lane + 1 < m ? lane + 1 : 0][t];
+    if (__any_sync(FULL, lane < m && (q.z & 0x0fffffff) >= PM_VIRT)) return ST_SPARSE;
+    if (m > PM_MAXDEG) return ST_DEGREE;
+    ll area2 = lane < m ? (ll)q.x * q2.y - (ll)q.y * q2.x : 0;
+    for (int o = 16; o > 0; o >>= 1) area2 += __shfl_xor_sync(FULL, area2, o);
+    const ull key = lane < m ? start_key(Inversion{Xp, cw}, q.x, q.y, q.z, n, cy) : 0;
+    ull best = key;
+    for (int o = 16; o > 0; o >>= 1) best = max(best, (ull)__shfl_xor_sync(FULL, best, o));
+    const int k0 = __ffs(__ballot_sync(FULL, key == best)) - 1;
+    if (lane < m) nbr[(ll)(lane >= k0 ? lane - k0 : lane + m - k0) * np + p] = q.z;
+    if (lane == 0) {
+        deg[p] = (unsigned char)m;
+        vol[p] = (float)area2 * vol_scale;
+        if (COUNT && m > 12) wc.over++;
+    }
+    return 0;
+}
+
+template <class Mesh, bool COUNT>
+__global__ void __launch_bounds__(LBLK) k_delaunay_last(Mesh M, const uint2 *__restrict__ pos,
+                                                        const int *__restrict__ perm, int *__restrict__ nbr,
+                                                        unsigned char *__restrict__ deg, float *__restrict__ vol,
+                                                        int *__restrict__ status, Lists L, ull *__restrict__ wsum) {
+    constexpr int NB = LBLK / 32;
+    __shared__ int4 sq[LCAP][NB];
+    __shared__ float4 sv[LCAP][NB];
+    const int hard = L.counts[2], ties = L.counts[1] < EXACT_MIN ? L.counts[1] : 0;
+    WorkCount wc;
+    const int w = threadIdx.x >> 5;
+    PolyS<NB> P{sq, sv, w};
+    for (ll j = (ll)blockIdx.x * NB + w; j < (ll)hard + ties; j += (ll)gridDim.x * NB) {
+        const int p = j < hard ? L.last[j] : L.exact[j - hard];
+        PM_CHK(p >= 0 && p < M.np, 207, continue)
+        const int k = M.instance(p);
+        const int err = star_warp<COUNT>(P, p, M.geo(k), M.np, pos, M.cells(k), perm, nbr, deg, vol, M.scale(k), wc);
+        if (err && (threadIdx.x & 31) == 0) fail_star(err, p, deg, vol, status);
+        __syncwarp();
+    }
+    add_counts<COUNT>(wc, wsum, 6);
 }
 
 // Batched passes: the particle's instance comes from the packed offsets; its
 // mesh, cell ranges and volume scale from the instance table. Stars hold
 // packed sorted indices (< 2^28 in total).
 __global__ void __launch_bounds__(HBLK, HMINB) k_delaunay_b(BTab t, const uint2 *__restrict__ pos,
-                                                     const int *__restrict__ cell_start, const int *__restrict__ perm,
-                                                     int *__restrict__ nbr,
-                                                     unsigned char *__restrict__ deg, float *__restrict__ vol,
-                                                     Lists L) {
+                                                     const int *__restrict__ cell_start, int *__restrict__ nbr,
+                                                     unsigned char *__restrict__ deg, float *__restrict__ vol, Lists L) {
     __shared__ int ids[HL + 4][HBLK];
     __shared__ float4 stk[HDEG][HBLK];
     const ll pl = (ll)blockIdx.x * HBLK + threadIdx.x;
     const bool live = pl < t.NP;
+    const int ties = L.counts[1];
+    const uint2 Xp = live ? pos[pl] : make_uint2(0u, 0u);
+    WorkCount wc;
+    int e = HULL_EXACT;
     const int k = find_slot(t.poff, t.ninst, live ? pl : t.NP - 1);
     const Geo g = batch_geo(t, k);
-    WorkCount wc;
-    const int e = star_hull<false>(ids, stk, live, (int)pl, g, t.NP, pos, cell_start + __ldg(t.coff + k), perm, nbr, deg, vol,
-                                   t.inst[k].vol_scale, wc);
+    const int *cs = cell_start + __ldg(t.coff + k);
+    if (!on_lattice(live, Xp, g, pos, cs))
+        e = star_hull<false>(ids, stk, live, (int)pl, Xp, ties, g, t.NP, pos, cs, nbr, deg, vol, t.inst[k].vol_scale, wc);
+    else if (live)
+        nbr[pl] = -1;
     push_list(live && e == HULL_WIDER, (int)pl, t.NP, L.wide, L.counts);
     push_list(live && e == HULL_EXACT, (int)pl, t.NP, L.exact, L.counts + 1);
 }
@@ -1181,40 +1517,7 @@ __global__ void __launch_bounds__(WBLK) k_delaunay_wide_b(BTab t, const uint2 *_
         const Geo g = batch_geo(t, k);
         const int e = star_wide<false>(G[gid], live, p, g, t.NP, pos, cell_start + __ldg(t.coff + k), perm, nbr, deg,
                                        vol, t.inst[k].vol_scale, wc);
-        push_list(live && e != HULL_DONE && (threadIdx.x & 7) == 0, p, t.NP, L.exact, L.counts + 1);
-    }
-}
-
-template <int CAP, int NB, bool LAST>
-__global__ void __launch_bounds__(NB) k_delaunay_retry_b(BTab t, const uint2 *__restrict__ pos,
-                                                         const int *__restrict__ cell_start,
-                                                         const int *__restrict__ perm, int *__restrict__ nbr,
-                                                         unsigned char *__restrict__ deg, float *__restrict__ vol,
-                                                         int *__restrict__ status, int *__restrict__ retry,
-                                                         const int *__restrict__ nretry) {
-    __shared__ int4 sq[CAP][NB];
-    __shared__ float4 sv[CAP][NB];
-    const int cnt = *nretry;
-    WorkCount wc;
-    PolyS<NB> P{sq, sv, (int)threadIdx.x};
-    for (ll j = (ll)blockIdx.x * NB + threadIdx.x; j < cnt; j += (ll)gridDim.x * NB) {
-        int p = retry[j];
-        if (LAST) {
-            if (p >= 0) continue;
-            p = ~p;
-        }
-        PM_CHK(p >= 0 && p < t.NP, 208, continue)
-        const int k = find_slot(t.poff, t.ninst, (ll)p);
-        const Geo g = batch_geo(t, k);
-        const int err = star_of<CAP, NB, false>(P, p, g, t.NP, pos, cell_start + __ldg(t.coff + k), perm, nbr, deg,
-                                                vol, t.inst[k].vol_scale, wc);
-        if (!LAST && err == ST_OVERFLOW) {
-            retry[j] = ~p;
-        } else if (err) {
-            atomicOr(status, (err & ~ST_OVERFLOW) | (err == ST_OVERFLOW ? ST_DEGREE : 0));
-            deg[p] = 0;
-            vol[p] = 0.0f;
-        }
+        push_list(live && e != HULL_DONE && (threadIdx.x & 7) == 0, p, t.NP, L.last, L.counts + 2);
     }
 }
 
@@ -1255,23 +1558,26 @@ __global__ void k_export(ll np, const uint2 *__restrict__ pos, const int *__rest
 
 namespace {
 // The passes' lists: the sort's scratch is free once the particles are sorted.
-Lists pass_lists(const Work &w) { return Lists{w.tmp, w.key, w.nretry}; }
+Lists pass_lists(const Work &w) { return Lists{w.tmp, w.key, w.slot, w.nretry}; }
 
-// Grids of the list passes (grid-stride): the wide pass with 8 resident blocks
-// per SM, the first exact pass with 17, the last (rare entries) with 8.
-constexpr int kWideGrid = 8 * 152, kExactGrid = 17 * 152, kLastGrid = 8 * 152;
+// Grids of the list passes (grid-stride): resident blocks per SM.
+constexpr int kWideGrid = 8 * 152, kExactGrid = EMINB * 152, kLastGrid = 12 * 152;
+
+template <class Mesh, bool COUNT>
+void exact_passes(const Mesh &M, Work &w, const Lists &L, ull *wsum, cudaStream_t st) {
+    k_delaunay_exact<Mesh, COUNT><<<min(kExactGrid, div_up(M.np, EBLK)), EBLK, 0, st>>>(M, w.pos, w.perm, w.nbr, w.deg,
+                                                                                    w.vol, w.status, L, wsum);
+    k_delaunay_last<Mesh, COUNT><<<min(kLastGrid, div_up(M.np, LBLK / 32)), LBLK, 0, st>>>(M, w.pos, w.perm, w.nbr, w.deg,
+                                                                                       w.vol, w.status, L, wsum);
+}
 
 template <bool COUNT>
 void triangulate_passes(const Geo &g, Work &w, ll np, float scale, ull *wsum, cudaStream_t st) {
     const Lists L = pass_lists(w);
-    k_delaunay<COUNT><<<div_up(np, HBLK), HBLK, 0, st>>>(g, np, w.pos, w.cell_start, w.perm, w.nbr, w.deg, w.vol, scale,
-                                                         L, wsum);
+    k_delaunay<COUNT><<<div_up(np, HBLK), HBLK, 0, st>>>(g, np, w.pos, w.cell_start, w.nbr, w.deg, w.vol, scale, L, wsum);
     k_delaunay_wide<COUNT><<<min(kWideGrid, div_up(np, WG)), WBLK, 0, st>>>(g, np, w.pos, w.cell_start, w.perm, w.nbr,
                                                                             w.deg, w.vol, scale, L, wsum);
-    k_delaunay_retry<R1CAP, R1BLK, false, COUNT><<<min(kExactGrid, div_up(np, R1BLK)), R1BLK, 0, st>>>(
-        g, np, w.pos, w.cell_start, w.perm, w.nbr, w.deg, w.vol, scale, w.status, L.exact, L.counts + 1, wsum);
-    k_delaunay_retry<RCAP, RBLK, true, COUNT><<<min(kLastGrid, div_up(np, RBLK)), RBLK, 0, st>>>(
-        g, np, w.pos, w.cell_start, w.perm, w.nbr, w.deg, w.vol, scale, w.status, L.exact, L.counts + 1, wsum);
+    exact_passes<OneMesh, COUNT>(OneMesh{g, np, w.cell_start, scale}, w, L, wsum, st);
 }
 }  // namespace
 
@@ -1279,7 +1585,7 @@ void launch_triangulate(const Geo &g, Work &w, ll np, cudaStream_t st, bool coun
     if (np <= 0) return;
     double u = g.L / 4294967296.0;
     float scale = (float)(u * u / 6.0);
-    cudaMemsetAsync(w.nretry, 0, 2 * sizeof(int), st);
+    cudaMemsetAsync(w.nretry, 0, 4 * sizeof(int), st);
     if (count_work)
         triangulate_passes<true>(g, w, np, scale, w.wsum, st);
     else
@@ -1289,15 +1595,12 @@ void launch_triangulate(const Geo &g, Work &w, ll np, cudaStream_t st, bool coun
 
 void launch_triangulate_batched(const BTab &t, Work &w, cudaStream_t st) {
     if (t.NP <= 0) return;
-    cudaMemsetAsync(w.nretry, 0, 2 * sizeof(int), st);
+    cudaMemsetAsync(w.nretry, 0, 4 * sizeof(int), st);
     const Lists L = pass_lists(w);
-    k_delaunay_b<<<div_up(t.NP, HBLK), HBLK, 0, st>>>(t, w.pos, w.cell_start, w.perm, w.nbr, w.deg, w.vol, L);
+    k_delaunay_b<<<div_up(t.NP, HBLK), HBLK, 0, st>>>(t, w.pos, w.cell_start, w.nbr, w.deg, w.vol, L);
     k_delaunay_wide_b<<<min(kWideGrid, div_up(t.NP, WG)), WBLK, 0, st>>>(t, w.pos, w.cell_start, w.perm, w.nbr, w.deg,
                                                                          w.vol, L);
-    k_delaunay_retry_b<R1CAP, R1BLK, false><<<min(kExactGrid, div_up(t.NP, R1BLK)), R1BLK, 0, st>>>(
-        t, w.pos, w.cell_start, w.perm, w.nbr, w.deg, w.vol, w.status, L.exact, L.counts + 1);
-    k_delaunay_retry_b<RCAP, RBLK, true><<<min(kLastGrid, div_up(t.NP, RBLK)), RBLK, 0, st>>>(
-        t, w.pos, w.cell_start, w.perm, w.nbr, w.deg, w.vol, w.status, L.exact, L.counts + 1);
+    exact_passes<BatchMesh, false>(BatchMesh{t, t.NP, w.cell_start}, w, L, nullptr, st);
     count_launches(4);
 }
 

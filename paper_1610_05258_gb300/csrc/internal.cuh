@@ -175,7 +175,7 @@ struct Work {
     float *corr;           // [F][ncell] network output
     double *hres;          // [PM_MAXF] pinned host: delta-start residual per field (network gating)
     ull *wsum;             // [8] triangulation work counters (counting mode)
-    int *nretry;           // [2] particles handed to the triangulation's wide and exact passes
+    int *nretry;           // [4] particles handed to the triangulation's wide, exact and last passes, the exact pass's next
     // mesh -> particle projections (particle-sized, sorted order)
     unsigned *meshmax;     // [PM_MAXF] max |Ab| bit patterns
     float *pc;             // [F][np] right-hand side c
