@@ -6,7 +6,6 @@
 #include "pmt.h"
 
 #define PM_MAXDEG 24   // Delaunay degree stored per particle
-#define PM_MAXW 32     // capacity of the working Voronoi polygon
 #define PM_MAXF 8      // fields per call
 #define PM_POS_PAD 8    // slots past the last sorted position that a load may touch (its value is not used)
 #define PM_RCAP 12     // rings of cells searched by the triangulation
@@ -212,6 +211,27 @@ __device__ __forceinline__ void two_sum(float a, float b, float &s, float &e) {
     s = __fadd_rn(a, b);
     float z = __fsub_rn(s, a);
     e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, z)), __fsub_rn(b, z));
+}
+
+// Two floats of a packed FP32 operation.
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pk2(float a, float b) {
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ void up2(f32x2 v, float &a, float &b) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+    f32x2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
 }
 
 // Accumulators. The library's arithmetic is the compensated one (PM_SUMS

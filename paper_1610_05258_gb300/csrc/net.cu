@@ -553,28 +553,11 @@ __global__ void __launch_bounds__(256, 2) k_wgrad_mid(const bf16 *__restrict__ g
 // weight walking over all pixels. Per-block partials [608 + 289].
 #define WTX 64
 #define WTY 4
-typedef unsigned long long f32x2;
-__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
-    f32x2 r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-    return r;
-}
-__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
-    f32x2 r;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
 __device__ __forceinline__ f32x2 bf2(uint32_t v) {  // two BF16 -> two FP32
     f32x2 r;
     asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "r"(v << 16), "r"(v & 0xffff0000u));
     return r;
 }
-__device__ __forceinline__ f32x2 dup2(float v) {
-    f32x2 r;
-    asm("mov.b64 %0, {%1, %1};" : "=l"(r) : "f"(v));
-    return r;
-}
-
 __global__ void __launch_bounds__(256, 2) k_wgrad_thin(const bf16 *__restrict__ gz1, const float *__restrict__ x,
                                                     const float *__restrict__ gout, const bf16 *__restrict__ a3, int B,
                                                     int n, float *__restrict__ part) {
@@ -582,6 +565,7 @@ __global__ void __launch_bounds__(256, 2) k_wgrad_thin(const bf16 *__restrict__ 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, hw = lane >> 4, cp = lane & 15;
     const int tiles_x = n / WTX, tiles_y = n / WTY, ntiles = B * tiles_x * tiles_y;
     const ll npx = (ll)n * n;
+    auto twice = [](float v) { return pk2(v, v); };
     f32x2 w0[2][9], b0 = 0, w3[9];
     KSum b3;
 #pragma unroll
@@ -594,9 +578,9 @@ __global__ void __launch_bounds__(256, 2) k_wgrad_thin(const bf16 *__restrict__ 
         for (int i = tid; i < (WTY + 2) * (WTX + 2); i += 256) {
             const int ly = i / (WTX + 2), lx = i % (WTX + 2);
             const ll o = (ll)wrapn(y0 + ly - 1, n) * n + wrapn(x0 + lx - 1, n);
-            sx[0][ly][lx] = dup2(__bfloat162float(__float2bfloat16(x[((ll)img * 2) * npx + o])));
-            sx[1][ly][lx] = dup2(__bfloat162float(__float2bfloat16(x[((ll)img * 2 + 1) * npx + o])));
-            so[ly][lx] = dup2(gout[(ll)img * npx + o]);
+            sx[0][ly][lx] = twice(__bfloat162float(__float2bfloat16(x[((ll)img * 2) * npx + o])));
+            sx[1][ly][lx] = twice(__bfloat162float(__float2bfloat16(x[((ll)img * 2 + 1) * npx + o])));
+            so[ly][lx] = twice(gout[(ll)img * npx + o]);
         }
         __syncthreads();
         const ll p0 = (ll)img * npx + (ll)(y0 + ty) * n + x0 + tx0;
