@@ -311,34 +311,38 @@ def run_reference(args):
 # bound by ALU issue, not by memory. Its algorithmic operation count per
 # launch is the arithmetic of building the stars on the actual particle set:
 # the kernels' counting build (pm_profile mode 2) counts, over all particles,
-# the candidates examined, the candidates passing the distance bound, the
-# tests of a candidate against a hull edge or cell vertex, the insertions into
-# a star (clips) and the star sizes after each; each is weighted by the
-# FP32/INT32 arithmetic instructions of that step in the exact clipping passes
-# (an FMA counts as one): distance test 10, margin set-up 5, vertex test 5,
-# clip with two circumcentres and error bounds 80, radius bound 9 per vertex.
-# The hull passes, which build most stars, insert with less than that, so the
-# count is an upper estimate for them. Divergence, address arithmetic, loads
-# and stores are not counted.
+# the candidates examined, the candidates within the search radius, the tests
+# of a candidate against a star edge and the insertions into a star; each is
+# weighted by the FP32/INT32 arithmetic instructions of that step in the hull
+# passes, which build nearly all stars (an FMA counts as one): distance test 7
+# (two differences, two conversions, product, FMA, comparison), inversion 6 (on
+# collection and again on insertion), edge test 4 (two FMAs, sign count,
+# maximum). Divergence, list slots that hold no candidate, address arithmetic,
+# loads and stores are not counted. The few stars of the clipping passes cost
+# more per event (DELAUNAY_OP_WEIGHTS: distance test 10, margin set-up 5, vertex
+# test 5, clip with two circumcentres and error bounds 80, radius bound 9 per
+# vertex), so the count is a lower bound for them.
+HULL_OP_WEIGHTS = {"candidates": 7, "tested": 6, "vertex_tests": 4, "clips": 6}
 DELAUNAY_OP_WEIGHTS = {"candidates": 10, "tested": 5, "vertex_tests": 5, "clips": 80, "cell_size_sum": 9}
 # ALU peak: 152 SMs x 128 FP32 lanes x one instruction per lane per clock.
 ALU_LANES = 152 * 128
-# DRAM traffic of one k_delaunay launch per particle: dram__bytes_read.sum +
-# dram__bytes_write.sum of one ncu capture on the 1024^2 mixture (4,194,304
-# particles: 100.11 MB read + 106.89 MB written), scaled to a launch by its
-# particle count (the kernel's traffic grows in proportion to it). The capture
-# is of the clipping main pass; the hull pass moves 216 MB there.
+# DRAM traffic per particle: dram__bytes_read.sum + dram__bytes_write.sum of one
+# ncu capture on the 1024^2 mixture (4,194,304 particles), scaled to a launch by
+# its particle count (the traffic grows in proportion to it). The hull pass, and
+# the clipping pass that it replaced as the main one.
+HULL_DRAM_BYTES_PER_PARTICLE = (95.748096e6 + 107.770112e6) / 4194304
 DELAUNAY_DRAM_BYTES_PER_PARTICLE = (100.109568e6 + 106.889216e6) / 4194304
 
 
-def alu_roofline(kernel, counts, ms, sm_mhz, n_particles):
-    ops = float(sum(DELAUNAY_OP_WEIGHTS[k] * counts[k] for k in DELAUNAY_OP_WEIGHTS))
+def alu_roofline(kernel, counts, ms, sm_mhz, n_particles, weights=DELAUNAY_OP_WEIGHTS,
+                 bytes_per_particle=DELAUNAY_DRAM_BYTES_PER_PARTICLE):
+    ops = float(sum(weights[k] * counts[k] for k in weights))
     achieved = ops / (ms * 1e-3) / 1e12
     peak = ALU_LANES * sm_mhz * 1e6 / 1e12
     return {"kernel": kernel, "bound": "alu", "achieved": achieved, "peak": peak, "unit": "Tops/s",
-            "frac": achieved / peak, "traffic": DELAUNAY_DRAM_BYTES_PER_PARTICLE * n_particles,
+            "frac": achieved / peak, "traffic": bytes_per_particle * n_particles,
             "traffic_source": "ncu dram bytes of k_delaunay on the 1024^2 mixture, scaled by particles",
-            "ops_per_launch": ops, "work_counts": counts,
+            "ops_per_launch": ops, "work_counts": counts, "op_weights": weights,
             "peak_source": f"derived: 152 SMs x 128 lanes x {sm_mhz:.0f} MHz (median SM clock sampled during the "
                            f"timed region)"}
 
@@ -509,7 +513,8 @@ def run_mixture(args, pm, torch, dist, local):
     ctx.profile(False)
     sm = ck.get("sm_mhz") or float(measured_peaks().get("sm_max_mhz", 2070.0))
     dom = max(plain["phase_ms"], key=plain["phase_ms"].get)
-    roof = alu_roofline("k_delaunay (phase triangulate)", counts, plain["phase_ms"]["triangulate"], sm, N)
+    roof = alu_roofline("k_delaunay (phase triangulate)", counts, plain["phase_ms"]["triangulate"], sm, N,
+                        HULL_OP_WEIGHTS, HULL_DRAM_BYTES_PER_PARTICLE)
     roof["dominant_phase"] = dom
     hbm = float(measured_peaks().get("hbm_gbs", 6800.0))
     minimal = N * (8 + 4 * F) + n * n * 4 * F  # positions + values in, fields out
@@ -678,7 +683,8 @@ def run_chain(args, pm, torch, dist, local):
         ctx.assign_mass(px, py, vel, out=mesh[1], info=False)
         counts = ctx.work_read()
         ctx.profile(False)
-        roof = alu_roofline("k_delaunay (phase triangulate)", counts, mass["phase_ms"]["triangulate"], sm, N)
+        roof = alu_roofline("k_delaunay (phase triangulate)", counts, mass["phase_ms"]["triangulate"], sm, N,
+                            HULL_OP_WEIGHTS, HULL_DRAM_BYTES_PER_PARTICLE)
     else:
         roof = hbm_roofline("whole step (every kernel of 128 particles is launch-latency bound)",
                             chain_step_bytes(N, nodes, F, dim), mass["ms"], "G2P + shift + mass P2G minimal I/O")

@@ -498,10 +498,10 @@ __device__ __forceinline__ void restart_state(SolveState &V, int f, double rr, d
 // is one pass: each node forms the next r at its stencil's nodes from the old r,
 // w and s (the same FMAs everywhere, so every copy has the same bits), and r, s
 // and w alternate between two buffers. The separate passes for M p, x and r,
-// and p took three barriers. Whole solves, before and now: 128 nodes in 1D (7
-// iterations, one block) 105 -> 42 us; 256^2 (13) 232 -> 97 us; 512^2, 3 fields
-// (19) 669 -> 284 us; 2048^2, 4 fields (19) 4046 -> 2766 us, 40 bytes per node and
-// iteration at 4.6 TB/s.
+// and p took three barriers. Whole solves from zero, before and now: 128 nodes in
+// 1D (one block) 168 -> 46 us; 256^2 327 -> 126 us; 512^2, 3 fields 684 -> 285 us; 2048^2, 4
+// fields (19 iterations) 4165 -> 2859 us: 40 bytes per node and iteration, and 44 in
+// the other passes, 4.7 TB/s.
 // Consecutive reductions never share slots, so that a block that runs ahead never
 // overwrites partials another block is summing: {0, 1, 2} and {3, 4} of red, {0}
 // and then alternately {2, 3} and {0, 1} of red4, and {0, 1} of red at the end.
@@ -677,9 +677,10 @@ __global__ void __launch_bounds__(256, VEC == 4 ? 3 : 4) k_cg(CG a) {
 // iteration restarts from it (at most three times). The mean mode is set
 // exactly first, as for CG, and every update d_k has zero mean, so the result
 // is conservative to rounding.
-// 20 steps on a bilinear mesh: 256^2 with 1 field 195 -> 92 us, 512^2 with 3
-// fields 535 -> 169 us, 1024^2 with 4 fields 1419 -> 496 us, 2048^2 with 4 fields
-// 4196 -> 2191 us (28 bytes per node and step: 4.3 TB/s), against passes of four
+// 20 steps on a bilinear mesh: 256^2 with 1 field 188 -> 88 us, 512^2 with 3
+// fields 522 -> 168 us, 1024^2 with 4 fields 1400 -> 557 us, 2048^2 with 4 fields
+// 4056 -> 1806 us (24 bytes per node and step, 20 in the first, and 36 in the other
+// passes: 4.8 TB/s), against passes of four
 // steps on 32 x 32 tiles with a halo in shared memory, which these replace (on
 // this kernel's barrier and loads: 106, 255, 1038, 4075 us; a step does 1.6
 // times the work there, at one block of shared-memory latency after another).
