@@ -214,13 +214,14 @@ pm_status pm_ctx_create_mesh(pm_ctx **out, int dim, int n, double L, long long m
               alloc(c, &w.psum, 2 * PM_MAXF * (ll)w.nblk_psum) &&
               alloc(c, &w.epart, 2 * PM_MAXF * (ll)energy_blocks()) && alloc(c, &w.r, F * nc) && alloc(c, &w.r2, F * nc) &&
               alloc(c, &w.p, F * nc) && alloc(c, &w.q, F * nc) && alloc(c, &w.b, F * nc) &&
-              alloc(c, &w.red, 6LL * PM_MAXF * 4096) && alloc(c, &w.red4, 4LL * PM_MAXF * 4096) && alloc(c, &w.scal, 16LL * PM_MAXF) &&
+              alloc(c, &w.red, 14LL * PM_MAXF * 4096) && alloc(c, &w.scal, 16LL * PM_MAXF) &&
               alloc(c, &w.bar, 2) && alloc(c, &w.status, 1) && alloc(c, &w.empty, 1) && alloc(c, &w.ntri, 1) &&
               alloc(c, &w.wsum, 8) && alloc(c, &w.nretry, 4) && alloc(c, &w.meshmax, PM_MAXF) &&
               alloc(c, &w.pc, F * np) && alloc(c, &w.px, pcg_width((int)F) * np) &&
               alloc(c, &w.pq, pcg_width((int)F) * np) && alloc(c, &w.prp, 2LL * pcg_width((int)F) * np) &&
               alloc(c, &w.pp2, pcg_width((int)F) * np);
     w.cfix = (ll *)w.prp;
+    w.red4 = (float4 *)(w.red + 6LL * PM_MAXF * 4096);  // behind the six slots of red
     w.red_blocks = 4096;
     if (ok && dim == 2)
         ok = alloc(c, &w.nbr, (ll)PM_MAXDEG * np) && alloc(c, &w.pcoef, (ll)PM_MAXDEG * np);

@@ -160,7 +160,7 @@ struct Work {
     double *epart;      // [2 PM_MAXF][energy_blocks()] block partials of the stability diagnostics
     // solver
     float *r, *p, *q, *b;  // [F][ncell]
-    double *red;           // reduction partials [6 PM_MAXF][grid]
+    double *red;           // reduction partials [6 PM_MAXF][grid], red4 behind them
     float4 *red4;          // reduction partials of the iterations [4 PM_MAXF][grid]
     int red_blocks;        // grid capacity of both (blocks per slot); persistent solves never exceed it
     double *scal;          // solver scalars per field
