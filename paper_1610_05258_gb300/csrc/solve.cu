@@ -99,12 +99,14 @@ __device__ bool grid_sync(unsigned *bar, int *status, unsigned &passed) {
 //    red[(slot + kind) * F + f][block]. The start, the closing residual.
 //  put_scaled, flush_scaled, grid_scaled: the inner products of an iteration,
 //    brought to order one by powers of two, so that no exponents are carried;
-//    Sum3 in red4[(slot + kind) * F + f][block].
+//    Sum3 in red4[(slot + kind) * F + f][block]. A single block keeps its totals
+//    in shared memory.
 // An FP64 addition takes 62 cycles here, a sum over a warp 680 in FP64 and 228 in
 // Sum3 (180 in FP32 pairs, which this replaces: whole solves by CG take the
 // same time to 5 %, 256^2 122.5 -> 125.7 us, 255^2 166 -> 147 us).
 struct BlockSums {
     Sum3 v[3][PM_MAXF][8];
+    Sum3 one[2 * PM_MAXF];  // totals of a single block's inner products
 };
 __device__ __forceinline__ void put_sum(BlockSums &B, int kind, int f, const Dot2 &a) {
     const Sum3 t = fold_warp(warp_parts(a));
@@ -149,7 +151,7 @@ __device__ __forceinline__ void put_scaled(BlockSums &B, int f, const Dot2 &a0, 
     const Sum3 t = fold_warp(scaled_parts(a0, s0, 0), scaled_parts(a1, s1, 0));
     if ((threadIdx.x & 15) == 0) B.v[threadIdx.x >> 4 & 1][f][threadIdx.x >> 5] = t;
 }
-__device__ __forceinline__ void flush_scaled(const BlockSums &B, int kinds, int F, float4 *red4, int slot) {
+__device__ __forceinline__ void flush_scaled(BlockSums &B, int kinds, int F, float4 *red4, int slot) {
     __syncthreads();
     const int t = threadIdx.x;
     if (t < kinds * F) {
@@ -161,27 +163,36 @@ __device__ __forceinline__ void flush_scaled(const BlockSums &B, int kinds, int 
             add_parts(b, v[w + 4].a, v[w + 4].b, v[w + 4].c);
         }
         add_parts(a, b.a, b.b, b.c);
+        if (gridDim.x == 1) {
+            B.one[t] = a;
+            return;
+        }
         red4[(ll)(slot * F + t) * gridDim.x + blockIdx.x] = make_float4(a.a, a.b, a.c, 0.0f);
     }
 }
 // Totals of field f in K consecutive slots (1 or 2) over all blocks, by one
 // warp, half of it for each of two slots; lane 0 has them.
 template <int K>
-__device__ __forceinline__ void grid_scaled(const float4 *red4, int F, int slot, int f, double (&out)[K]) {
+__device__ __forceinline__ void grid_scaled(const BlockSums &B, const float4 *red4, int F, int slot, int f,
+                                            double (&out)[K]) {
     constexpr int W = 32 / K;
     const unsigned lane = threadIdx.x & 31;
-    const float4 *src = red4 + (ll)((slot + (int)(lane / W)) * F + f) * gridDim.x;
     Sum3 s{0.0f, 0.0f, 0.0f, 0};
-    // eight loads in flight, also at the end: a load is an L2 latency
-    for (unsigned i = lane % W; i < gridDim.x; i += 8 * W) {
-        float4 t[8];
+    if (gridDim.x == 1) {
+        s = B.one[(int)(lane / W) * F + f];
+    } else {
+        const float4 *src = red4 + (ll)((slot + (int)(lane / W)) * F + f) * gridDim.x;
+        // eight loads in flight, also at the end: a load is an L2 latency
+        for (unsigned i = lane % W; i < gridDim.x; i += 8 * W) {
+            float4 t[8];
 #pragma unroll
-        for (int j = 0; j < 8; ++j) t[j] = i + j * W < gridDim.x ? __ldcg(src + i + j * W) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            for (int j = 0; j < 8; ++j) t[j] = i + j * W < gridDim.x ? __ldcg(src + i + j * W) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
 #pragma unroll
-        for (int j = 0; j < 8; ++j) add_parts(s, t[j].x, t[j].y, t[j].z);
+            for (int j = 0; j < 8; ++j) add_parts(s, t[j].x, t[j].y, t[j].z);
+        }
+#pragma unroll
+        for (int o = W / 2; o > 0; o >>= 1) fold_down(s, o);
     }
-#pragma unroll
-    for (int o = W / 2; o > 0; o >>= 1) fold_down(s, o);
     out[0] = ((double)s.a + (double)s.b) + (double)s.c;
     if (K == 2) out[K - 1] = __shfl_down_sync(0xffffffffu, out[0], W);
 }
@@ -560,7 +571,7 @@ __global__ void __launch_bounds__(256, VEC == 4 ? 3 : 4) k_cg(CG a) {
             if (!grid_sync(a.bar, a.status, passed)) return;
             if (wf < F && V.act[wf]) {
                 double t[1];
-                grid_scaled<1>(a.red4, F, 0, wf, t);
+                grid_scaled<1>(B, a.red4, F, 0, wf, t);
                 if (lane0) {
                     const double wr = t[0];
                     V.pMp[wf] = wr;
@@ -618,7 +629,7 @@ __global__ void __launch_bounds__(256, VEC == 4 ? 3 : 4) k_cg(CG a) {
                 if (!grid_sync(a.bar, a.status, passed)) return;
                 if (wf < F && V.act[wf]) {
                     double t[2];
-                    grid_scaled<2>(a.red4, F, slot, wf, t);
+                    grid_scaled<2>(B, a.red4, F, slot, wf, t);
                     if (lane0) {
                         const double rr = t[0], wr = t[1];
                         const double beta = rr / V.rr[wf], pMp = wr - beta * (beta * V.pMp[wf]);
@@ -1203,7 +1214,7 @@ __global__ void __launch_bounds__(256, FF == 8 ? 2 : 4) k_pcg(PCG a) {
         if (!grid_sync(a.bar, a.status, passed)) return;
         if (wf < F) {
             double t[1];
-            grid_scaled<1>(a.red4, F, 0, wf, t);
+            grid_scaled<1>(B, a.red4, F, 0, wf, t);
             if (lane0) {
                 S.al[wf] = S.act[wf] ? (float)(S.rz[wf] / t[0]) : 0.0f;
                 S.ap[wf] = S.al[wf] * S.iS[wf];
@@ -1236,7 +1247,7 @@ __global__ void __launch_bounds__(256, FF == 8 ? 2 : 4) k_pcg(PCG a) {
         if (!grid_sync(a.bar, a.status, passed)) return;
         if (wf < F) {
             double t[2];
-            grid_scaled<2>(a.red4, F, 1, wf, t);
+            grid_scaled<2>(B, a.red4, F, 1, wf, t);
             if (lane0) {
                 S.be[wf] = 0.0f;
                 if (S.act[wf]) {
